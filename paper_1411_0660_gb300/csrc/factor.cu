@@ -910,72 +910,119 @@ __global__ void __launch_bounds__(256) k_fwd_narrow(const SolveDesc *sdescs, con
     }
 }
 
-// Backward narrow step: lane c accumulates x_panel[c] = sum_r G[r][c] v[r] over 32-row chunks;
-// lane j of a chunk reads row j of v (yfw, Zs or the ancestors' x, as in k_bwd_step) and the
-// values broadcast by shuffles.  Every panel is handled by one warp, so there are no partial sums.
-template <class T, int PB>
+// Backward narrow step (every panel of the level at most CW columns wide): x_panel[c] = sum_r G[r][c] v[r]
+// with v read as in k_bwd_step (yfw, Zs or the ancestors' x).  NW warps share a panel, warp i taking the
+// 32-row chunks i, i + NW, ...; in a chunk, lane (rg, c) of the warp takes column c and the CW rows
+// [CW rg, CW rg + CW), its entries of G in 16-byte loads, and the chunk's rows of v are staged in shared
+// memory and read as broadcasts.  The lane groups' sums meet by shuffles, the warps' in shared memory, both
+// in a fixed order.
+// Bound by latency: a chunk is one dependent chain (row list -> x -> products), so the chain is as long as
+// a warp has chunks.  One warp a panel and 32 lanes of one column each, with the v entries broadcast by 8
+// shuffles a row, took 32 us a launch at L = 16 (FP32, 8 right-hand sides; a refined solve of one
+// right-hand side 1.24 ms, now 1.09).
+template <class T, int PB, int NW, int CW>
 __global__ void __launch_bounds__(256) k_bwd_narrow(const SolveDesc *sdescs, int nd, const int64_t *zo,
                                                     const int32_t *nc, const int32_t *sn_start,
                                                     const int64_t *rows_off, const int32_t *rows,
                                                     const SolveBufs<T> *jb, int p, LaunchTrace *tr) {
+    static_assert((CW == 16 || CW == 32) && 8 % NW == 0, "lane groups of a warp, warps of a CTA");
+    constexpr int E = 16 / sizeof(T), RG = 32 / CW, QC = 8;  // QC right-hand sides at a time through vs
+    constexpr int VLD = 32 * QC + RG * E;                    // a warp's chunk of v; lane groups E apart: no bank conflict
+    using V = typename Vec16<T>::type;
     TraceScope trace_scope(tr);
+    __shared__ __align__(16) T vs_all[8 * VLD];
     const T *Gp = jb[blockIdx.z].G, *yfw = jb[blockIdx.z].yfw;
     T *Zs = jb[blockIdx.z].Zs, *x = jb[blockIdx.z].y;
-    const int lane = threadIdx.x & 31, di = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (di >= nd) {
-        pdl_wait();
-        return;
-    }
-    const SolveDesc d = sdescs[di];
-    const int s = d.front, k0 = d.k0, w = d.w, R = w + d.m2, ncs = nc[s];
-    const int64_t zb = zo[s] + k0, ld = sg_ld(R), g0 = (int64_t)sn_start[s] + k0;
-    const T *G = Gp + d.goff + (int64_t)lane * ld;  // this lane's column
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, wi = wp % NW;
+    const int di = blockIdx.x * (8 / NW) + wp / NW;
+    const bool live = di < nd;  // the panel's warps are live together; all of them reach the barriers
+    const SolveDesc d = sdescs[live ? di : nd - 1];
+    const int s = d.front, k0 = d.k0, w = d.w, R = live ? w + d.m2 : 0, ncs = nc[s];
+    const int64_t zb = zo[s] + k0, ld = sg_ld(w + d.m2), g0 = (int64_t)sn_start[s] + k0;
+    const int c = lane % CW, rg = lane / CW;
+    const T *G = Gp + d.goff + (int64_t)c * ld;  // this lane's column
     const int32_t *rw = rows + rows_off[s] + k0;
-    T gl[32];
+    T *vs = vs_all + wp * VLD;
+    T gl[CW];
+    int rowx = 0;
+    auto load_chunk = [&](int rb) {  // entries of G (zero past the column's padded end) and the row of x
 #pragma unroll
-    for (int j = 0; j < 32; ++j) gl[j] = (lane < w && j < R) ? G[j] : T(0);
-    const int rowx = lane < R && k0 + lane >= ncs ? rw[lane] : 0;
-    pdl_wait();
-    pdl_trigger();
+        for (int j = 0; j < CW; j += E) {
+            V g{};
+            if (c < w && rb + rg * CW + j < R) g = *reinterpret_cast<const V *>(G + rb + rg * CW + j);
+#pragma unroll
+            for (int e = 0; e < E; ++e) gl[j + e] = Vec16<T>::get(g, e);
+        }
+        rowx = rb + lane < R && k0 + rb + lane >= ncs ? rw[rb + lane] : 0;
+    };
     T acc[PB];
 #pragma unroll
     for (int q = 0; q < PB; ++q) acc[q] = T(0);
-    for (int rb = 0; rb < R; rb += 32) {
+    int rb = 32 * wi;
+    if (rb < R) load_chunk(rb);
+    pdl_wait();
+    pdl_trigger();
+    for (; rb < R; rb += 32 * NW) {
         const int rr = rb + lane;
-        T vr[PB];
-        {
-            const T *sp = nullptr;
-            T sg = T(0);
-            if (rr < R) {
-                if (rr < w) {
-                    sp = yfw + (g0 + rr) * p;
-                    sg = T(1);
-                } else if (k0 + rr < ncs) {
-                    sp = Zs + (zb + rr) * p;
-                    sg = T(-1);
-                } else {
-                    sp = x + (int64_t)(rb == 0 ? rowx : rw[rr]) * p;
-                    sg = T(-1);
+        const T *sp = yfw;
+        T sg = T(0);
+        if (rr < R) {
+            sg = rr < w ? T(1) : T(-1);
+            sp = rr < w ? yfw + (g0 + rr) * p : (k0 + rr < ncs ? Zs + (zb + rr) * p : x + (int64_t)rowx * p);
+        }
+#pragma unroll
+        for (int q0 = 0; q0 < PB; q0 += QC) {
+            T *vr = vs + lane * QC + (lane / CW) * E;
+            if (p == PB) {  // 16-byte aligned rows
+#pragma unroll
+                for (int u = 0; u < QC; u += E) {
+                    const V v = *reinterpret_cast<const V *>(sp + q0 + u);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) vr[u + e] = rr < R ? sg * Vec16<T>::get(v, e) : T(0);
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < QC; ++u) vr[u] = rr < R && q0 + u < p ? sg * sp[q0 + u] : T(0);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < CW; ++j) {
+                const V *vv = reinterpret_cast<const V *>(vs + (rg * CW + j) * QC + rg * E);
+#pragma unroll
+                for (int u = 0; u < QC / E; ++u) {
+                    const V v = vv[u];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) acc[q0 + u * E + e] += gl[j] * Vec16<T>::get(v, e);
                 }
             }
-#pragma unroll
-            for (int q = 0; q < PB; ++q) vr[q] = (sp && q < p) ? sg * sp[q] : T(0);
+            __syncwarp();
         }
-        if (rb > 0) {  // this chunk's column entries, all loads in flight before the products
-#pragma unroll
-            for (int j = 0; j < 32; ++j) gl[j] = (lane < w && rb + j < R) ? G[rb + j] : T(0);
-        }
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-#pragma unroll
-            for (int q = 0; q < PB; ++q) acc[q] += gl[j] * __shfl_sync(0xffffffffu, vr[q], j);
+        if (rb + 32 * NW < R) load_chunk(rb + 32 * NW);
     }
-    if (lane < w) {
 #pragma unroll
-        for (int q = 0; q < PB; ++q) {
-            if (q >= p) break;
-            Zs[(zb + lane) * p + q] = acc[q];
-            x[(g0 + lane) * p + q] = acc[q];
+    for (int q = 0; q < PB; ++q)
+#pragma unroll
+        for (int o = CW; o < 32; o *= 2) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    // the panel's NW warps, QC right-hand sides at a time: red[warp][q][c]
+    T *red = vs_all + (wp - wi) * VLD;
+    static_assert(VLD >= QC * CW, "a warp's partial sums fit its chunk of v");
+#pragma unroll
+    for (int q0 = 0; q0 < PB; q0 += QC) {
+        __syncthreads();
+        if (rg == 0) {
+#pragma unroll
+            for (int u = 0; u < QC; ++u) vs[u * CW + c] = acc[q0 + u];
+        }
+        __syncthreads();
+        for (int o = wi * 32 + lane; o < QC * CW; o += 32 * NW) {
+            const int u = o / CW, cc = o % CW, q = q0 + u;
+            T v = T(0);
+#pragma unroll
+            for (int i = 0; i < NW; ++i) v += red[i * VLD + o];
+            if (live && cc < w && q < p) {
+                Zs[(zb + cc) * p + q] = v;
+                x[(g0 + cc) * p + q] = v;
+            }
         }
     }
 }
@@ -1484,10 +1531,17 @@ static void solve_levels(const Plan &pl, const SolveBufs<T> *jb, unsigned K, int
     }
     for (int l = pl.nlevels - 1; l >= 0; --l) {
         const SolveDesc *sdl = pl.d_sdescs.data() + pl.lvl_d0[l];
-        if (pl.lvl_maxw[l] <= 32 && pl.lvl_maxr[l] <= 512) {  // single narrow, short panels: a warp each
-            launch_pdl(k_bwd_narrow<T, PB>, dim3((unsigned)((pl.lvl_nd[l] + 7) / 8), 1, K), dim3(256), 0, st, sdl,
-                       pl.lvl_nd[l], pl.d_sn_zo.data(), pl.d_sn_nc.data(), pl.d_sn_start.data(),
-                       pl.d_sn_rows_off.data(), pl.d_rows.data(), jb, p, next_tr(2));
+        if (pl.lvl_maxw[l] <= 32 && pl.lvl_maxr[l] <= 1024) {
+            // single narrow, short panels: two warps a panel where the longest has at most five 32-row chunks
+            // (the leaves: thousands of panels of some twenty rows), else eight (hundreds of rows)
+            auto narrow = [&](auto kern, int nw) {
+                launch_pdl(kern, dim3((unsigned)((pl.lvl_nd[l] * nw + 7) / 8), 1, K), dim3(256), 0, st, sdl,
+                           pl.lvl_nd[l], pl.d_sn_zo.data(), pl.d_sn_nc.data(), pl.d_sn_start.data(),
+                           pl.d_sn_rows_off.data(), pl.d_rows.data(), jb, p, next_tr(2));
+            };
+            const bool two = pl.lvl_maxr[l] <= 160;
+            if (pl.lvl_maxw[l] <= 16) two ? narrow(k_bwd_narrow<T, PB, 2, 16>, 2) : narrow(k_bwd_narrow<T, PB, 8, 16>, 8);
+            else two ? narrow(k_bwd_narrow<T, PB, 2, 32>, 2) : narrow(k_bwd_narrow<T, PB, 8, 32>, 8);
         } else {
             launch_pdl(k_bwd_step<T, PB>, dim3((unsigned)pl.lvl_nrbk[l], (pl.lvl_maxw[l] + RBB - 1) / RBB, K),
                        dim3(256), bsm, st, sdl, (const int32_t *)pl.d_lvl_bblk_desc.data() + pl.lvl_bblk0[l],
