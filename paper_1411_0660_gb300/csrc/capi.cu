@@ -365,6 +365,8 @@ void mbl_ctx_destroy(mbl_ctx *ctx) {
     ctx->ent.clear();
     cudaStreamSynchronize(ctx->stream);
     cudaStreamDestroy(ctx->stream);
+    if (ctx->side_ev) cudaEventDestroy(ctx->side_ev);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
     {
         std::lock_guard<std::mutex> lk(g_ctx_mu);
         live_ctx().erase(ctx);

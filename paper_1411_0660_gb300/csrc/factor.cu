@@ -608,74 +608,67 @@ __device__ __forceinline__ int find_sdesc_b(const SolveDesc *d, int nd, int64_t 
     return lo;
 }
 
-// M of one solve panel, 32 columns per CTA, in FP64: the forward sequence (pivot permutation,
-// unit-lower substitution, elimination of the later rows of the panel) applied to unit vectors.
+// M of one solve panel, 8 columns per CTA, in FP64: the forward sequence (pivot permutation,
+// unit-lower substitution, elimination of the later rows of the panel) applied to unit vectors.  A warp
+// takes one column and keeps it in registers (lane l holds rows l, l + 32, ...): step t broadcasts entry t
+// and every lane subtracts its rows' share, so a column is one chain of w shuffles and FMAs without a
+// barrier.  M is block lower triangular in the NB-wide sub-panels: a unit vector is zero above its own.
+// Bound by the FP64 rate (two FMAs a clock and SM); 8 columns a CTA spread the 256 columns of a panel over
+// 32 SMs, so that a step of one or two panels is not held on a few.
 template <class T>
 __global__ void __launch_bounds__(256) k_build_m(const SolveDesc *sdescs, const int64_t *fo, const int32_t *fsz,
-                                                 const int32_t *sn_start, const T *arena, const int32_t *piv,
-                                                 T *Mall) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    double(*Zc)[33] = reinterpret_cast<double(*)[33]>(smraw);                          // SPW x 33
-    double(*Zp)[33] = reinterpret_cast<double(*)[33]>(smraw + 8 * SPW * 33);           // NB x 33
-    double(*Lb)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(smraw + 8 * (SPW + NB) * 33);
+                                                 const int32_t *sn_start, const T *__restrict__ arena,
+                                                 const int32_t *piv, T *Mall) {
+    static_assert(NB == 64 && SPW == 256, "two rows per lane and sub-panel");
+    __shared__ double perm[8][NB];
     const SolveDesc d = sdescs[blockIdx.x];
-    const int c0 = blockIdx.y * 32;
-    if (c0 >= d.w) return;
-    const int ncol = min(32, d.w - c0), w = d.w, s = d.front, f = fsz[s], k0 = d.k0;
-    const T *F = arena + fo[s];
-    const int64_t g0 = (int64_t)sn_start[s] + k0;
-    for (int idx = threadIdx.x; idx < w * 32; idx += blockDim.x) {
-        int r = idx / 32, c = idx % 32;
-        Zc[r][c] = (c < ncol && r == c0 + c) ? 1.0 : 0.0;
-    }
-    __syncthreads();
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, w = d.w, c = blockIdx.y * 8 + wp;
+    if (c >= w) return;
+    const int f = fsz[d.front], k0 = d.k0;
+    const T *F = arena + fo[d.front] + (int64_t)k0 * f + k0;  // the panel's diagonal block
+    const int32_t *pv = piv + (int64_t)sn_start[d.front] + k0;
+    double z[SPW / 32];
+#pragma unroll
+    for (int i = 0; i < SPW / 32; ++i) z[i] = lane + 32 * i == c ? 1.0 : 0.0;
+#pragma unroll
     for (int u = 0; u < SUBS; ++u) {
         const int s0 = u * NB;
-        if (s0 >= w) break;
-        const int ws = min(NB, w - s0);
-        for (int idx = threadIdx.x; idx < ws * ws; idx += blockDim.x) {
-            int r = idx % ws, c = idx / ws;
-            Lb[r][c] = (r > c) ? (double)F[(int64_t)(k0 + s0 + c) * f + k0 + s0 + r] : 0.0;
-        }
-        for (int idx = threadIdx.x; idx < ws * 32; idx += blockDim.x) {
-            int t = idx / 32, c = idx % 32;
-            Zp[t][c] = Zc[piv[g0 + s0 + t] - k0][c];
-        }
-        __syncthreads();
-        // forward substitution with the unit-lower L11, one thread per column
-        if (threadIdx.x < 32) {
-            const int c = threadIdx.x;
-            for (int t = 1; t < ws; ++t) {
-                double acc = Zp[t][c];
-                for (int k = 0; k < t; ++k) acc -= Lb[t][k] * Zp[k][c];
-                Zp[t][c] = acc;
+        if (s0 + NB <= c || s0 >= w) continue;
+        perm[wp][lane] = z[2 * u];
+        perm[wp][lane + 32] = z[2 * u + 1];
+        __syncwarp();
+        z[2 * u] = s0 + lane < w ? perm[wp][pv[s0 + lane] - k0 - s0] : 0.0;
+        z[2 * u + 1] = s0 + 32 + lane < w ? perm[wp][pv[s0 + 32 + lane] - k0 - s0] : 0.0;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int tn = min(32, w - s0 - 32 * h);
+#pragma unroll 4
+            for (int tt = 0; tt < tn; ++tt) {
+                const int t = s0 + 32 * h + tt;
+                const T *Fc = F + (int64_t)t * f;
+                const double zt = __shfl_sync(0xffffffffu, z[2 * u + h], tt);
+#pragma unroll
+                for (int i = 2 * u + h; i < SPW / 32; ++i) {
+                    const int r = lane + 32 * i;
+                    const double l = r > t && r < w ? (double)Fc[r] : 0.0;
+                    z[i] = fma(-l, zt, z[i]);
+                }
             }
         }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < ws * 32; idx += blockDim.x) {
-            int t = idx / 32, c = idx % 32;
-            Zc[s0 + t][c] = Zp[t][c];
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < (w - s0 - ws) * 32; idx += blockDim.x) {
-            int r = s0 + ws + idx / 32, c = idx % 32;
-            double acc = 0.0;
-            for (int t = 0; t < ws; ++t) acc += (double)F[(int64_t)(k0 + s0 + t) * f + k0 + r] * Zc[s0 + t][c];
-            Zc[r][c] -= acc;
-        }
-        __syncthreads();
     }
-    T *M = Mall + d.moff;
-    for (int idx = threadIdx.x; idx < ncol * w; idx += blockDim.x) {
-        int c = idx / w, r = idx % w;
-        M[(int64_t)(c0 + c) * w + r] = (T)Zc[r][c];
-    }
+    T *M = Mall + d.moff + (int64_t)c * w;
+#pragma unroll
+    for (int i = 0; i < SPW / 32; ++i)
+        if (lane + 32 * i < w) M[lane + 32 * i] = (T)z[i];
 }
 
 // G = [M; L21 M] of a solve panel (rows [k0, f) of the front x the panel's w columns) into the
 // packed solve factor (column-major, leading dimension sg_ld(f - k0)).  CTA (x: the step's RBB-row
 // tiles, y: 256-column halves of the panel) computes a 64 x 256 block of L21 M in 32-deep chunks
-// of the contraction (16 x 16 threads, 4 x 16 outputs each); rows of the panel itself take M.
+// of the contraction (16 x 16 threads, 4 x 16 outputs each); rows of the panel itself take M.  M is
+// block lower triangular in the NB-wide sub-panels, so a chunk above a column's sub-panel is skipped:
+// three eighths of the products of a full panel.
 template <class T>
 __global__ void __launch_bounds__(256) k_apply_m(const SolveDesc *sdescs, int nd, const int64_t *fo,
                                                  const int32_t *fsz, const T *arena, const T *Mall, T *Gp) {
@@ -714,17 +707,23 @@ __global__ void __launch_bounds__(256) k_apply_m(const SolveDesc *sdescs, int nd
                 Ms[k * MSL + c] = (k < kc && cb + c < w) ? M[(int64_t)(cb + c) * w + kc0 + k] : T(0);
             }
             __syncthreads();
+            // columns of sub-panels 0 .. ju (NB / 16 of a thread's columns each) have entries in this chunk
+            const int ju = (kc0 - cb) / NB;
 #pragma unroll 4
             for (int k = 0; k < KC; ++k) {
-                T a[4], bv[16];
+                T a[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) a[i] = As[(tr + 16 * i) * (KC + 1) + k];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) bv[j] = Ms[k * MSL + tc + 16 * j];
+                for (int jb = 0; jb < 16; jb += NB / 16) {
+                    if (jb / (NB / 16) > ju) break;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                    for (int j = jb; j < jb + NB / 16; ++j) {
+                        const T bv = Ms[k * MSL + tc + 16 * j];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[i][j] += a[i] * bv[j];
+                        for (int i = 0; i < 4; ++i) acc[i][j] += a[i] * bv;
+                    }
+                }
             }
         }
     }
@@ -919,7 +918,7 @@ __global__ void __launch_bounds__(256) k_fwd_narrow(const SolveDesc *sdescs, con
 // Bound by latency: a chunk is one dependent chain (row list -> x -> products), so the chain is as long as
 // a warp has chunks.  One warp a panel and 32 lanes of one column each, with the v entries broadcast by 8
 // shuffles a row, took 32 us a launch at L = 16 (FP32, 8 right-hand sides; a refined solve of one
-// right-hand side 1.24 ms, now 1.09).
+// right-hand side 1.24 ms, now 1.09); this form takes 4 to 8 us.
 template <class T, int PB, int NW, int CW>
 __global__ void __launch_bounds__(256) k_bwd_narrow(const SolveDesc *sdescs, int nd, const int64_t *zo,
                                                     const int32_t *nc, const int32_t *sn_start,
@@ -1228,8 +1227,6 @@ __global__ void __launch_bounds__(256) k_bwd_step(const SolveDesc *sdescs, const
 // Host drivers
 // ------------------------------------------------------------------------------------------
 template <class T>
-static size_t build_m_smem() { return 8 * ((size_t)(SPW + NB) * 33 + (size_t)NB * (NB + 1)); }
-template <class T>
 static size_t trsm_smem() { return sizeof(T) * (size_t)2 * NB * (NB + 1); }
 template <class T>
 static size_t apply_m_smem() { return sizeof(T) * ((size_t)RBB * 33 + (size_t)32 * 257); }
@@ -1268,12 +1265,34 @@ static int64_t resident_grid(K *kern, size_t smem) {
 
 template <class T>
 static void set_solve_attrs() {
-    smem_limit((const void *)k_build_m<T>, build_m_smem<T>());
     smem_limit((const void *)k_apply_m<T>, apply_m_smem<T>());
     set_step_attrs<T, 8>();
     set_step_attrs<T, 16>();
     set_step_attrs<T, 32>();
 }
+
+// Work of `main` that may run beside it: the context's side stream, joined to `main` when the scope ends
+// (also by an exception, so that memory freed on `main` afterwards is not in use on the side).
+struct SideStream {
+    Ctx *ctx;
+    cudaStream_t main;
+    bool on;
+    SideStream(Ctx *c, cudaStream_t m, bool use) : ctx(c), main(m), on(use) {
+        if (!on) return;
+        if (!ctx->side) MBL_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
+        if (!ctx->side_ev) MBL_CUDA(cudaEventCreateWithFlags(&ctx->side_ev, cudaEventDisableTiming));
+    }
+    cudaStream_t stream() const { return ctx->side; }
+    void after_main() {  // the side's later work follows main's work so far
+        MBL_CUDA(cudaEventRecord(ctx->side_ev, main));
+        MBL_CUDA(cudaStreamWaitEvent(ctx->side, ctx->side_ev, 0));
+    }
+    ~SideStream() {
+        if (on && (cudaEventRecord(ctx->side_ev, ctx->side) != cudaSuccess ||
+                   cudaStreamWaitEvent(main, ctx->side_ev, 0) != cudaSuccess))
+            cudaStreamSynchronize(ctx->side);
+    }
+};
 
 template <class T>
 static void factor_impl(Factorization &fz, cudaStream_t st) {
@@ -1285,26 +1304,30 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
     T *wscr = static_cast<T *>(fz.wscr.m.p);
     T *Gp = static_cast<T *>(fz.gpk.m.p);
     MBL_CUDA(cudaMemsetAsync(Gp, 0, (size_t)p.sg_elems * sizeof(T), st));  // padding rows of G stay zero
-    // G = [M; L21 M] of the solve panels of level l (the panels' M blocks first)
-    auto build_g_level = [&](int l) {
-        if (p.lvl_nd[l] <= 0) return;
-        ProfScope ps_g(fz.ctx, "f_build_g", 0.0, st);
-        k_build_m<T><<<dim3((unsigned)p.lvl_nd[l], SPW / 32), 256, build_m_smem<T>(), st>>>(
-            p.d_sdescs.data() + p.lvl_d0[l], p.d_sn_fo.data(), p.d_sn_f.data(), p.d_sn_start.data(), arena,
-            fz.piv.data(), static_cast<T *>(fz.M.m.p));
+    // G = [M; L21 M] of the panels of solve step si into the packed solve factor (their M blocks first)
+    auto build_g_step = [&](int si, cudaStream_t sg) {
+        const SolveStep &ss = p.ssteps[si];
+        if (ss.nd <= 0) return;
+        ProfScope ps_g(fz.ctx, "f_build_g", 0.0, sg);
+        k_build_m<T><<<dim3((unsigned)ss.nd, (ss.maxw + 7) / 8), 256, 0, sg>>>(
+            p.d_sdescs.data() + ss.d0, p.d_sn_fo.data(), p.d_sn_f.data(), p.d_sn_start.data(), arena, fz.piv.data(),
+            static_cast<T *>(fz.M.m.p));
         MBL_LAUNCH_CHECK();
-        for (int si = p.lvl_sstep_ptr[l]; si < p.lvl_sstep_ptr[l + 1]; ++si) {
-            const SolveStep &ss = p.ssteps[si];
-            k_apply_m<T><<<dim3((unsigned)ss.nrbb, (SPW + 255) / 256), 256, apply_m_smem<T>(), st>>>(
-                p.d_sdescs.data() + ss.d0, ss.nd, p.d_sn_fo.data(), p.d_sn_f.data(), arena,
-                static_cast<const T *>(fz.M.m.p), Gp);
-            MBL_LAUNCH_CHECK();
-        }
+        k_apply_m<T><<<dim3((unsigned)ss.nrbb, (SPW + 255) / 256), 256, apply_m_smem<T>(), sg>>>(
+            p.d_sdescs.data() + ss.d0, ss.nd, p.d_sn_fo.data(), p.d_sn_f.data(), arena,
+            static_cast<const T *>(fz.M.m.p), Gp);
+        MBL_LAUNCH_CHECK();
     };
     smem_limit((const void *)k_panel_trsm<T>, trsm_smem<T>());
     set_solve_attrs<T>();
     MBL_CUDA(cudaMemsetAsync(fz.counters.data(), 0, 5 * sizeof(unsigned long long), st));
     MBL_CUDA(cudaMemsetAsync(fz.counters.data() + 4, 0x7f, sizeof(unsigned int), st));  // min |d| starts huge
+    // A solve panel's columns are final with its last factor panel, so its G is built beside the following
+    // panel steps, on the context's side stream (the memory-lean arena releases the columns level by level
+    // and keeps the order): the panel steps are a chain of short launches that leave most SMs idle.  With all
+    // of G built after the last level, a factorization and a refined solve took 6.9 ms at L = 14, 163 ms at
+    // L = 19 (FP32) and 542 ms at L = 18 with FP64 fronts; beside the steps 5.8, 149 and 480.
+    SideStream side(fz.ctx, st, !lean);
     for (int l = 0; l < p.nlevels; ++l) {
         int na = p.asm_ptr[l + 1] - p.asm_ptr[l];
         if (lean)
@@ -1374,30 +1397,18 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                     MBL_LAUNCH_CHECK();
                 }
             }
+            if (!lean && (stp.kk % SUBS == SUBS - 1 || si + 1 == p.lvl_step_ptr[l + 1])) {
+                side.after_main();
+                build_g_step(p.lvl_sstep_ptr[l] + stp.kk / SUBS, side.stream());
+            }
         }
         if (lean) {  // the level's factor columns move to G; then they, and its root fronts, can go
-            build_g_level(l);
+            for (int q = p.lvl_sstep_ptr[l]; q < p.lvl_sstep_ptr[l + 1]; ++q) build_g_step(q, st);
             MBL_CUDA(cudaStreamSynchronize(st));
             for (int64_t i = p.lean_prefix_ptr[l]; i < p.lean_prefix_ptr[l + 1]; ++i)
                 lean->unmap_chunk(p, (size_t)p.lean_prefix[i].first, (size_t)p.lean_prefix[i].second);
             for (size_t r = 0; r < p.regions.size(); ++r)
                 if (p.regions[r].level == l && p.regions[r].release == l) lean->unmap_region(p, r);
-        }
-    }
-    if (lean) return;
-    // block operators of the solve panels, then G = [M; L21 M] of each panel into the packed solve factor
-    if (!p.sdescs.empty()) {
-        ProfScope ps_g(fz.ctx, "f_build_g", 0.0, st);
-        dim3 grid((unsigned)p.sdescs.size(), SPW / 32);
-        k_build_m<T><<<grid, 256, build_m_smem<T>(), st>>>(p.d_sdescs.data(), p.d_sn_fo.data(), p.d_sn_f.data(),
-                                                           p.d_sn_start.data(), arena, fz.piv.data(),
-                                                           static_cast<T *>(fz.M.m.p));
-        MBL_LAUNCH_CHECK();
-        for (const SolveStep &ss : p.ssteps) {
-            k_apply_m<T><<<dim3((unsigned)ss.nrbb, (SPW + 255) / 256), 256, apply_m_smem<T>(), st>>>(p.d_sdescs.data() + ss.d0, ss.nd,
-                                                                           p.d_sn_fo.data(), p.d_sn_f.data(), arena,
-                                                                           static_cast<const T *>(fz.M.m.p), Gp);
-            MBL_LAUNCH_CHECK();
         }
     }
 }

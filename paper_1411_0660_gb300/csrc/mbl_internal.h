@@ -170,6 +170,8 @@ struct Ctx {
     size_t in_use = 0;
     size_t peak = 0;
     cudaStream_t stream = nullptr;
+    cudaStream_t side = nullptr;  // work beside `stream`, made at first use and always joined to it
+    cudaEvent_t side_ev = nullptr;
     std::string last_error;
     std::shared_ptr<PlanCache> plans = std::make_shared<PlanCache>();  // per L; shared with serving workers
     std::map<int, std::shared_ptr<EntTables>> ent;  // per sector (sector_key)
