@@ -178,9 +178,10 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int n, int x) {
     return lo;
 }
 
-// threads of the column-maximum and trsm kernels (one CTA per RB-row block): more than the block's
+// threads of the column-maximum kernel (one CTA per RB-row block): more than the block's
 // rows, so that their loads of the panel are in flight together
 constexpr int PANEL_THREADS = 256;
+constexpr int TRSM_THREADS = 128;
 
 // descriptor whose [off, off + count) range holds `b` (descs of one step are ordered by off)
 __device__ __forceinline__ int find_desc2(const PanelDesc *d, int nd, int64_t b) {
@@ -264,247 +265,286 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_panel_colmax(const PanelDesc 
     }
 }
 
-// LDL^T of a panel's w x w diagonal block with symmetric 1x1 pivoting, 128 threads.  The block is
-// kept whole (both triangles) in shared memory so that every candidate pivot's off-diagonal entries
-// lie in its own row.  A pair of threads owns row t + 1 + i of the trailing block during the update
-// of step t (the two threads take alternate columns) and the same index as candidate t + 1 + i in the
-// pivot choice of step t + 1, so the largest off-diagonal magnitude that the choice needs falls out
-// of the update.  Both mirror entries of the update subtract u_a l_b with one rounding (a the larger
-// index, u the unscaled pivot column, l = u / d), so the block stays exactly symmetric.
+// |x| as a non-negative float whose bit pattern orders like the magnitude (FP64: the high word's 20
+// mantissa bits, without a conversion on the slow FP64 pipe)
+__device__ __forceinline__ unsigned int mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned int mag_bits(double x) { return (unsigned int)__double2hiint(x) & 0x7fffffffu; }
 template <class T>
-__global__ void __launch_bounds__(128) k_panel_diag(const PanelDesc *descs, const int64_t *fo, const int32_t *fsz,
+__device__ __forceinline__ float mag_float(unsigned int b) {
+    return sizeof(T) == 4 ? __uint_as_float(b) : (float)__hiloint2double((int)b, 0);
+}
+// u / d.  FP64: by a reciprocal seeded in FP32 and two Newton steps, with the quotient's own residual
+// added: nine FP64 operations where the compiler's division takes some thirty
+__device__ __forceinline__ float pdiv(float u, float d) { return u / d; }
+__device__ __forceinline__ double pdiv(double u, double d) {
+    const float df = (float)d;
+    if (!(fabsf(df) > 1e-30f && fabsf(df) < 1e30f)) return u / d;
+    double r = (double)(1.0f / df);
+    r = fma(fma(-d, r, 1.0), r, r);
+    r = fma(fma(-d, r, 1.0), r, r);
+    const double q = u * r;
+    const double l = fma(fma(-q, d, u), r, q);
+    return fabs(q) < 1e300 ? l : u / d;  // (also infinities and NaN)
+}
+
+// LDL^T of a panel's w x w diagonal block with symmetric 1x1 pivoting, 256 threads.  The whole block
+// (both triangles) is kept in registers: thread (r, h) holds row r, columns [16 h, 16 h + 16).  Rows are
+// never exchanged: a pivot row is marked done, its column of the remaining rows becomes zero by the update
+// itself (its multiplier is 1), and the order of the pivots is applied when the factor is written.  Per
+// step: the candidates' scores go to shared memory, every warp finds the best one, the threads that hold
+// the pivot's column publish it with its multipliers, and the block updates its registers; the largest
+// off-diagonal magnitude that the next choice needs falls out of the update.  Both mirror entries of the
+// update subtract u_a l_b with one rounding (a the larger index, u the unscaled pivot column, l = u / d),
+// so the block stays exactly symmetric.
+// Bound by the chain of w dependent steps on one SM (FP64: by the SM's two FMAs a clock too).  With the
+// block in shared memory, rows exchanged and a thread pair a row, a step took 1.2 us (79 us a launch inside
+// an L = 19 factorization); this one takes 0.9 us (58), with FP64 fronts 409 -> 225 us.
+template <class T>
+__global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, const int64_t *fo, const int32_t *fsz,
                                                     const int32_t *sn_start, T *arena, T *Dg, int32_t *piv,
                                                     double tiny, unsigned long long *counters,
                                                     const unsigned int *cmax) {
-    __shared__ T B[NB][NB + 1];
-    __shared__ T ucol[NB], lcol[NB], dvec[NB];
-    __shared__ int perm[NB];
-    __shared__ float cm[NB];
-    __shared__ unsigned int s_k1[4], s_k2[4];
-    __shared__ int s_jj[4];
-    __shared__ unsigned int s_npert, s_nneg;
-    static_assert(NB == 64, "two threads per row of a 64-wide block on 128 threads");
+    static_assert(NB == 64, "four threads per row of a 64-wide block on 256 threads");
+    constexpr int CPT = NB / 4;
+    constexpr int E = 16 / sizeof(T);
+    using V = typename Vec16<T>::type;
+    __shared__ __align__(16) T ucol[NB], lcol[NB];
+    __shared__ T Ls[NB][NB + 1];  // Ls[t][r]: multiplier of row r in step t
+    __shared__ T dcand[NB], dvec[NB];
+    __shared__ int order[NB];
+    __shared__ unsigned int s_k1[NB], s_k2[NB];
     const PanelDesc d = descs[blockIdx.x];
     const int s = d.front, f = fsz[s], k0 = d.k0, w = d.w;
     T *F = arena + fo[s];
-    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, pi = tid >> 1, h = tid & 1;
-    for (int idx = tid; idx < w * w; idx += 128) {
-        const int r = idx % w, c = idx / w;
-        if (r >= c) {
-            const T v = F[(int64_t)(k0 + c) * f + k0 + r];
-            B[r][c] = v;
-            B[c][r] = v;
-        }
+    const int tid = threadIdx.x, lane = tid & 31, r = tid >> 2, h = tid & 3, c0 = h * CPT;
+    T B[CPT];
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) {
+        const int c = c0 + k, hi = max(r, c), lo = min(r, c);
+        B[k] = hi < w ? F[(int64_t)(k0 + lo) * f + k0 + hi] : T(0);
     }
-    if (tid < w) {
-        perm[tid] = tid;
-        cm[tid] = __uint_as_float(cmax[(size_t)blockIdx.x * NB + tid]);
-    }
-    if (tid == 0) s_npert = s_nneg = 0u;
-    __syncthreads();
-    // off-diagonal magnitude of candidate pi's row over the whole block (step 0)
-    float om = 0.f;
-    if (pi < w) {
-        for (int c = h; c < w; c += 2)
-            if (c != pi) om = fmaxf(om, (float)tabs(B[pi][c]));
-    }
-    om = fmaxf(om, __shfl_xor_sync(0xffffffffu, om, 1));
+    T dr = r < w ? F[(int64_t)(k0 + r) * f + k0 + r] : T(0);  // the row's diagonal entry
+    const float cm = r < w ? __uint_as_float(cmax[(size_t)blockIdx.x * NB + r]) : 0.f;
+    bool active = r < w;
+    unsigned int om = 0u;  // largest off-diagonal magnitude of the thread's part of the row
+#pragma unroll
+    for (int k = 0; k < CPT; ++k)
+        if (c0 + k != r) om = max(om, mag_bits(B[k]));
+    unsigned int npert = 0u, nneg = 0u;
     for (int t = 0; t < w; ++t) {
         // pivot: the candidate whose diagonal is largest relative to the rest of its column (inside the
         // block and, from before this panel, in the rows below), which bounds the multipliers; order:
         // largest score, then largest |d|, then the smallest index.  Scores and |d| are non-negative
-        // floats, so their bit patterns order like their values: a warp's choice is three redux.sync
-        // steps (score, then |d| among the best scores, then the smallest index).
-        {
-            const int j = t + pi;
-            const bool valid = j < w;
-            unsigned int k1 = 0u, k2 = 0u;
-            if (valid) {
-                const float o = fmaxf(om, cm[perm[j]]);
-                const float dj = (float)tabs(B[j][j]);
-                const float sc = o > 0.f ? dj / o : 3.0e38f;
-                k1 = __float_as_uint(sc) + 1u;  // 0 marks a lane without a candidate
-                k2 = __float_as_uint(dj);
-            }
-            const unsigned int m1 = __reduce_max_sync(0xffffffffu, k1);
-            const unsigned int m2 = __reduce_max_sync(0xffffffffu, k1 == m1 ? k2 : 0u);
-            const unsigned int jm =
-                __reduce_min_sync(0xffffffffu, (valid && k1 == m1 && k2 == m2) ? (unsigned int)j : (unsigned int)w);
-            if (lane == 0) {
-                s_k1[wp] = m1;
-                s_k2[wp] = m2;
-                s_jj[wp] = (int)jm;
-            }
+        // floats, so their bit patterns order like their values.
+        om = max(om, __shfl_xor_sync(0xffffffffu, om, 1));
+        om = max(om, __shfl_xor_sync(0xffffffffu, om, 2));
+        if (h == 0) {
+            const float o = fmaxf(mag_float<T>(om), cm);
+            const unsigned int db = mag_bits(dr);
+            const float sc = o > 0.f ? mag_float<T>(db) / o : 3.0e38f;
+            s_k1[r] = active ? __float_as_uint(sc) + 1u : 0u;  // 0 marks a row that is no candidate
+            s_k2[r] = db;
+            dcand[r] = dr;
         }
         __syncthreads();
-        int j = s_jj[0];
+        int j;
         {
-            // the warps hold candidates in increasing order: a later warp wins only if strictly better
-            unsigned int b1 = s_k1[0], b2 = s_k2[0];
-#pragma unroll
-            for (int v = 1; v < 4; ++v) {
-                const unsigned int k1 = s_k1[v], k2 = s_k2[v];
-                if (k1 > b1 || (k1 == b1 && k2 > b2)) {
-                    b1 = k1;
-                    b2 = k2;
-                    j = s_jj[v];
-                }
-            }
-            if (b1 == 0u || j >= w) j = t;
+            const unsigned int a1 = s_k1[lane], b1 = s_k1[lane + 32];
+            const unsigned int m1 = __reduce_max_sync(0xffffffffu, max(a1, b1));
+            const unsigned int a2 = a1 == m1 ? s_k2[lane] : 0u, b2 = b1 == m1 ? s_k2[lane + 32] : 0u;
+            const unsigned int m2 = __reduce_max_sync(0xffffffffu, max(a2, b2));
+            const unsigned int ja = a1 == m1 && a2 == m2 ? lane : NB, jb = b1 == m1 && b2 == m2 ? lane + 32 : NB;
+            j = (int)__reduce_min_sync(0xffffffffu, min(ja, jb));
         }
-        if (j != t) {
-            // symmetric exchange of indices t and j: rows over every column (the computed L rows
-            // included), then columns over the trailing rows
-            if (tid < w) {
-                const T x = B[t][tid];
-                B[t][tid] = B[j][tid];
-                B[j][tid] = x;
-            }
-            if (tid == 0) {
-                const int pp = perm[t];
-                perm[t] = perm[j];
-                perm[j] = pp;
-            }
-            __syncthreads();
-            if (tid >= t && tid < w) {
-                const T x = B[tid][t];
-                B[tid][t] = B[tid][j];
-                B[tid][j] = x;
-            }
-        }
-        __syncthreads();
-        // the pivot (a tiny one replaced by +-tiny, statically); the column: u keeps the unscaled
-        // entries, the column itself becomes L's
-        // (B[t][t] itself is left as it is: D goes to dvec)
-        T dv = B[t][t];
+        // the pivot (a tiny one replaced by +-tiny, statically)
+        T dv = dcand[j];
         const bool pert = !(tabs(dv) >= (T)tiny);
         if (pert) dv = (dv >= T(0)) ? (T)tiny : (T)(-tiny);
-        const int r = t + 1 + pi;
-        const bool own = r < w;
-        T ur = (own && h == 0) ? B[r][t] : T(0);
-        ur = __shfl_sync(0xffffffffu, ur, lane & ~1);  // the pair's second thread never reads B[r][t]
-        const T lr = own ? ur / dv : T(0);
-        if (own && h == 0) {
-            B[r][t] = lr;
-            ucol[r] = ur;
-            lcol[r] = lr;
+        // its column: u keeps the unscaled entries, l the multipliers (0 in done rows, so that they keep)
+        if (h == j / CPT) {
+            T u8[8], u4[4];  // B[j % CPT] by halving: an indexed read would put B in local memory
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u8[k] = j & 8 ? B[k + 8] : B[k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) u4[k] = j & 4 ? u8[k + 4] : u8[k];
+            const T ua = j & 2 ? u4[2] : u4[0], ub = j & 2 ? u4[3] : u4[1];
+            T u = j & 1 ? ub : ua;
+            if (!active) u = T(0);
+            if (r == j) u = dv;
+            ucol[r] = u;
+            if (sizeof(T) == 4) {
+                const T l = pdiv(u, dv);
+                lcol[r] = l;
+                Ls[t][r] = l;
+            }
+        }
+        if (sizeof(T) == 8) {  // the divisions on two full warps: FP64 instructions cost the same half empty
+            __syncthreads();
+            if (tid < NB) {
+                const T l = pdiv(ucol[tid], dv);
+                lcol[tid] = l;
+                Ls[t][tid] = l;
+            }
         }
         if (tid == 0) {
             dvec[t] = dv;
-            s_npert += pert ? 1u : 0u;
-            s_nneg += dv < T(0) ? 1u : 0u;
+            order[t] = j;
+            npert += pert ? 1u : 0u;
+            nneg += dv < T(0) ? 1u : 0u;
         }
         __syncthreads();
-        // trailing update of row r over the columns of this thread, both triangles.  The next step's
-        // choice reads only the thread's own row, so no barrier closes the step.
-        om = 0.f;
-        if (own) {
-#pragma unroll 4
-            for (int c = t + 1 + h; c < w; c += 2) {
-                const T v = c <= r ? fnms(ur, lcol[c], B[r][c]) : fnms(ucol[c], lr, B[r][c]);
-                B[r][c] = v;
-                if (c != r) om = fmaxf(om, (float)tabs(v));
+        if (r == j) active = false;
+        const T ur = active ? ucol[r] : T(0), lr = active ? lcol[r] : T(0);
+        dr = fnms(ur, lr, dr);
+        om = 0u;
+#pragma unroll
+        for (int k0v = 0; k0v < CPT; k0v += E) {
+            const V uv = *reinterpret_cast<const V *>(ucol + c0 + k0v), lv = *reinterpret_cast<const V *>(lcol + c0 + k0v);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int k = k0v + e, c = c0 + k;
+                const T uc = Vec16<T>::get(uv, e), lc = Vec16<T>::get(lv, e);
+                const T v = fnms(c <= r ? ur : uc, c <= r ? lc : lr, B[k]);
+                B[k] = v;
+                if (c != r) om = max(om, mag_bits(v));
             }
         }
-        om = fmaxf(om, __shfl_xor_sync(0xffffffffu, om, 1));
     }
     __syncthreads();
     if (tid == 0) {
-        if (s_npert) atomicAdd(&counters[0], (unsigned long long)s_npert);
-        if (s_nneg) atomicAdd(&counters[1], (unsigned long long)s_nneg);
+        if (npert) atomicAdd(&counters[0], (unsigned long long)npert);
+        if (nneg) atomicAdd(&counters[1], (unsigned long long)nneg);
     }
-    // write L11 (strictly lower), D on the diagonal, pivots
-    for (int idx = tid; idx < w * w; idx += 128) {
-        const int r = idx % w, c = idx / w;
-        if (r >= c) F[(int64_t)(k0 + c) * f + k0 + r] = r == c ? dvec[r] : B[r][c];
+    // write L11 (strictly lower) in pivot order, D on the diagonal, pivots
+    for (int idx = tid; idx < w * w; idx += 256) {
+        const int i = idx % w, c = idx / w;
+        if (i >= c) F[(int64_t)(k0 + c) * f + k0 + i] = i == c ? dvec[c] : Ls[c][order[i]];
     }
     const int64_t g0 = (int64_t)sn_start[s] + k0;
     if (tid < w) {
         Dg[g0 + tid] = dvec[tid];
-        piv[g0 + tid] = k0 + perm[tid];
+        piv[g0 + tid] = k0 + order[tid];
         float lmax = 0.f;
-        for (int r = tid + 1; r < w; ++r) lmax = fmaxf(lmax, (float)tabs(B[r][tid]));
+        for (int i = tid + 1; i < w; ++i) lmax = fmaxf(lmax, (float)tabs(Ls[tid][order[i]]));
         atomicMax(reinterpret_cast<unsigned int *>(counters + 3), __float_as_uint(lmax));
         atomicMin(reinterpret_cast<unsigned int *>(counters + 4), __float_as_uint((float)tabs(dvec[tid])));
     }
 }
 
 // W21 = A21 L11^-T by forward substitution (one thread per row, no explicit inverse), then
-// L21 = W21 D^-1.  The columns of A21 are read in the panel's pivoted order.
+// L21 = W21 D^-1.  The columns of A21 are read in the panel's pivoted order.  A row is held in registers
+// and eliminated column by column: 2016 independent FMAs with the entries of L11 broadcast from shared
+// memory, where the row in shared memory and one running sum was a chain of as many dependent ones.
+// Bound by latency (a few CTAs of two working warps): 16 us a launch at L = 19 where that took 37.
 template <class T>
-__global__ void __launch_bounds__(PANEL_THREADS) k_panel_trsm(const PanelDesc *descs, int nd, const int64_t *fo,
+__global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *descs, int nd, const int64_t *fo,
                                                    const int32_t *fsz, const int32_t *sn_start, T *arena,
                                                    const T *Dg, const int32_t *piv, T *wscr,
                                                    unsigned long long *stats, void *pieces, int64_t prow,
                                                    int pmode) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T(*Lb)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(smraw);                      // L11
-    T(*As)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(smraw + sizeof(T) * NB * (NB + 1));
+    static_assert(RB == NB && NB == 64, "a thread per row, a register per column");
+    constexpr int E = 16 / sizeof(T);
+    using V = typename Vec16<T>::type;
+    __shared__ __align__(16) T Ls[NB * NB];  // L11 by columns; then W21 by rows
     __shared__ T Dinv[NB];
     __shared__ int pv[NB];
     const int di = find_desc2(descs, nd, blockIdx.x);
     const PanelDesc d = descs[di];
     const int s = d.front, f = fsz[s], k0 = d.k0, w = d.w, m2 = d.m2;
-    const int r0 = k0 + w + (int)(blockIdx.x - d.off2) * RB;
+    const int rb = (int)(blockIdx.x - d.off2) * RB, r0 = k0 + w + rb;  // rb: relative to the trailing block
     const int nr = min(RB, f - r0);
     T *F = arena + fo[s];
     const int tid = threadIdx.x;
     const int64_t g0 = (int64_t)sn_start[s] + k0;
-    for (int idx = tid; idx < w * w; idx += blockDim.x) {
-        int r = idx % w, c = idx / w;
-        Lb[r][c] = (r > c) ? F[(int64_t)(k0 + c) * f + k0 + r] : T(0);
+    for (int idx = tid; idx < NB * NB; idx += TRSM_THREADS) {
+        const int r = idx % NB, c = idx / NB;
+        Ls[idx] = (r > c && r < w) ? F[(int64_t)(k0 + c) * f + k0 + r] : T(0);
     }
-    if (tid < w) {
-        Dinv[tid] = T(1) / Dg[g0 + tid];
-        pv[tid] = piv[g0 + tid];
-    }
-    __syncthreads();
-    for (int idx = tid; idx < nr * w; idx += blockDim.x) {
-        int i = idx % nr, k = idx / nr;
-        As[i][k] = F[(int64_t)pv[k] * f + r0 + i];
+    if (tid < NB) {
+        Dinv[tid] = tid < w ? T(1) / Dg[g0 + tid] : T(0);
+        pv[tid] = tid < w ? piv[g0 + tid] : 0;
     }
     __syncthreads();
-    if (tid < nr) {
-        T *a = As[tid];
-        for (int t = 1; t < w; ++t) {
-            T acc = a[t];
-            for (int k = 0; k < t; ++k) acc -= a[k] * Lb[t][k];
-            a[t] = acc;
-        }
-    }
-    __syncthreads();
-    T *W = wscr + d.woff;
+    const bool own = tid < nr;
     float lmax = 0.f;
-    for (int idx = tid; idx < nr * w; idx += blockDim.x) {
-        int i = idx % nr, t = idx / nr;
-        T x = As[i][t];
-        T l = x * Dinv[t];
-        F[(int64_t)(k0 + t) * f + r0 + i] = l;
-        W[(int64_t)(r0 - k0 - w + i) + (int64_t)t * m2] = x;
-        lmax = fmaxf(lmax, (float)tabs(l));
+    T x[NB];
+    if (tid < RB) {
+#pragma unroll
+        for (int k = 0; k < NB; ++k) x[k] = own && k < w ? F[(int64_t)pv[k] * f + r0 + tid] : T(0);
+#pragma unroll
+        for (int t = 0; t < NB - 1; ++t) {
+            if (t % 16 == 0 && t >= w) break;
+#pragma unroll
+            for (int k = (t + 1) / E * E; k < NB; k += E) {
+                const V l = *reinterpret_cast<const V *>(Ls + t * NB + k);
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (k + e > t) x[k + e] = fnms(x[t], Vec16<T>::get(l, e), x[k + e]);
+            }
+        }
+        if (own) {
+            T *W = wscr + d.woff + rb + tid;
+#pragma unroll
+            for (int t = 0; t < NB; ++t) {
+                if (t >= w) break;
+                const T l = x[t] * Dinv[t];
+                F[(int64_t)(k0 + t) * f + r0 + tid] = l;
+                W[(int64_t)t * m2] = x[t];
+                lmax = fmaxf(lmax, (float)tabs(l));
+            }
+        }
     }
     if (sizeof(T) == 4 && pmode) {
         // tensor-core operand pieces of this block's rows of L21 and W21 (pieces 0/1 and 2/3), row-major
-        // with NB per row, zero past the panel width; rows start at the descriptor's woff / NB
-        const int64_t rb = d.woff / NB + (r0 - k0 - w);
-        for (int idx = tid; idx < nr * NB; idx += blockDim.x) {
-            const int i = idx / NB, t = idx - i * NB;
-            const float xv = t < w ? (float)As[i][t] : 0.f;
-            const float lv = t < w ? (float)(As[i][t] * Dinv[t]) : 0.f;
-            const int64_t e = (rb + i) * NB + t;
+        // with NB per row, zero past the panel width; rows start at the descriptor's woff / NB.  W21 goes
+        // through shared memory (16-byte group g of row i at g ^ (i % 16): no bank conflicts) so that
+        // the pieces leave in whole rows.
+        __syncthreads();
+        V *Wv = reinterpret_cast<V *>(Ls);
+        if (tid < RB) {
+#pragma unroll
+            for (int g = 0; g < NB / E; ++g) {
+                V v;
+                T *ve = reinterpret_cast<T *>(&v);
+#pragma unroll
+                for (int e = 0; e < E; ++e) ve[e] = x[g * E + e];
+                Wv[tid * (NB / E) + (g ^ (tid % (NB / E)))] = v;
+            }
+        }
+        __syncthreads();
+        const int64_t p0 = d.woff / NB + rb;
+        for (int idx = tid; idx < nr * (NB / 4); idx += TRSM_THREADS) {
+            const int i = idx / (NB / 4), g = idx % (NB / 4);
+            const float *xr = reinterpret_cast<const float *>(Wv) + ((size_t)i * (NB / 4) + (g ^ (i % (NB / 4)))) * 4;
+            const int64_t e = (p0 + i) * NB + g * 4;
             if (pmode == 1) {
+                uint32_t v[4][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    split_tf32((float)(xr[u] * (float)Dinv[g * 4 + u]), v[0][u], v[1][u]);
+                    split_tf32(xr[u], v[2][u], v[3][u]);
+                }
                 uint32_t *P = static_cast<uint32_t *>(pieces);
-                split_tf32(lv, P[e], P[prow * NB + e]);
-                split_tf32(xv, P[2 * prow * NB + e], P[3 * prow * NB + e]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    *reinterpret_cast<uint4 *>(P + q * prow * NB + e) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
             } else {
+                uint16_t v[4][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    split_bf16((float)(xr[u] * (float)Dinv[g * 4 + u]), v[0][u], v[1][u]);
+                    split_bf16(xr[u], v[2][u], v[3][u]);
+                }
                 uint16_t *P = static_cast<uint16_t *>(pieces);
-                split_bf16(lv, P[e], P[prow * NB + e]);
-                split_bf16(xv, P[2 * prow * NB + e], P[3 * prow * NB + e]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    *reinterpret_cast<uint2 *>(P + q * prow * NB + e) =
+                        make_uint2(v[q][0] | (uint32_t)v[q][1] << 16, v[q][2] | (uint32_t)v[q][3] << 16);
             }
         }
     }
     for (int o = 16; o > 0; o >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-    if ((tid & 31) == 0) atomicMax(reinterpret_cast<unsigned int *>(stats), __float_as_uint(lmax));
+    if ((tid & 31) == 0 && lmax > 0.f) atomicMax(reinterpret_cast<unsigned int *>(stats), __float_as_uint(lmax));
 }
 
 // Trailing update of one 64 x 64 lower tile: C[i][j] -= sum_t L21[i][t] W21[j][t]
@@ -1227,8 +1267,6 @@ __global__ void __launch_bounds__(256) k_bwd_step(const SolveDesc *sdescs, const
 // Host drivers
 // ------------------------------------------------------------------------------------------
 template <class T>
-static size_t trsm_smem() { return sizeof(T) * (size_t)2 * NB * (NB + 1); }
-template <class T>
 static size_t apply_m_smem() { return sizeof(T) * ((size_t)RBB * 33 + (size_t)32 * 257); }
 template <class T, int PB>
 static size_t fwd_step_smem() { return fwd_gtile_bytes<T>() + sizeof(T) * (size_t)SPW * PB; }
@@ -1318,7 +1356,6 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
             static_cast<const T *>(fz.M.m.p), Gp);
         MBL_LAUNCH_CHECK();
     };
-    smem_limit((const void *)k_panel_trsm<T>, trsm_smem<T>());
     set_solve_attrs<T>();
     MBL_CUDA(cudaMemsetAsync(fz.counters.data(), 0, 5 * sizeof(unsigned long long), st));
     MBL_CUDA(cudaMemsetAsync(fz.counters.data() + 4, 0x7f, sizeof(unsigned int), st));  // min |d| starts huge
@@ -1359,11 +1396,11 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                                                                        cmax);
                     MBL_LAUNCH_CHECK();
                 }
-                k_panel_diag<T><<<stp.nd, 128, 0, st>>>(dd, p.d_sn_fo.data(), p.d_sn_f.data(), p.d_sn_start.data(), arena,
+                k_panel_diag<T><<<stp.nd, 256, 0, st>>>(dd, p.d_sn_fo.data(), p.d_sn_f.data(), p.d_sn_start.data(), arena,
                                                         Dg, fz.piv.data(), fz.tiny, fz.counters.data(), cmax);
                 MBL_LAUNCH_CHECK();
                 if (stp.n2 > 0) {
-                    k_panel_trsm<T><<<(unsigned)stp.n2, PANEL_THREADS, trsm_smem<T>(), st>>>(dd, stp.nd, p.d_sn_fo.data(),
+                    k_panel_trsm<T><<<(unsigned)stp.n2, TRSM_THREADS, 0, st>>>(dd, stp.nd, p.d_sn_fo.data(),
                                                                                  p.d_sn_f.data(), p.d_sn_start.data(), arena,
                                                                                  Dg, fz.piv.data(), wscr,
                                                                                  fz.counters.data() + 3,
