@@ -273,9 +273,13 @@ template <class T>
 __device__ __forceinline__ float mag_float(unsigned int b) {
     return sizeof(T) == 4 ? __uint_as_float(b) : (float)__hiloint2double((int)b, 0);
 }
-// u / d.  FP64: by a reciprocal seeded in FP32 and two Newton steps, with the quotient's own residual
-// added: nine FP64 operations where the compiler's division takes some thirty
-__device__ __forceinline__ float pdiv(float u, float d) { return u / d; }
+// u / d by a reciprocal and the quotient's own residual (a shorter chain than the division's).  FP64: the
+// reciprocal from FP32 by two Newton steps, nine FP64 operations where the division takes some thirty.
+__device__ __forceinline__ float pdiv(float u, float d) {
+    const float r = __fdividef(1.0f, d), q = u * r;
+    if (!(fabsf(d) > 1e-30f && fabsf(d) < 1e30f && fabsf(q) < 1e30f && (fabsf(q) > 1e-30f || u == 0.0f))) return u / d;
+    return __fmaf_rn(__fmaf_rn(-q, d, u), r, q);
+}
 __device__ __forceinline__ double pdiv(double u, double d) {
     const float df = (float)d;
     if (!(fabsf(df) > 1e-30f && fabsf(df) < 1e30f)) return u / d;
@@ -298,7 +302,7 @@ __device__ __forceinline__ double pdiv(double u, double d) {
 // so the block stays exactly symmetric.
 // Bound by the chain of w dependent steps on one SM (FP64: by the SM's two FMAs a clock too).  With the
 // block in shared memory, rows exchanged and a thread pair a row, a step took 1.2 us (79 us a launch inside
-// an L = 19 factorization); this one takes 0.9 us (58), with FP64 fronts 409 -> 225 us.
+// an L = 19 factorization); this one takes 0.75 us (50), with FP64 fronts 409 -> 230 us.
 template <class T>
 __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, const int64_t *fo, const int32_t *fsz,
                                                     const int32_t *sn_start, T *arena, T *Dg, int32_t *piv,
@@ -341,7 +345,7 @@ __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, cons
         if (h == 0) {
             const float o = fmaxf(mag_float<T>(om), cm);
             const unsigned int db = mag_bits(dr);
-            const float sc = o > 0.f ? mag_float<T>(db) / o : 3.0e38f;
+            const float sc = o > 0.f ? pdiv(mag_float<T>(db), o) : 3.0e38f;
             s_k1[r] = active ? __float_as_uint(sc) + 1u : 0u;  // 0 marks a row that is no candidate
             s_k2[r] = db;
             dcand[r] = dr;
@@ -648,22 +652,34 @@ __device__ __forceinline__ int find_sdesc_b(const SolveDesc *d, int nd, int64_t 
     return lo;
 }
 
-// M of one solve panel, 8 columns per CTA, in FP64: the forward sequence (pivot permutation,
+// FP32 to FP64 by the bits: the conversion instruction runs on the FP64 pipe, two lanes a clock and SM
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned int u = __float_as_uint(x), e = (u >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// M of one solve panel, 4 columns per CTA, in FP64: the forward sequence (pivot permutation,
 // unit-lower substitution, elimination of the later rows of the panel) applied to unit vectors.  A warp
 // takes one column and keeps it in registers (lane l holds rows l, l + 32, ...): step t broadcasts entry t
-// and every lane subtracts its rows' share, so a column is one chain of w shuffles and FMAs without a
-// barrier.  M is block lower triangular in the NB-wide sub-panels: a unit vector is zero above its own.
-// Bound by the FP64 rate (two FMAs a clock and SM); 8 columns a CTA spread the 256 columns of a panel over
-// 32 SMs, so that a step of one or two panels is not held on a few.
+// and every lane subtracts its rows' share.  The CTA stages BM_T columns of L at a time, widened once, in
+// shared memory.  M is block lower triangular in the NB-wide sub-panels: a unit vector is zero above its
+// own.
+// Bound by the FP64 rate (two FMAs a clock and SM), so the work is spread thin: 4 columns a CTA put one
+// panel on 64 SMs.  A step's launch takes 166 us at L = 19 (beside the panel steps); with 8 columns a CTA and
+// each warp widening L for itself it took 303.
+constexpr int BM_T = 16;
 template <class T>
-__global__ void __launch_bounds__(256) k_build_m(const SolveDesc *sdescs, const int64_t *fo, const int32_t *fsz,
+__global__ void __launch_bounds__(128) k_build_m(const SolveDesc *sdescs, const int64_t *fo, const int32_t *fsz,
                                                  const int32_t *sn_start, const T *__restrict__ arena,
                                                  const int32_t *piv, T *Mall) {
-    static_assert(NB == 64 && SPW == 256, "two rows per lane and sub-panel");
-    __shared__ double perm[8][NB];
+    static_assert(NB == 64 && SPW == 256 && BM_T == 16, "two rows per lane and sub-panel, two chunks per row slot");
+    __shared__ double perm[4][NB];
+    __shared__ double Lc[BM_T][SPW];
     const SolveDesc d = sdescs[blockIdx.x];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, w = d.w, c = blockIdx.y * 8 + wp;
-    if (c >= w) return;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, w = d.w, cf = blockIdx.y * 4, c = cf + wp;
+    if (cf >= w) return;
     const int f = fsz[d.front], k0 = d.k0;
     const T *F = arena + fo[d.front] + (int64_t)k0 * f + k0;  // the panel's diagonal block
     const int32_t *pv = piv + (int64_t)sn_start[d.front] + k0;
@@ -673,7 +689,7 @@ __global__ void __launch_bounds__(256) k_build_m(const SolveDesc *sdescs, const 
 #pragma unroll
     for (int u = 0; u < SUBS; ++u) {
         const int s0 = u * NB;
-        if (s0 + NB <= c || s0 >= w) continue;
+        if (s0 + NB <= cf || s0 >= w) continue;
         perm[wp][lane] = z[2 * u];
         perm[wp][lane + 32] = z[2 * u + 1];
         __syncwarp();
@@ -681,22 +697,27 @@ __global__ void __launch_bounds__(256) k_build_m(const SolveDesc *sdescs, const 
         z[2 * u + 1] = s0 + 32 + lane < w ? perm[wp][pv[s0 + 32 + lane] - k0 - s0] : 0.0;
         __syncwarp();
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int tn = min(32, w - s0 - 32 * h);
-#pragma unroll 4
-            for (int tt = 0; tt < tn; ++tt) {
-                const int t = s0 + 32 * h + tt;
-                const T *Fc = F + (int64_t)t * f;
-                const double zt = __shfl_sync(0xffffffffu, z[2 * u + h], tt);
+        for (int ch = 0; ch < NB / BM_T; ++ch) {
+            const int t0 = s0 + BM_T * ch;
+            if (t0 >= w) break;
+            __syncthreads();
 #pragma unroll
-                for (int i = 2 * u + h; i < SPW / 32; ++i) {
-                    const int r = lane + 32 * i;
-                    const double l = r > t && r < w ? (double)Fc[r] : 0.0;
-                    z[i] = fma(-l, zt, z[i]);
+            for (int tt = 0; tt < BM_T; ++tt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int r = (int)threadIdx.x + 128 * h, t = t0 + tt;
+                    if (128 * h + 127 > t0) Lc[tt][r] = r > t && r < w && t < w ? widen(F[(int64_t)t * f + r]) : 0.0;
                 }
+            __syncthreads();
+#pragma unroll
+            for (int tt = 0; tt < BM_T; ++tt) {
+                const double zt = __shfl_sync(0xffffffffu, z[2 * u + ch / 2], (ch % 2) * BM_T + tt);
+#pragma unroll
+                for (int i = 2 * u + ch / 2; i < SPW / 32; ++i) z[i] = fma(-Lc[tt][lane + 32 * i], zt, z[i]);
             }
         }
     }
+    if (c >= w) return;
     T *M = Mall + d.moff + (int64_t)c * w;
 #pragma unroll
     for (int i = 0; i < SPW / 32; ++i)
@@ -1347,7 +1368,7 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
         const SolveStep &ss = p.ssteps[si];
         if (ss.nd <= 0) return;
         ProfScope ps_g(fz.ctx, "f_build_g", 0.0, sg);
-        k_build_m<T><<<dim3((unsigned)ss.nd, (ss.maxw + 7) / 8), 256, 0, sg>>>(
+        k_build_m<T><<<dim3((unsigned)ss.nd, (ss.maxw + 3) / 4), 128, 0, sg>>>(
             p.d_sdescs.data() + ss.d0, p.d_sn_fo.data(), p.d_sn_f.data(), p.d_sn_start.data(), arena, fz.piv.data(),
             static_cast<T *>(fz.M.m.p));
         MBL_LAUNCH_CHECK();
