@@ -247,18 +247,22 @@ struct Num<float> {
     static __device__ __forceinline__ float tiny() { return FLT_MIN; }
 };
 
+// Sum over the block (at most 32 warps), the same value in every thread.  red: 32 entries that no thread
+// still reads from an earlier call without a barrier in between.
 template <class R>
-__device__ R block_sum(R v, R *red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
+__device__ R block_sum1(R v, R *red) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (lane == 0) red[w] = v;
     __syncthreads();
-    R s = R(0);
-    int nw = (blockDim.x + 31) >> 5;
-    for (int i = 0; i < nw; ++i) s += red[i];
-    __syncthreads();
+    R s = lane < (int)(blockDim.x >> 5) ? red[lane] : R(0);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
+}
+template <class R>
+__device__ R block_sum(R v, R *red) {
+    __syncthreads();
+    return block_sum1(v, red);
 }
 
 // Sturm count: number of eigenvalues of T(d, e2) below x.
@@ -274,6 +278,64 @@ __device__ int sturm_count(int m, const R *d, const R *e2, R x, R pivmin) {
         c += q < R(0);
     }
     return c;
+}
+
+// The same count from the leading minors p_i = (d_i - x) p_{i-1} - e2_{i-1} p_{i-2} themselves (Givens,
+// 1954): their sign changes.  Three FP64 operations a row where the quotient form's division takes some
+// thirty, on a part with two FP64 FMAs a clock and SM.  T scaled to a norm of about 1 (so that two rows
+// change a minor by no more than 2^+-400: a zero minor is replaced by -2^-200 times the last, as the
+// quotient form replaces a zero pivot); both minors are rescaled when they leave [2^-300, 2^300].
+__device__ __forceinline__ int sturm_count_minors(int m, const double *d, const double *e2, double x) {
+    double p0 = 1.0, p1 = d[0] - x;
+    if (p1 == 0.0) p1 = -0x1p-200;
+    int c = __double2hiint(p1) < 0;
+    for (int i = 1; i < m; ++i) {
+        double p2 = fma(d[i] - x, p1, -(e2[i - 1] * p0));
+        if (p2 == 0.0) p2 = p1 * -0x1p-200;
+        c += (__double2hiint(p2) ^ __double2hiint(p1)) < 0;
+        p0 = p1;
+        p1 = p2;
+        if (i & 1) {
+            const int x0 = (__double2hiint(p0) >> 20) & 0x7ff, x1 = (__double2hiint(p1) >> 20) & 0x7ff, xm = max(x0, x1);
+            if ((unsigned)(xm - 723) > 600u) {
+                const double f = __hiloint2double((2046 - xm) << 20, 0);
+                p0 *= f;
+                p1 *= f;
+            }
+        }
+    }
+    return c;
+}
+
+// c, s, r of the rotation that takes (x, z) to (r, 0): FP32 by the reciprocal square root and one Newton
+// step (a chain of some 60 clocks against 200 of hypotf and a division)
+__device__ __forceinline__ void ql_rotation(float x, float z, float &c, float &s, float &r) {
+    const float r2 = fmaf(x, x, z * z);
+    if (r2 > 1e-30f && r2 < 1e30f) {
+        float ir = rsqrtf(r2);
+        ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.0f), ir);
+        c = x * ir;
+        s = z * ir;
+        r = r2 * ir;
+        return;
+    }
+    r = hypotf(x, z);
+    c = 1.0f;
+    s = 0.0f;
+    if (r != 0.0f) {
+        c = x / r;
+        s = z / r;
+    }
+}
+__device__ __forceinline__ void ql_rotation(double x, double z, double &c, double &s, double &r) {
+    r = hypot(x, z);
+    c = 1.0;
+    s = 0.0;
+    if (r != 0.0) {
+        const double ir = 1.0 / r;
+        c = x * ir;
+        s = z * ir;
+    }
 }
 
 // One implicit QL sweep on the unreduced block lo..hi of (d, e), recording the rotations:
@@ -298,13 +360,8 @@ __device__ void ql_sweep_record(int lo, int hi, R *d, R *e, R *cs, R *sn) {
         // the entries the next rotation meets first
         const R a_next = k > lo ? d[k - 1] : R(0);
         const R em_next = k - 1 > lo ? e[k - 2] : R(0);
-        R r = hypot(x, z);
-        R c = R(1), s = R(0);
-        if (r != R(0)) {
-            R ir = R(1) / r;
-            c = x * ir;
-            s = z * ir;
-        }
+        R r, c, s;
+        ql_rotation(x, z, c, s, r);
         if (k < hi - 1) e[k + 1] = r;
         const R bb = ek, dd = dk1;
         const R dk = a * c * c - R(2) * bb * c * s + dd * s * s;
@@ -328,52 +385,56 @@ __device__ void ql_sweep_record(int lo, int hi, R *d, R *e, R *cs, R *sn) {
     d[lo] = dk1;
 }
 
-// Householder reduction of the symmetric m x m matrix a (column-major, lower triangle used, leading
-// dimension lda) to tridiagonal form, by the whole block: afterwards the diagonal and subdiagonal are
-// on a's diagonals, the reflectors' tails below the subdiagonal and their scalings in beta.
+// Householder reduction of the symmetric m x m matrix a (column-major, leading dimension lda) to
+// tridiagonal form, by the whole block: afterwards the diagonal and subdiagonal are on a's diagonals, the
+// reflectors' tails below the subdiagonal and their scalings in beta.  red: 64 entries.  Bound by the chain
+// of m steps: four barriers a step (the norm, the reflector, the product, the update); four lanes share a
+// row of the product.
 template <class R>
 __device__ void householder_tridiag(R *a, int lda, int m, R *beta, R *vv, R *pp, R *red) {
     for (int k = 0; k + 2 < m; ++k) {
-        int len = m - k - 1;
+        const int len = m - k - 1;
         R *x = a + (size_t)k * lda + (k + 1);
         R loc = R(0);
         for (int i = threadIdx.x; i < len; i += blockDim.x) loc += x[i] * x[i];
-        R alpha2 = block_sum(loc, red);
+        const R alpha2 = block_sum1(loc, red);
         if (alpha2 == R(0)) {
             if (threadIdx.x == 0) beta[k] = R(0);
             __syncthreads();
             continue;
         }
-        R x0 = x[0];
-        R sgn = x0 >= R(0) ? R(1) : R(-1);
-        R alpha = sqrt(alpha2);
-        R v0 = x0 + sgn * alpha;
-        R iv0 = R(1) / v0;
-        loc = R(0);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) {
-            R v = (i == 0) ? R(1) : x[i] * iv0;
-            vv[i] = v;
-            if (i > 0) loc += v * v;
-        }
-        R vtv = R(1) + block_sum(loc, red);
-        R bk = R(2) / vtv;
+        const R x0 = x[0];
+        const R sgn = x0 >= R(0) ? R(1) : R(-1);
+        const R alpha = sqrt(alpha2);
+        const R v0 = x0 + sgn * alpha;
+        const R iv0 = R(1) / v0;
+        // v = x / v0 with v_0 = 1: 2 / |v|^2 = |v0| / alpha
+        const R bk = fabs(v0) / alpha;
+        for (int i = threadIdx.x; i < len; i += blockDim.x) vv[i] = i == 0 ? R(1) : x[i] * iv0;
+        __syncthreads();
         R *A22 = a + (size_t)(k + 1) * lda + (k + 1);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) {
-            R s = R(0);
-            for (int j = 0; j < len; ++j) s = fma(A22[(size_t)j * lda + i], vv[j], s);
-            pp[i] = bk * s;
-        }
-        __syncthreads();
+        const int part = threadIdx.x & 3, step = blockDim.x >> 2;
         loc = R(0);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) loc += pp[i] * vv[i];
-        R K = R(0.5) * bk * block_sum(loc, red);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) pp[i] -= K * vv[i];
-        __syncthreads();
-        for (int t = threadIdx.x; t < len * len; t += blockDim.x) {
-            int i = t % len, j = t / len;
-            A22[(size_t)j * lda + i] -= vv[i] * pp[j] + pp[i] * vv[j];
+        for (int i0 = 0; i0 < len; i0 += step) {
+            const int i = i0 + (int)(threadIdx.x >> 2);
+            R s = R(0);
+            if (i < len)
+                for (int j = part; j < len; j += 4) s = fma(A22[(size_t)j * lda + i], vv[j], s);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (i < len && part == 0) {
+                s *= bk;
+                pp[i] = s;
+                loc += s * vv[i];
+            }
         }
-        __syncthreads();
+        const R K = R(0.5) * bk * block_sum1(loc, red + 32);
+        // A22 -= v w^T + w v^T with w = p - K v
+        for (int t = threadIdx.x; t < len * len; t += blockDim.x) {
+            const int i = t % len, j = t / len;
+            const R vi = vv[i], vj = vv[j];
+            A22[(size_t)j * lda + i] -= vi * (pp[j] - K * vj) + (pp[i] - K * vi) * vj;
+        }
         for (int i = threadIdx.x; i < len; i += blockDim.x) x[i] = (i == 0) ? -sgn * alpha : vv[i];
         if (threadIdx.x == 0) beta[k] = bk;
         __syncthreads();
@@ -389,7 +450,8 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
                                                       size_t wstride, int *info, int smem_m, int zsm) {
     extern __shared__ __align__(16) unsigned char smraw[];
     R *sm = reinterpret_cast<R *>(smraw);
-    __shared__ R red[EIG_THREADS / 32];
+    __shared__ R red[64];
+    __shared__ R q_d[EIG_QL_MAX], q_e[EIG_QL_MAX];
     __shared__ R s_gl, s_gu, s_pivmin, s_atol;
     int b = blockIdx.x;
     int m = mv[b];
@@ -421,7 +483,9 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
     }
     int lda = m;
     // ---- 1. Householder tridiagonalization ----
-    householder_tridiag(a, lda, m, beta, vv, pp, red);
+    // (its vectors in shared memory where they fit: every lane reads them in every step)
+    if (m <= EIG_QL_MAX) householder_tridiag(a, lda, m, beta, q_d, q_e, red);
+    else householder_tridiag(a, lda, m, beta, vv, pp, red);
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
         d[i] = a[(size_t)i * lda + i];
         if (i + 1 < m) {
@@ -452,6 +516,31 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
         // every eigenvalue to an absolute accuracy of 2 eps ||T|| (LAPACK's choice of ABSTOL for
         // eigenvalues to full accuracy relative to the norm): an eigenvalue near zero -- most of an
         // entanglement spectrum -- is not bisected on to its own relative precision
+        if constexpr (sizeof(R) == 8) {
+            if (m <= EIG_QL_MAX) {
+                // counts from the minors, on T scaled by a power of two to a norm in [1, 2)
+                const double tn = fmax(fabs(s_gl), fabs(s_gu));
+                const int ex = tn > 0.0 && tn < INFINITY ? ilogb(tn) : 0;
+                for (int i = threadIdx.x; i < m; i += blockDim.x) {
+                    q_d[i] = scalbn(d[i], -ex);
+                    const double es = i + 1 < m ? scalbn(e[i], -ex) : 0.0;
+                    q_e[i] = es * es;
+                }
+                __syncthreads();
+                const double atol = scalbn(s_atol, -ex);
+                for (int j = threadIdx.x; j < m; j += blockDim.x) {
+                    double lo = scalbn(s_gl, -ex), hi = scalbn(s_gu, -ex);
+                    for (int it = 0; it < 200; ++it) {
+                        const double mid = 0.5 * (lo + hi);
+                        if (hi - lo <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) || hi - lo <= atol || mid == lo || mid == hi)
+                            break;
+                        if (sturm_count_minors(m, q_d, q_e, mid) > j) hi = mid; else lo = mid;
+                    }
+                    W[j] = scalbn(0.5 * (lo + hi), ex);
+                }
+                return;
+            }
+        }
         for (int j = threadIdx.x; j < m; j += blockDim.x) {
             R lo = s_gl, hi = s_gu;
             for (int it = 0; it < 200; ++it) {
@@ -466,68 +555,85 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
         return;
     }
     // ---- 3. implicit QL on (d, e) accumulating Z (column-major m x m, starts as identity) ----
-    // the sweeps run on one thread as a chain of dependent updates of d, e and the rotation list:
-    // keep those in shared memory (global memory would put an L2 round trip in every link)
-    __shared__ R q_d[EIG_QL_MAX], q_e[EIG_QL_MAX], q_cs[EIG_QL_MAX], q_sn[EIG_QL_MAX];
-    R *cs = pp, *sn = vv;  // reuse the Householder scratch for the sweep's rotations
+    // one lane generates a sweep's rotations (a chain of dependent updates of d, e and the rotation list,
+    // kept in shared memory: global memory would put an L2 round trip in every link); the other warps apply
+    // the sweep before it to Z meanwhile.  Two rotation lists alternate.
+    __shared__ R q_cs[2][EIG_QL_MAX], q_sn[2][EIG_QL_MAX];
+    __shared__ int s_lo[2], s_hi[2], s_done[2], s_fail;
+    R *cs = pp;  // the order of the eigenvalues, later
     {
-        if (m <= EIG_QL_MAX) {
+        const bool qsm = m <= EIG_QL_MAX;
+        if (qsm) {
             for (int i = threadIdx.x; i < m; i += blockDim.x) {
                 q_d[i] = d[i];
                 q_e[i] = e[i];
             }
             d = q_d;
             e = q_e;
-            cs = q_cs;
-            sn = q_sn;
         }
+        R *csb[2] = {qsm ? q_cs[0] : work + 3 * m, qsm ? q_cs[1] : work + 5 * m};  // (vv and e2 are free now)
+        R *snb[2] = {qsm ? q_sn[0] : work + 6 * m, qsm ? q_sn[1] : work + 7 * m};
         for (int t = threadIdx.x; t < m * m; t += blockDim.x) Z[t] = ((t / m) == (t % m)) ? R(1) : R(0);
-        __shared__ int s_lo, s_hi, s_done, s_fail;
-        if (threadIdx.x == 0) { s_lo = 0; s_done = 0; s_fail = 0; }
+        if (threadIdx.x == 0) s_fail = 0;
         __syncthreads();
-        int iter = 0;
-        while (true) {
-            if (threadIdx.x == 0) {
-                int lo = s_lo;
-                s_hi = -1;
-                while (lo < m - 1) {
-                    if (fabs(e[lo]) <= Num<R>::eps() * (fabs(d[lo]) + fabs(d[lo + 1]))) {
-                        e[lo] = R(0);
-                        ++lo;
-                        iter = 0;
-                        continue;
+        const int lane = threadIdx.x & 31;
+        int iter = 0, nlo = 0;  // (warp 0)
+        for (int buf = 0;; buf ^= 1) {
+            if (threadIdx.x < 32) {
+                // first entry of e at or after `from` that is negligible (want = true) or not, else m - 1
+                auto scan = [&](int from, bool want) {
+                    for (int k0 = from; k0 < m - 1; k0 += 32) {
+                        const int k = k0 + lane;
+                        const bool small = k < m - 1 && fabs(e[k]) <= Num<R>::eps() * (fabs(d[k]) + fabs(d[k + 1]));
+                        const unsigned int hit = __ballot_sync(0xffffffffu, k < m - 1 && small == want);
+                        if (hit) return k0 + __ffs(hit) - 1;
                     }
-                    int hi = lo + 1;
-                    while (hi < m - 1 && !(fabs(e[hi]) <= Num<R>::eps() * (fabs(d[hi]) + fabs(d[hi + 1])))) ++hi;
-                    if (hi < m - 1) e[hi] = R(0);
-                    if (++iter > 100) { s_fail = 1; lo = m; break; }
-                    ql_sweep_record(lo, hi, d, e, cs, sn);
-                    s_hi = hi;
-                    break;
+                    return m - 1;
+                };
+                const int lo = scan(nlo, false);
+                if (lo != nlo) {
+                    for (int k = nlo + lane; k < lo; k += 32) e[k] = R(0);
+                    iter = 0;
+                    nlo = lo;
                 }
-                s_lo = lo;
-                if (lo >= m - 1) s_done = 1;
+                int hi = -1;
+                bool done = lo >= m - 1;
+                if (!done) {
+                    hi = scan(lo + 1, true);
+                    if (++iter > 100) {
+                        done = true;
+                        hi = -1;
+                        if (lane == 0) s_fail = 1;
+                    } else if (lane == 0) {
+                        if (hi < m - 1) e[hi] = R(0);
+                        ql_sweep_record(lo, hi, d, e, csb[buf], snb[buf]);
+                    }
+                }
+                if (lane == 0) {
+                    s_lo[buf] = lo;
+                    s_hi[buf] = hi;
+                    s_done[buf] = done;
+                }
+                __syncwarp();
             }
             __syncthreads();
-            // every thread takes the exit decision here, between the barriers: thread 0 rewrites
-            // s_done (and s_lo, s_hi) as soon as it has passed the barrier below, so a thread
-            // reading s_done after that barrier could see the next sweep's value, leave the loop
-            // one sweep early and reach the barriers after the loop out of step with the block
-            const bool done = s_done != 0;
-            if (s_hi >= 0) {
-                int lo = s_lo, hi = s_hi;
-                // Z is column-major (column k contiguous): thread r walks its row down the sweep,
+            // this sweep is applied while warp 0 generates the next one into the other list (which the
+            // previous sweep's application left before this barrier)
+            const int lo = s_lo[buf], hi = s_hi[buf];
+            if (threadIdx.x >= 32 && hi >= 0) {
+                const R *c_ = csb[buf], *s_ = snb[buf];
+                // Z is column-major (column k contiguous): a thread walks its row down the sweep,
                 // carrying the rotated entry of column k + 1; accesses coalesce across threads
                 // (the next rotation's inputs are loaded before this one's store, which the compiler
                 // could not otherwise move ahead of it: Z and the rotation list might alias)
-                for (int r = threadIdx.x; r < m; r += blockDim.x) {
+                for (int r = (int)threadIdx.x - 32; r < m; r += (int)blockDim.x - 32) {
                     R a1 = Z[(size_t)hi * m + r];
                     R a0 = Z[(size_t)(hi - 1) * m + r];
-                    R c = cs[hi - 1], sv = sn[hi - 1];
+                    R c = c_[hi - 1], sv = s_[hi - 1];
                     for (int k = hi - 1; k >= lo; --k) {
                         const bool more = k > lo;
                         const R a0n = more ? Z[(size_t)(k - 1) * m + r] : R(0);
-                        const R cn = more ? cs[k - 1] : R(0), svn = more ? sn[k - 1] : R(0);
+                        const R cn = more ? c_[k - 1] : R(0), svn = more ? s_[k - 1] : R(0);
                         Z[(size_t)(k + 1) * m + r] = sv * a0 + c * a1;
                         a1 = c * a0 - sv * a1;
                         a0 = a0n;
@@ -537,22 +643,20 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
                     Z[(size_t)lo * m + r] = a1;
                 }
             }
-            __syncthreads();
-            if (done) break;
-        }
-        if (threadIdx.x == 0) {
-            // selection sort of the eigenvalues; the permutation is kept in cs
-            for (int i = 0; i < m; ++i) cs[i] = (R)i;
-            for (int i = 0; i < m - 1; ++i) {
-                int mi = i;
-                for (int j = i + 1; j < m; ++j) if (d[j] < d[mi]) mi = j;
-                R t = d[i]; d[i] = d[mi]; d[mi] = t;
-                t = cs[i]; cs[i] = cs[mi]; cs[mi] = t;
-            }
-            if (info) info[b] = s_fail;
+            if (s_done[buf]) break;  // (no sweep was recorded with it; uniform: written before the barrier,
+                                     // and next rewritten two sweeps later)
         }
         __syncthreads();
-        for (int j = threadIdx.x; j < m; j += blockDim.x) W[j] = (double)d[j];
+        // ascending order: the rank of each eigenvalue (ties by index); cs[rank] = its column of Z
+        for (int j = threadIdx.x; j < m; j += blockDim.x) {
+            const R dj = d[j];
+            int rank = 0;
+            for (int k = 0; k < m; ++k) rank += d[k] < dj || (d[k] == dj && k < j);
+            W[rank] = (double)dj;
+            cs[rank] = (R)j;
+        }
+        if (threadIdx.x == 0 && info) info[b] = s_fail;
+        __syncthreads();
         // the columns of Z are put in ascending order at the write-out (the back-transformation acts
         // on each column alone)
     }
@@ -597,7 +701,7 @@ template <class R>
 __global__ void __launch_bounds__(EIG_THREADS) k_bi_tridiag(int m, double *A, R *work) {
     extern __shared__ __align__(16) unsigned char smraw[];
     R *a = reinterpret_cast<R *>(smraw);
-    __shared__ R red[EIG_THREADS / 32];
+    __shared__ R red[64];
     R *d = work, *e = work + m, *e2 = work + 2 * m, *beta = work + 3 * m, *vv = work + 4 * m, *pp = work + 5 * m;
     for (int t = threadIdx.x; t < m * m; t += blockDim.x) a[t] = (R)A[t];
     __syncthreads();
