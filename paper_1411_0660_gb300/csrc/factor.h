@@ -16,7 +16,27 @@ struct SolveBufs {
     T *y, *yfw;          // permuted right-hand side / solution; forward result
     T *P;                // backward partial sums
     unsigned int *cnt;   // backward arrival counters (per solve descriptor and column chunk)
+    // FP64 fronts: G holds digits (solve_fx.cu), these the powers of two of its rows and columns
+    const int32_t *rex, *cex;
 };
+
+// Device bytes of the packed solve factor, and of the scratch its digits are made from (FP64 fronts).
+inline double solve_factor_bytes(const Plan &p, int prec) {
+    return prec == MBL_PREC_FP64 ? 4096.0 * (double)p.x_tiles + 4.0 * (double)(p.x_rows + p.x_cols) : 4.0 * (double)p.sg_elems;
+}
+inline double solve_factor_scratch(const Plan &p, int prec) { return prec == MBL_PREC_FP64 ? 8.0 * (double)p.max_step_g : 0.0; }
+
+// Steps of the FP64 level sequence (solve_fx.cu).  fx_pack_step: the digits of one solve step's G (FP64, from
+// its first panel's goff on).  fx_prepare: kernel attributes, before a launch or a capture.
+void fx_prepare();
+void fx_pack_step(const Plan &pl, const SolveStep &ss, const double *G, int32_t *cex, int32_t *rex, double *out,
+                  cudaStream_t st);
+void fx_forward(const Plan &pl, const SolveStep &ss, const SolveBufs<double> *jb, unsigned K, int p, LaunchTrace *tr,
+                cudaStream_t st);
+void fx_backward_level(const Plan &pl, int l, const SolveBufs<double> *jb, unsigned K, int p, LaunchTrace *tr,
+                       cudaStream_t st);
+void fx_backward_update(const Plan &pl, const BwdUpd &bu, const SolveBufs<double> *jb, unsigned K, int p,
+                        LaunchTrace *tr, cudaStream_t st);
 
 struct LeanArena;  // physical backing of the memory-lean fronts arena (factor.cu)
 
@@ -36,7 +56,11 @@ struct Factorization {
     int prec = MBL_PREC_FP32;
     double tiny = 0.0;
     DVec<char> arena, D, wscr, cmax, M, zwork, zsolved, ywork, yfw, pwork;
-    DVec<char> gpk;           // packed solve factor: every solve panel's G = [M; L21 M] (Plan::sg_elems)
+    DVec<char> gpk;           // packed solve factor: every solve panel's G = [M; L21 M] (Plan::sg_elems), or
+                              // its digits (FP64 fronts of the level sequence: fx)
+    bool fx = false;
+    DVec<char> gstep;         // fx: one solve step's G in FP64 while the factor is built
+    DVec<int32_t> rex, cex;   // fx: row and column scales
     DVec<int32_t> piv;
     DVec<unsigned int> scnt;  // per (solve panel, column chunk) arrival counters of the backward step
     DVec<int32_t> dfcnt;      // dataflow solve: per-front completion counters (4 ns) and two tickets

@@ -1,0 +1,120 @@
+// fixed_digits.cuh -- FP64 products on the FP16 tensor cores by exact integer digits.
+//
+// A block of FP64 numbers that are summed over together is written as 62-bit integers on one power-of-two
+// scale (its largest magnitude), each integer as eight balanced base-256 digits d_0 (leading) ... d_7 in
+// [-128, 127].  Digits are exact in FP16, and a sum of products of digits stays an integer below 2^24, exact
+// in the tensor core's FP32 accumulator (the error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012, with
+// integer slices).  The products of digit i of one factor and digit j of the other are kept for i + j <= 8
+// (43 of 64): what is left out is of the size of the splittings' own 2^-63 of a scale, so that a term loses
+// 2^-62 of the product of the two scales, where FP64 arithmetic loses 2^-53 of the term: terms as small as 2^-9
+// of the largest keep FP64's accuracy, and a sum's error stays that of its largest terms.  The digit sums A_l
+// (l = i + j) are put together in integers:
+//   sum x y = (hi 2^40 + lo) 2^48 on the scale 2^-124, hi = sum_{l<4} A_l 256^(3-l), lo = sum_{l>=4} A_l 256^(8-l),
+// so that the only other rounding is one at the end.
+//
+// Why: GB300 does two FP64 FMAs a clock and SM (1.2 TFLOP/s in all).  43 FP16 products of 16 x 8 x 16 a tile
+// replace 2048 of them.
+#pragma once
+
+#include <cstdint>
+
+namespace mbl {
+
+constexpr int FX_ND = 8;                 // digits
+constexpr int FX_NL = 9;                 // digit sums kept: i + j < FX_NL
+constexpr int FX_NOZERO = -(1 << 16);    // exponent of a zero
+constexpr int FX_BAD = 1 << 19;          // exponents from here on: an infinity or a NaN is among the numbers
+
+// biased exponent of v with an extra power of two e: |v| 2^e < 2^(result - 1022); FX_NOZERO for zero
+// (denormals count as zero: 2^-1022 is no size a sum here is accurate to)
+__device__ __forceinline__ int fx_exp(double v, int e) {
+    const int b = (__double2hiint(v) >> 20) & 0x7ff;
+    if (e >= FX_BAD / 2) return FX_BAD;
+    return b == 0 ? FX_NOZERO : (b == 0x7ff ? FX_BAD : b + e);
+}
+
+// rint(v 2^e 2^(62 - (E - 1022))) + the bias that makes its base-256 digits' bytes d + 128; E: the largest
+// fx_exp of the block
+__device__ __forceinline__ uint64_t fx_bytes(double v, int e, int E) {
+    const uint64_t u = (uint64_t)__double_as_longlong(v);
+    const int b = (int)(u >> 52) & 0x7ff;
+    uint64_t m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int sh = 9 - (E - (b + e));
+    if (b == 0 || b == 0x7ff || sh < -53) m = 0;
+    else if (sh >= 0) m <<= sh;
+    else m = (m + (1ull << (-sh - 1))) >> -sh;
+    return 0x8080808080808080ull + (v < 0.0 ? (uint64_t)0 - m : m);
+}
+
+// A block whose numbers span more than 2^FX_SPAN is taken in several passes: a number smaller than that share of
+// the scale keeps what its digits left out (and the others are done), so that every number counts with a
+// relative error below 2^-(63 - FX_SPAN) = 2^-43 whatever stands beside it.
+constexpr int FX_SPAN = 20;
+
+// fx_bytes, and v becomes what the next pass takes
+__device__ __forceinline__ uint64_t fx_take(double &v, int e, int E, bool again) {
+    const uint64_t y = fx_bytes(v, e, E);
+    if (again) {
+        const int b = fx_exp(v, e);
+        const int64_t x = (int64_t)(y - 0x8080808080808080ull);
+        v = b != FX_NOZERO && b < FX_BAD && E - b > FX_SPAN ? v - scalbn((double)x, E - 1084 - e) : 0.0;
+    }
+    return y;
+}
+
+// FP16 pair (digits of the bytes selected by sel's nibbles 0 and 2; 0x64 in the others makes 1024 + byte)
+__device__ __forceinline__ uint32_t fx_half2(uint32_t bytes, uint32_t sel) {
+    uint32_t h, r;
+    asm("prmt.b32 %0, %1, 0x64646464, %2;" : "=r"(h) : "r"(bytes), "r"(sel));
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));  // - (1024 + 128)
+    return r;
+}
+// digit j of x (low half) and y (high half)
+template <int J>
+__device__ __forceinline__ uint32_t fx_pair(uint64_t x, uint64_t y) {
+    constexpr int byte = FX_ND - 1 - J;
+    const uint32_t xs = (uint32_t)(x >> (32 * (byte / 4))), ys = (uint32_t)(y >> (32 * (byte / 4)));
+    uint32_t b, r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(b) : "r"(xs), "r"(ys), "n"((byte % 4) | 0x70 | (4 + byte % 4) << 8 | 0x7000));
+    b = (b & 0x00ff00ffu) | 0x64006400u;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(b), "r"(0x64806480u));
+    return r;
+}
+
+__device__ __forceinline__ void fx_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// exact integer of an accumulator
+__device__ __forceinline__ int fx_int(float a) { return __float2int_rn(a); }
+
+// hi and lo of one output from its digit sums acc[l][k]
+template <int N>
+__device__ __forceinline__ void fx_collect(const float (&acc)[FX_NL][N], int k, int64_t &hi, int64_t &lo) {
+    hi = ((int64_t)fx_int(acc[0][k]) << 24) + ((int64_t)fx_int(acc[1][k]) << 16) + ((int64_t)fx_int(acc[2][k]) << 8) +
+         fx_int(acc[3][k]);
+    lo = ((int64_t)fx_int(acc[4][k]) << 32) + ((int64_t)fx_int(acc[5][k]) << 24) + ((int64_t)fx_int(acc[6][k]) << 16) +
+         ((int64_t)fx_int(acc[7][k]) << 8) + fx_int(acc[8][k]);
+}
+
+// (hi 2^40 + lo) 2^48 2^(ea - 62) 2^(eb - 62), rounded once: ea, eb the scales' powers of two.  In integers
+// (|hi| < 2^60, |lo| < 2^60): the conversions would run on the FP64 pipe.
+__device__ __forceinline__ double fx_value(int64_t hi, int64_t lo, int ea, int eb) {
+    if (ea >= FX_BAD / 2 || eb >= FX_BAD / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    const int s = min(40, __clzll(hi < 0 ? -hi : hi) - 2);
+    const int64_t x = (hi << s) + (lo >> (40 - s));
+    if (x == 0) return 0.0;
+    uint64_t m = (uint64_t)(x < 0 ? -x : x);
+    const int z = __clzll((int64_t)m), e = 63 - z + 40 - s + 48 - 124 + ea + eb;
+    m <<= z;
+    m = (m >> 11) + (m >> 10 & 1);  // 53 bits (a carry out of them lands in the exponent)
+    const uint64_t sign = x < 0 ? 0x8000000000000000ull : 0ull;
+    if (e > -1022 && e < 1023) return __longlong_as_double((int64_t)(sign | (((uint64_t)(e + 1022) << 52) + m)));
+    const double v = scalbn((double)m, e - 52);
+    return x < 0 ? -v : v;
+}
+
+}  // namespace mbl

@@ -1313,8 +1313,8 @@ static std::vector<int> nearest_sorted(const std::vector<double> &th, double sig
 // solve factor and panel scratch against the device's total memory (less a margin for the rest of the
 // job) and the context budget.
 static bool fp64_fits_plan(const Plan &p, int arena_mode, const Ctx *ctx) {
-    const double need = arena_peak_bytes(p, MBL_PREC_FP64, arena_mode) + 8.0 * (double)p.sg_elems +
-                        12.0 * (double)p.n + 8.0 * (double)(p.m_elems + p.wscratch_elems);
+    const double need = arena_peak_bytes(p, MBL_PREC_FP64, arena_mode) + solve_factor_bytes(p, MBL_PREC_FP64) +
+                        solve_factor_scratch(p, MBL_PREC_FP64) + 12.0 * (double)p.n + 8.0 * (double)(p.m_elems + p.wscratch_elems);
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -1329,8 +1329,8 @@ static bool fp64_fits_plan(const Plan &p, int arena_mode, const Ctx *ctx) {
 // fz releases, and the context budget.
 static bool fp64_fits(const Factorization &fz, int arena_mode) {
     const Plan &p = *fz.plan;
-    const double need = arena_peak_bytes(p, MBL_PREC_FP64, arena_mode) + 8.0 * (double)p.sg_elems +
-                        12.0 * (double)p.n + 8.0 * (double)(p.m_elems + p.wscratch_elems);
+    const double need = arena_peak_bytes(p, MBL_PREC_FP64, arena_mode) + solve_factor_bytes(p, MBL_PREC_FP64) +
+                        solve_factor_scratch(p, MBL_PREC_FP64) + 12.0 * (double)p.n + 8.0 * (double)(p.m_elems + p.wscratch_elems);
     const double freed = 4.0 * (double)p.sg_elems + 8.0 * (double)p.n;
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {

@@ -35,14 +35,15 @@ size_t job_bytes(const Plan &p, int nev, int block, int prec) {
     const double ldv = 2.0 * nev + 3.0 * pb;
     const double held = 20.0 * n + 12.0 * (double)p.nnzA      // sector
                         + 8.0 * n * nev + 64.0 * nev;         // outputs
-    const double factor_keep = (double)p.sg_elems * es + n * (es + 4.0);  // packed solve factor, D, pivots
+    const double factor_keep = solve_factor_bytes(p, prec) + n * (es + 4.0);  // packed solve factor, D, pivots
     const double krylov = 8.0 * n * (3.0 * ldv + 2.0 * nev + 30.0 * pb)  // Krylov, Rayleigh-Ritz, refinement
                           + 2.0 * (double)p.zwork_elems * pb * es + 2.0 * n * pb * es  // solve work
                           + (double)std::max(p.max_sstep_nrbk, p.max_lvl_nrbk) * SUBS * RBB * pad * es;
     const double bounds = 8.0 * n * 480.0;  // extremal-bounds Lanczos basis
     const double factor = arena_peak_bytes(p, prec, ARENA_AUTO) + factor_keep +
-                          (double)std::max<int64_t>(p.wscratch_elems, 1) * 5.0 * es + (double)p.m_elems * es +
-                          krylov;  // W21 scratch and the four operand-piece arrays
+                          (double)std::max<int64_t>(p.wscratch_elems, 1) * (prec == MBL_PREC_FP64 ? 1.0 : 5.0) * es +
+                          (double)p.m_elems * es + solve_factor_scratch(p, prec) +
+                          krylov;  // W21 scratch and (FP32 fronts) the four operand-piece arrays
     const double solve = factor_keep + krylov;
     const double peak = held + std::max(bounds, std::max(factor, solve));
     return (size_t)(1.05 * peak) + ((size_t)128 << 20);

@@ -1,0 +1,885 @@
+// solve_fx.cu -- steps of the level-by-level triangular solves with FP64 fronts.
+//
+// The same steps as factor.cu's FP32 ones (z_panel <- M z_panel, z_below -= (L21 M) z_panel forward;
+// x_panel <- G^T [y_panel; -x_below] backward, G = [M; L21 M] packed per 256-column solve panel), with the
+// products of G and a p-wide block formed from integer digits on the FP16 tensor cores (fixed_digits.cuh).
+// In FP64 arithmetic these steps are bound by the two FP64 FMAs a clock and SM: a whole L = 16 job of 43
+// block applications took 244 ms that way and takes 215 ms this way; the unrefined solve's error against a
+// dense 64-bit solve is 0.8 to 0.95 of what it was (geometric means over L = 10 to 14, 24 cases each).
+//
+// Packed form of one panel's G (R x w): column c is scaled by 2^-cex[c] and row r by 2^-rex[r] (powers of
+// two that put every column's, then every row's largest magnitude in [1/2, 1)), the entry becomes eight
+// digits, and the digits lie in tiles of 32 rows x 16 columns, 4 KB each: eight planes (leading digit first)
+// of 32 lanes x 16 bytes, one A operand fragment a lane.  With lane = 4 g + t, word 2 h + s of the 16 bytes
+// holds rows 4 g + 2 s, + 1 of column 2 t + 8 h, then the same rows of column 2 t + 1 + 8 h.  That is the
+// fragment of G itself for rows (4 g + 2 s, 4 g + 2 s + 1) and, after one 8 x 8 transposition (movmatrix)
+// of each word's halves, the fragment of G^T: both sweeps read one copy, of FP64's size.  Tiles run over the
+// panel's columns first; rows and columns past the panel are zero.
+#include "factor.h"
+#include "fixed_digits.cuh"
+#include "solve_tile.cuh"
+
+namespace mbl {
+
+namespace {
+
+constexpr int FT_ROWS = 32, FT_COLS = 16;
+constexpr int FT_WORDS = FX_ND * 32 * 4;  // 32-bit words of a tile
+
+__device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+}
+
+// digit J of the eight numbers y (two k16 blocks: y[4 s .. 4 s + 3] are k = 2t, 2t+1, 2t+8, 2t+9 of block s)
+template <int J>
+__device__ __forceinline__ void fx_b(const uint64_t (&y)[8], int s, uint32_t &b0, uint32_t &b1) {
+    b0 = fx_pair<J>(y[4 * s], y[4 * s + 1]);
+    b1 = fx_pair<J>(y[4 * s + 2], y[4 * s + 3]);
+}
+__device__ __forceinline__ void fx_b_all(const uint64_t (&y)[8], int s, uint32_t (&b)[FX_ND][2]) {
+    fx_b<0>(y, s, b[0][0], b[0][1]);
+    fx_b<1>(y, s, b[1][0], b[1][1]);
+    fx_b<2>(y, s, b[2][0], b[2][1]);
+    fx_b<3>(y, s, b[3][0], b[3][1]);
+    fx_b<4>(y, s, b[4][0], b[4][1]);
+    fx_b<5>(y, s, b[5][0], b[5][1]);
+    fx_b<6>(y, s, b[6][0], b[6][1]);
+    fx_b<7>(y, s, b[7][0], b[7][1]);
+}
+
+// G z of one tile: acc[m][l] += digits (rows (4 g + 2 m, + 1)) x b; word(i) = the lane's 16 bytes of plane i
+template <class W>
+__device__ __forceinline__ void tile_forward(W &&word, const uint32_t (&b)[FX_ND][2], float (&acc)[2][FX_NL][4]) {
+#pragma unroll
+    for (int i = 0; i < FX_ND; ++i) {
+        const uint4 q = word(i);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const uint32_t w0 = m ? q.y : q.x, w1 = m ? q.w : q.z;
+            const uint32_t a[4] = {fx_half2(w0, 0x4240), fx_half2(w0, 0x4341), fx_half2(w1, 0x4240), fx_half2(w1, 0x4341)};
+#pragma unroll
+            for (int j = 0; j < FX_ND && i + j < FX_NL; ++j) fx_mma(acc[m][i + j], a, b[j][0], b[j][1]);
+        }
+    }
+}
+
+// G^T v of one tile (32 rows of v, in b[s]: rows 8 t + 2 s, + 1, + 4, + 5): acc[l] += ..., columns (g, g + 8)
+template <class W>
+__device__ __forceinline__ void tile_backward(W &&word, const uint32_t (&b)[2][FX_ND][2], float (&acc)[FX_NL][4]) {
+#pragma unroll
+    for (int i = 0; i < FX_ND; ++i) {
+        const uint4 q = word(i);
+        const uint32_t tr[4] = {movmatrix(q.x), movmatrix(q.y), movmatrix(q.z), movmatrix(q.w)};
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const uint32_t a[4] = {fx_half2(tr[s], 0x4140), fx_half2(tr[2 + s], 0x4140), fx_half2(tr[s], 0x4342),
+                                   fx_half2(tr[2 + s], 0x4342)};
+#pragma unroll
+            for (int j = 0; j < FX_ND && i + j < FX_NL; ++j) fx_mma(acc[i + j], a, b[s][j][0], b[s][j][1]);
+        }
+    }
+}
+
+// largest and smallest value of the four lanes t of a group
+__device__ __forceinline__ int max_over_t(int x) {
+    x = max(x, __shfl_xor_sync(0xffffffffu, x, 1));
+    return max(x, __shfl_xor_sync(0xffffffffu, x, 2));
+}
+__device__ __forceinline__ int min_over_t(int x) {
+    x = min(x, __shfl_xor_sync(0xffffffffu, x, 1));
+    return min(x, __shfl_xor_sync(0xffffffffu, x, 2));
+}
+// the smallest exponent leaves zeros out
+__device__ __forceinline__ int min_exp(int m, int e) { return e == FX_NOZERO ? m : min(m, e); }
+constexpr int FX_NOMIN = 1 << 20;
+
+__device__ __forceinline__ uint4 ld_tile(const double *G, int64_t tile, int plane, int lane) {
+    return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint32_t *>(G) + tile * FT_WORDS) + plane * 32 +
+                 lane);
+}
+
+// Powers of two of the columns of the step's panels: |column c| < 2^cex[c].  A warp per column.  G: the
+// step's operators in FP64 (column-major, leading dimension sg_ld), from `base` of the packed order on.
+__global__ void __launch_bounds__(256) k_fx_colexp(const SolveDesc *sdescs, const double *G, int64_t base, int32_t *cex) {
+    const SolveDesc d = sdescs[blockIdx.x];
+    const int lane = threadIdx.x & 31, c = blockIdx.y * 8 + (threadIdx.x >> 5), R = d.w + d.m2;
+    if (c >= (d.w + FT_COLS - 1) / FT_COLS * FT_COLS) return;
+    const double *g = G + (d.goff - base) + (int64_t)c * sg_ld(R);
+    int e = FX_NOZERO;
+    if (c < d.w)
+        for (int r = lane; r < R; r += 32) e = max(e, fx_exp(g[r], 0));
+    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if (lane == 0) cex[d.xcol + c] = e <= FX_NOZERO || e >= FX_BAD ? 0 : e - 1022;
+}
+
+// Row scales and digits of one 32-row block of a panel.
+__global__ void __launch_bounds__(256) k_fx_pack(const SolveDesc *sdescs, const int32_t *blk_desc, const double *G,
+                                                 int64_t base, const int32_t *cex, int32_t *rex, double *out) {
+    __shared__ int wmax[8][FT_ROWS], rmax[FT_ROWS];
+    const SolveDesc d = sdescs[blk_desc[blockIdx.x]];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, w = d.w, R = w + d.m2;
+    const int rb = (int)(blockIdx.x - d.off), r0 = rb * FT_ROWS, ncb = (w + FT_COLS - 1) / FT_COLS;
+    const int64_t ld = sg_ld(R);
+    const double *g = G + (d.goff - base) + r0;
+    int e = FX_NOZERO;
+    if (r0 + lane < R)
+        for (int c = wp; c < w; c += 8) e = max(e, fx_exp(g[(int64_t)c * ld + lane], -cex[d.xcol + c]));
+    wmax[wp][lane] = e;
+    __syncthreads();
+    if (wp == 0) {
+#pragma unroll
+        for (int i = 1; i < 8; ++i) e = max(e, wmax[i][lane]);
+        rmax[lane] = e;
+        rex[d.xrow + r0 + lane] = e >= FX_BAD ? FX_BAD : (e <= FX_NOZERO ? 0 : e - 1022);
+    }
+    __syncthreads();
+    const int gl = lane >> 2, t = lane & 3;
+    int E[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) E[i] = rmax[4 * gl + i];
+    for (int cb = wp; cb < ncb; cb += 8) {
+        uint64_t y[4][4];  // [column 2t, 2t+1, 2t+8, 2t+9][row 4g ..]
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = cb * FT_COLS + 2 * t + (k & 1) + 8 * (k >> 1);
+            const int ce = c < w ? -cex[d.xcol + c] : 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = 4 * gl + i;
+                y[k][i] = fx_bytes(c < w && r0 + r < R ? g[(int64_t)c * ld + r] : 0.0, ce, E[i]);
+            }
+        }
+        uint4 *o = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(out) +
+                                             (d.xoff + (int64_t)rb * ncb + cb) * FT_WORDS) + lane;
+#pragma unroll
+        for (int i = 0; i < FX_ND; ++i) {
+            const int sh = 8 * (FX_ND - 1 - i);
+            uint32_t wd[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+                    wd[2 * h + s] = (uint32_t)(y[2 * h][2 * s] >> sh & 255) | (uint32_t)(y[2 * h][2 * s + 1] >> sh & 255) << 8 |
+                                    (uint32_t)(y[2 * h + 1][2 * s] >> sh & 255) << 16 |
+                                    (uint32_t)(y[2 * h + 1][2 * s + 1] >> sh & 255) << 24;
+            o[i * 32] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+        }
+    }
+}
+
+// ---- forward ----------------------------------------------------------------------------------------
+
+// shared memory of the wide forward step: the row block's tiles, and the warps' partial sums (hi, lo)
+constexpr size_t FWD_TILE = (size_t)(SPW / FT_COLS) * FT_WORDS * 4;
+constexpr size_t FWD_SMEM = FWD_TILE + (size_t)8 * FT_ROWS * 8 * 16;
+
+// Row block (32 rows) of a panel with z = Z[panel]: warp i takes columns [32 i, 32 i + 32).  The tiles are
+// copied before the wait on the previous step; the warps agree on one scale of z per right-hand side, so
+// that their digit sums add up as integers.
+__global__ void __launch_bounds__(256, 2)
+    k_fx_fwd_step(const SolveDesc *sdescs, const int32_t *blk_desc, int nrb, int K, const int64_t *zo,
+                  const int32_t *sn_start, const SolveBufs<double> *jb, int p, LaunchTrace *tr) {
+    TraceScope trace_scope(tr);
+    extern __shared__ __align__(16) unsigned char smraw[];
+    uint4 *tiles = reinterpret_cast<uint4 *>(smraw);
+    int64_t *red = reinterpret_cast<int64_t *>(smraw + FWD_TILE);  // [warp][hi, lo][q][row]
+    __shared__ int smax[8][8], smin[8][8];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int nit = nrb * K;
+    bool waited = false;
+    for (int it = blockIdx.x; it < nit; it += gridDim.x) {
+        const int job = it / nrb, b = it - job * nrb;
+        const SolveBufs<double> J = jb[job];
+        const SolveDesc d = sdescs[blk_desc[b]];
+        const int s = d.front, k0 = d.k0, w = d.w, R = w + d.m2, ncb = (w + FT_COLS - 1) / FT_COLS;
+        const int rb = b - (int)d.off, r0 = rb * FT_ROWS, nr = min(FT_ROWS, R - r0), nw = (w + 31) / 32;
+        const int64_t zb = zo[s] + k0;
+        {
+            const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint32_t *>(J.G) +
+                                                               (d.xoff + (int64_t)rb * ncb) * FT_WORDS);
+            for (int u = threadIdx.x; u < ncb * (FT_WORDS / 4); u += 256) cp_async16(tiles + u, src + u);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+        const int oi = threadIdx.x & 31, oq = threadIdx.x >> 5, rr = r0 + oi;  // this thread's output
+        const int re = J.rex[d.xrow + rr];
+        const double dg = oi < nr && rr < w ? J.D[(int64_t)sn_start[s] + k0 + rr] : 1.0;
+        int ce[8];  // the column scales of this lane's eight entries of z
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int c = 32 * wp + 16 * (k >> 2) + 2 * t + (k & 1) + 8 * ((k >> 1) & 1);
+            ce[k] = c < w ? J.cex[d.xcol + c] : 0;
+        }
+        if (!waited) {
+            pdl_wait();
+            pdl_trigger();
+            waited = true;
+        }
+        for (int q0 = 0; q0 < p; q0 += 8) {
+            const int q = q0 + g;
+            double z[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int c = 32 * wp + 16 * (k >> 2) + 2 * t + (k & 1) + 8 * ((k >> 1) & 1);
+                z[k] = c < w && q < p ? J.Z[(zb + c) * p + q] : 0.0;
+            }
+            const double zold = oi < nr && q0 + oq < p && rr >= w ? J.Z[(zb + rr) * p + q0 + oq] : 0.0;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            double v = 0.0;
+            for (bool again = true; again;) {  // one pass unless z spans more than 2^FX_SPAN
+                int em = FX_NOZERO, el = FX_NOMIN;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int e = fx_exp(z[k], ce[k]);
+                    em = max(em, e);
+                    el = min_exp(el, e);
+                }
+                em = max_over_t(em);
+                el = min_over_t(el);
+                if (t == 0) {
+                    smax[wp][g] = em;
+                    smin[wp][g] = el;
+                }
+                __syncthreads();
+                int E = smax[0][g], Eo = smax[0][oq], El = smin[0][g];
+#pragma unroll
+                for (int i = 1; i < 8; ++i) {
+                    E = max(E, smax[i][g]);
+                    El = min(El, smin[i][g]);
+                    Eo = max(Eo, smax[i][oq]);
+                }
+                // (every warp holds all eight right-hand sides: the same answer in each)
+                again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+                if (wp < nw) {
+                    uint64_t y[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) y[k] = fx_take(z[k], ce[k], E, again);
+                    float acc[2][FX_NL][4];
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+#pragma unroll
+                        for (int l = 0; l < FX_NL; ++l)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) acc[m][l][k] = 0.f;
+#pragma unroll
+                    for (int kb = 0; kb < 2; ++kb) {
+                        if (32 * wp + 16 * kb >= w) break;
+                        uint32_t bq[FX_ND][2];
+                        fx_b_all(y, kb, bq);
+                        const uint4 *tl = tiles + (size_t)(2 * wp + kb) * (FT_WORDS / 4) + lane;
+                        tile_forward([&](int i) { return tl[i * 32]; }, bq, acc);
+                    }
+                    int64_t *rw = red + (size_t)wp * 512;
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            int64_t hi, lo;
+                            fx_collect(acc[m], k, hi, lo);
+                            const int row = 4 * g + 2 * m + (k >> 1), qq = 2 * t + (k & 1);
+                            rw[qq * 32 + row] = hi;
+                            rw[256 + qq * 32 + row] = lo;
+                        }
+                }
+                __syncthreads();
+                {
+                    int64_t hi = 0, lo = 0;
+                    for (int i = 0; i < nw; ++i) {
+                        hi += red[(size_t)i * 512 + oq * 32 + oi];
+                        lo += red[(size_t)i * 512 + 256 + oq * 32 + oi];
+                    }
+                    v += fx_value(hi, lo, re, Eo - 1022);
+                }
+                __syncthreads();  // red, smax and smin (and, in the end, the tiles) are used again
+            }
+            if (oi < nr && q0 + oq < p) {
+                if (rr < w) {
+                    // a panel row is final here: also its diagonal-scaled value for the backward sweep
+                    const int64_t gr = (int64_t)sn_start[s] + k0 + rr;
+                    J.Zs[(zb + rr) * p + q0 + oq] = v;
+                    J.yfw[gr * p + q0 + oq] = v / dg;
+                } else {
+                    J.Z[(zb + rr) * p + q0 + oq] = zold - v;
+                }
+            }
+        }
+    }
+    if (!waited) pdl_wait();
+}
+
+// Narrow forward step (every panel of the step at most 16 CB columns wide): a warp per 32-row block, its
+// tiles in registers before the wait on the previous step.
+template <int CB>
+__global__ void __launch_bounds__(256) k_fx_fwd_narrow(const SolveDesc *sdescs, const int32_t *blk_desc, int nblk,
+                                                       const int64_t *zo, const int32_t *sn_start,
+                                                       const SolveBufs<double> *jb, int p, LaunchTrace *tr) {
+    TraceScope trace_scope(tr);
+    const SolveBufs<double> J = jb[blockIdx.z];
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, item = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (item >= nblk) {
+        pdl_wait();
+        return;
+    }
+    const SolveDesc d = sdescs[blk_desc[item]];
+    const int s = d.front, k0 = d.k0, w = d.w, R = w + d.m2, ncb = (w + FT_COLS - 1) / FT_COLS;
+    const int rb = (int)(item - d.off), r0 = rb * FT_ROWS;
+    const int64_t zb = zo[s] + k0, g0 = (int64_t)sn_start[s] + k0;
+    uint4 G[CB][FX_ND];
+#pragma unroll
+    for (int kb = 0; kb < CB; ++kb)
+#pragma unroll
+        for (int i = 0; i < FX_ND; ++i)
+            G[kb][i] = kb < ncb ? ld_tile(J.G, d.xoff + (int64_t)rb * ncb + kb, i, lane)
+                                : make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+    int ce[8], re[4];
+    double dg[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int c = 16 * (k >> 2) + 2 * t + (k & 1) + 8 * ((k >> 1) & 1);
+        ce[k] = c < w ? J.cex[d.xcol + c] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int rr = r0 + 4 * g + i;
+        re[i] = J.rex[d.xrow + rr];
+        dg[i] = rr < w ? J.D[g0 + rr] : 1.0;
+    }
+    pdl_wait();
+    pdl_trigger();
+    for (int q0 = 0; q0 < p; q0 += 8) {
+        double z[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int c = 16 * (k >> 2) + 2 * t + (k & 1) + 8 * ((k >> 1) & 1);
+            z[k] = k < 4 * CB && c < w && q0 + g < p ? J.Z[(zb + c) * p + q0 + g] : 0.0;
+        }
+        double zold[4][2];  // rows 4 g + i, right-hand sides 2 t, 2 t + 1
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int rr = r0 + 4 * g + i, q = q0 + 2 * t + u;
+                zold[i][u] = rr >= w && rr < R && q < p ? J.Z[(zb + rr) * p + q] : 0.0;
+            }
+        double sum[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+        for (bool again = true; again;) {  // one pass unless z spans more than 2^FX_SPAN
+            int E = FX_NOZERO, El = FX_NOMIN;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int e = fx_exp(z[k], ce[k]);
+                E = max(E, e);
+                El = min_exp(El, e);
+            }
+            E = max_over_t(E);
+            El = min_over_t(El);
+            again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+            uint64_t y[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) y[k] = fx_take(z[k], ce[k], E, again);
+            float acc[2][FX_NL][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int l = 0; l < FX_NL; ++l)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[m][l][k] = 0.f;
+#pragma unroll
+            for (int kb = 0; kb < CB; ++kb) {
+                if (kb >= ncb) break;
+                uint32_t bq[FX_ND][2];
+                fx_b_all(y, kb, bq);
+                tile_forward([&](int i) { return G[kb][i]; }, bq, acc);
+            }
+            // the scale of right-hand side 2 t + u is with the lanes of group 2 t + u
+            const int e0 = __shfl_sync(0xffffffffu, E, 4 * (2 * t)), e1 = __shfl_sync(0xffffffffu, E, 4 * (2 * t + 1));
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    int64_t hi, lo;
+                    fx_collect(acc[m], k, hi, lo);
+                    sum[m][k] += fx_value(hi, lo, re[2 * m + (k >> 1)], ((k & 1) ? e1 : e0) - 1022);
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = 2 * m + (k >> 1), rr = r0 + 4 * g + i, q = q0 + 2 * t + (k & 1);
+                if (rr >= R || q >= p) continue;
+                const double v = sum[m][k];
+                if (rr < w) {
+                    J.Zs[(zb + rr) * p + q] = v;
+                    J.yfw[(g0 + rr) * p + q] = v / dg[i];
+                } else {
+                    J.Z[(zb + rr) * p + q] = zold[i][k & 1] - v;
+                }
+            }
+    }
+}
+
+// ---- backward ---------------------------------------------------------------------------------------
+
+constexpr int BW_RB = RBK / FT_ROWS + 1;  // most row blocks of one tile (the first may start inside a block)
+constexpr size_t BWD_TILE = (size_t)BW_RB * (RBB / FT_COLS) * FT_WORDS * 4;
+constexpr size_t BWD_SMEM = BWD_TILE + (size_t)8 * 2 * 8 * RBB * 8;  // and the warps' sums [warp][hi, lo][q][column]
+
+// Copies row blocks [rb0, rb0 + nrb) of the 64 columns from 16 cb0 on.
+__device__ __forceinline__ void bwd_issue(uint4 *tiles, const double *G, const SolveDesc &d, int rb0, int nrb, int cb0) {
+    const int ncb = (d.w + FT_COLS - 1) / FT_COLS, nc = min(RBB / FT_COLS, ncb - cb0), per = nc * (FT_WORDS / 4);
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(G) + (d.xoff + (int64_t)rb0 * ncb + cb0) * FT_WORDS;
+    for (int u = threadIdx.x; u < nrb * per; u += 256) {
+        const int r = u / per, v = u - r * per;
+        cp_async16(tiles + (size_t)r * (RBB / FT_COLS) * (FT_WORDS / 4) + v,
+                   reinterpret_cast<const uint4 *>(src + (int64_t)r * ncb * FT_WORDS) + v);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Digit sums of the tiles' columns for right-hand sides q0 .. q0 + 7, added over the CTA: thread o returns
+// the products of outputs o and o + 256 (column c = o % RBB, q = q0 + o / RBB).  vf(r, q): entry of v at row r
+// (relative to the first row block), zero outside.  rexp: the rows' scales, from the first row block on.
+template <class VF>
+__device__ __forceinline__ void bwd_products(uint4 *tiles, const SolveDesc &d, int nrb, int cb0, const int32_t *rexp,
+                                             const int32_t *cexp, int q0, int p, VF &&vf, double out[2]) {
+    __shared__ int smax[8][8], smin[8][8];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int nc = min(RBB / FT_COLS, (d.w + FT_COLS - 1) / FT_COLS - cb0);
+    // (at most two row blocks a warp: wp and, of nine, the last one for warp 0)
+    double v[2][8];
+    int re[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int rbk = wp + 8 * h, r = 32 * rbk + 8 * t + 2 * (k >> 2) + (k & 1) + 4 * ((k >> 1) & 1);
+            const bool in = rbk < nrb && q0 + g < p;
+            v[h][k] = in ? vf(r, q0 + g) : 0.0;
+            re[h][k] = in ? rexp[r] : 0;
+        }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    out[0] = out[1] = 0.0;
+    for (bool again = true; again;) {  // one pass unless v spans more than 2^FX_SPAN
+        int em = FX_NOZERO, el = FX_NOMIN;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int e = fx_exp(v[h][k], re[h][k]);
+                em = max(em, e);
+                el = min_exp(el, e);
+            }
+        em = max_over_t(em);
+        el = min_over_t(el);
+        if (t == 0) {
+            smax[wp][g] = em;
+            smin[wp][g] = el;
+        }
+        __syncthreads();
+        int E = smax[0][g], El = smin[0][g];
+#pragma unroll
+        for (int i = 1; i < 8; ++i) {
+            E = max(E, smax[i][g]);
+            El = min(El, smin[i][g]);
+        }
+        // (every warp holds all eight right-hand sides: the same answer in each)
+        again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+        int64_t hi[RBB / FT_COLS][4], lo[RBB / FT_COLS][4];
+#pragma unroll
+        for (int cb = 0; cb < RBB / FT_COLS; ++cb)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) hi[cb][k] = lo[cb][k] = 0;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int rbk = wp + 8 * h;
+            if (rbk >= nrb) break;
+            uint32_t b[2][FX_ND][2];
+            {
+                uint64_t y[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    double vk = h ? v[1][k] : v[0][k];
+                    y[k] = fx_take(vk, h ? re[1][k] : re[0][k], E, again);
+                    if (h) v[1][k] = vk;
+                    else v[0][k] = vk;
+                }
+                fx_b_all(y, 0, b[0]);
+                fx_b_all(y, 1, b[1]);
+            }
+#pragma unroll
+            for (int cb = 0; cb < RBB / FT_COLS; ++cb) {
+                if (cb >= nc) break;
+                float acc[FX_NL][4];
+#pragma unroll
+                for (int l = 0; l < FX_NL; ++l)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[l][k] = 0.f;
+                const uint4 *tl = tiles + (size_t)(rbk * (RBB / FT_COLS) + cb) * (FT_WORDS / 4) + lane;
+                tile_backward([&](int i) { return tl[i * 32]; }, b, acc);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    int64_t a, c;
+                    fx_collect(acc, k, a, c);
+                    hi[cb][k] += a;
+                    lo[cb][k] += c;
+                }
+            }
+        }
+        int64_t *red = reinterpret_cast<int64_t *>(tiles) + BWD_TILE / 8;
+        const int nwp = min(8, nrb);
+        if (wp < nwp) {
+            int64_t *rw = red + (size_t)wp * 16 * RBB;
+#pragma unroll
+            for (int cb = 0; cb < RBB / FT_COLS; ++cb)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int c = 16 * cb + g + 8 * (k >> 1), q = 2 * t + (k & 1);
+                    rw[q * RBB + c] = hi[cb][k];
+                    rw[8 * RBB + q * RBB + c] = lo[cb][k];
+                }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = threadIdx.x + 256 * h, c = o % RBB, q = o / RBB;
+            int64_t a = 0, b = 0;
+            for (int i = 0; i < nwp; ++i) {
+                a += red[(size_t)i * 16 * RBB + q * RBB + c];
+                b += red[(size_t)i * 16 * RBB + 8 * RBB + q * RBB + c];
+            }
+            int Eo = smax[0][q];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) Eo = max(Eo, smax[i][q]);
+            if (16 * cb0 + c < d.w) out[h] += fx_value(a, b, cexp[16 * cb0 + c], Eo - 1022);
+        }
+        __syncthreads();  // red, smax and smin are used again
+    }
+}
+
+// Start of the backward sweep of one level: see k_bwd_step in factor.cu (same blocks, same partial sums).
+// Block b >= 1 of a panel takes an even share of the 32-row blocks from the contribution block's first row on
+// (rows of the front's later panels in the first of them meet a zero v).
+template <int PB>
+__global__ void __launch_bounds__(256) k_fx_bwd_step(const SolveDesc *sdescs, const int32_t *blk_desc,
+                                                     const int64_t *zo, const int32_t *nc, const int32_t *sn_start,
+                                                     const int64_t *rows_off, const int32_t *rows,
+                                                     const SolveBufs<double> *jb, int64_t cnt_off, int p,
+                                                     LaunchTrace *tr) {
+    TraceScope trace_scope(tr);
+    extern __shared__ __align__(16) unsigned char smraw[];
+    uint4 *tiles = reinterpret_cast<uint4 *>(smraw);
+    __shared__ int s_last;
+    __shared__ const double *vrow[BW_RB * FT_ROWS];  // row of v (null: zero)
+    __shared__ double vsgn[BW_RB * FT_ROWS];
+    const SolveBufs<double> J = jb[blockIdx.z];
+    unsigned int *cnt = J.cnt + cnt_off;
+    const int di = blk_desc[blockIdx.x];
+    const SolveDesc d = sdescs[di];
+    const int cc = blockIdx.y * RBB;
+    if (cc >= d.w) {
+        pdl_wait();
+        return;
+    }
+    const int s = d.front, k0 = d.k0, w = d.w, ncs = nc[s], R = w + d.m2, cb0 = ncs - k0;
+    const int b = (int)(blockIdx.x - d.offk_l), nb = bwd_start_blocks(R, cb0);
+    int rb0 = 0, nrb = (w + FT_ROWS - 1) / FT_ROWS;
+    if (b > 0) {
+        const int f0 = cb0 / FT_ROWS, n32 = (R + FT_ROWS - 1) / FT_ROWS - f0, per = (n32 + nb - 2) / (nb - 1);
+        rb0 = f0 + (b - 1) * per;
+        nrb = max(0, min(per, n32 - (b - 1) * per));
+    }
+    const int wc = min(RBB, w - cc);
+    const int64_t zb = zo[s] + k0;
+    if (nrb > 0) bwd_issue(tiles, J.G, d, rb0, nrb, cc / FT_COLS);
+    for (int i = threadIdx.x; i < BW_RB * FT_ROWS; i += 256) {
+        const int rr = rb0 * FT_ROWS + i;
+        const double *sp = nullptr;
+        if (i < nrb * FT_ROWS) {
+            if (b == 0) sp = rr < w ? J.yfw + ((int64_t)sn_start[s] + k0 + rr) * p : nullptr;
+            else if (rr >= cb0 && rr < R) sp = J.y + (int64_t)rows[rows_off[s] + k0 + rr] * p;
+        }
+        vrow[i] = sp;
+        vsgn[i] = b == 0 ? 1.0 : -1.0;
+    }
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    const int64_t tile = (int64_t)RBB * PB;
+    double *out = J.P + ((d.offk_l + b) * SUBS + blockIdx.y) * tile;
+    double *zsp = J.Zs + (zb + cc) * p;
+    double *xp = k0 + w >= ncs ? J.y + ((int64_t)sn_start[s] + k0 + cc) * p : nullptr;
+    for (int q0 = 0; q0 < PB; q0 += 8) {
+        double o2[2];
+        bwd_products(tiles, d, nrb, cc / FT_COLS, J.rex + d.xrow + rb0 * FT_ROWS, J.cex + d.xcol, q0, p,
+                     [&](int r, int q) { return vrow[r] ? vsgn[r] * __ldcg(vrow[r] + q) : 0.0; }, o2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
+            if (nb == 1) {
+                if (c < wc && q < p) {
+                    zsp[c * p + q] = o2[h];
+                    if (xp) xp[c * p + q] = o2[h];
+                }
+            } else {
+                out[q * RBB + c] = o2[h];
+            }
+        }
+    }
+    if (nb == 1) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned int prev = atomicAdd(&cnt[(size_t)di * SUBS + blockIdx.y], 1u);
+        s_last = prev == (unsigned int)(nb - 1);
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    bwd_finish<double, PB>(J.P + (d.offk_l * SUBS + blockIdx.y) * tile, (int64_t)SUBS * tile, nb, wc, p, zsp, xp,
+                           reinterpret_cast<double *>(smraw));
+    if (threadIdx.x == 0) cnt[(size_t)di * SUBS + blockIdx.y] = 0u;
+}
+
+// Backward update: see k_bwd_update in factor.cu.
+__global__ void __launch_bounds__(256) k_fx_bwd_update(const SolveDesc *sdescs, const int32_t *items, const int64_t *zo,
+                                                       const int32_t *sn_start, const SolveBufs<double> *jb, int p,
+                                                       LaunchTrace *tr) {
+    static_assert(SPW % FT_ROWS == 0, "later panels start on a row block");
+    TraceScope trace_scope(tr);
+    extern __shared__ __align__(16) unsigned char smraw[];
+    uint4 *tiles = reinterpret_cast<uint4 *>(smraw);
+    const SolveBufs<double> J = jb[blockIdx.z];
+    const SolveDesc di = sdescs[items[2 * blockIdx.x]], dj = sdescs[items[2 * blockIdx.x + 1]];
+    const int cc = blockIdx.y * RBB;
+    if (cc >= di.w) {
+        pdl_wait();
+        return;
+    }
+    const int s = di.front, wc = min(RBB, di.w - cc), wj = dj.w, rb0 = (dj.k0 - di.k0) / FT_ROWS;
+    const int nrb = (wj + FT_ROWS - 1) / FT_ROWS;
+    bwd_issue(tiles, J.G, di, rb0, nrb, cc / FT_COLS);
+    const int64_t zi = zo[s] + di.k0 + cc, zj = zo[s] + dj.k0;
+    const bool fin = dj.k0 == di.k0 + di.w;
+    pdl_wait();
+    pdl_trigger();
+    double *xp = J.y + ((int64_t)sn_start[s] + di.k0 + cc) * p;
+    for (int q0 = 0; q0 < p; q0 += 8) {
+        double old[2], o2[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
+            old[h] = c < wc && q < p ? J.Zs[(zi + c) * p + q] : 0.0;
+        }
+        bwd_products(tiles, di, nrb, cc / FT_COLS, J.rex + di.xrow + rb0 * FT_ROWS, J.cex + di.xcol, q0, p,
+                     [&](int r, int q) { return r < wj ? J.Zs[(zj + r) * p + q] : 0.0; }, o2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
+            if (c < wc && q < p) {
+                const double v = old[h] - o2[h];
+                J.Zs[(zi + c) * p + q] = v;
+                if (fin) xp[c * p + q] = v;
+            }
+        }
+    }
+}
+
+// Backward narrow step (panels at most 16 CB columns wide): NW warps share a panel, each taking 32-row blocks
+// with its own scale of v; their results meet in FP64 in a fixed order.
+template <int CB, int NW>
+__global__ void __launch_bounds__(256) k_fx_bwd_narrow(const SolveDesc *sdescs, int nd, const int64_t *zo,
+                                                       const int32_t *nc, const int32_t *sn_start,
+                                                       const int64_t *rows_off, const int32_t *rows,
+                                                       const SolveBufs<double> *jb, int p, LaunchTrace *tr) {
+    TraceScope trace_scope(tr);
+    __shared__ double red[8][8][16 * CB];  // [warp][q][column]
+    const SolveBufs<double> J = jb[blockIdx.z];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, wi = wp % NW, g = lane >> 2, t = lane & 3;
+    const int di = blockIdx.x * (8 / NW) + wp / NW;
+    const bool live = di < nd;  // the panel's warps are live together; all of them reach the barriers
+    const SolveDesc d = sdescs[live ? di : nd - 1];
+    const int s = d.front, k0 = d.k0, w = d.w, R = w + d.m2, ncs = nc[s], ncb = (w + FT_COLS - 1) / FT_COLS;
+    const int nrb = live ? (R + FT_ROWS - 1) / FT_ROWS : 0;
+    const int64_t zb = zo[s] + k0, g0 = (int64_t)sn_start[s] + k0;
+    const int32_t *rw = rows + rows_off[s] + k0;
+    uint4 G[CB][FX_ND];
+    int rowx[8], re[8];
+    auto load_block = [&](int rb) {
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int i = 0; i < FX_ND; ++i)
+                G[cb][i] = cb < ncb ? ld_tile(J.G, d.xoff + (int64_t)rb * ncb + cb, i, lane)
+                                    : make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int r = 32 * rb + 8 * t + 2 * (k >> 2) + (k & 1) + 4 * ((k >> 1) & 1);
+            rowx[k] = r < R && k0 + r >= ncs ? rw[r] : 0;
+            re[k] = J.rex[d.xrow + r];
+        }
+    };
+    int ce[CB][2];
+#pragma unroll
+    for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) ce[cb][u] = cb < ncb ? J.cex[d.xcol + 16 * cb + g + 8 * u] : 0;
+    if (wi < nrb) load_block(wi);
+    pdl_wait();
+    pdl_trigger();
+    for (int q0 = 0; q0 < p; q0 += 8) {
+        double sum[CB][4];
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sum[cb][k] = 0.0;
+        for (int rb = wi; rb < nrb; rb += NW) {
+            if (rb != wi || (q0 > 0 && nrb > NW)) load_block(rb);
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int r = 32 * rb + 8 * t + 2 * (k >> 2) + (k & 1) + 4 * ((k >> 1) & 1);
+                v[k] = 0.0;
+                if (r < R && q0 + g < p)
+                    v[k] = r < w ? J.yfw[(g0 + r) * p + q0 + g]
+                                 : -(k0 + r < ncs ? J.Zs[(zb + r) * p + q0 + g] : J.y[(int64_t)rowx[k] * p + q0 + g]);
+            }
+            for (bool again = true; again;) {  // one pass unless v spans more than 2^FX_SPAN
+                int E = FX_NOZERO, El = FX_NOMIN;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int e = fx_exp(v[k], re[k]);
+                    E = max(E, e);
+                    El = min_exp(El, e);
+                }
+                E = max_over_t(E);
+                El = min_over_t(El);
+                again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+                uint32_t b[2][FX_ND][2];
+                {
+                    uint64_t y[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) y[k] = fx_take(v[k], re[k], E, again);
+                    fx_b_all(y, 0, b[0]);
+                    fx_b_all(y, 1, b[1]);
+                }
+                const int e0 = __shfl_sync(0xffffffffu, E, 4 * (2 * t)), e1 = __shfl_sync(0xffffffffu, E, 4 * (2 * t + 1));
+#pragma unroll
+                for (int cb = 0; cb < CB; ++cb) {
+                    if (cb >= ncb) break;
+                    float acc[FX_NL][4];
+#pragma unroll
+                    for (int l = 0; l < FX_NL; ++l)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) acc[l][k] = 0.f;
+                    tile_backward([&](int i) { return G[cb][i]; }, b, acc);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        int64_t hi, lo;
+                        fx_collect(acc, k, hi, lo);
+                        sum[cb][k] += fx_value(hi, lo, ce[cb][k >> 1], ((k & 1) ? e1 : e0) - 1022);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) red[wp][2 * t + (k & 1)][16 * cb + g + 8 * (k >> 1)] = sum[cb][k];
+        __syncthreads();
+        for (int o = wi * 32 + lane; o < 8 * 16 * CB; o += 32 * NW) {
+            const int c = o % (16 * CB), q = o / (16 * CB);
+            double v = 0.0;
+#pragma unroll
+            for (int i = 0; i < NW; ++i) v += red[wp - wi + i][q][c];
+            if (live && c < w && q0 + q < p) {
+                J.Zs[(zb + c) * p + q0 + q] = v;
+                J.y[(g0 + c) * p + q0 + q] = v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// CTAs of the wide forward step that the device holds at once (per device, computed once)
+int64_t fwd_resident() {
+    static std::atomic<int64_t> cache[64];
+    int occ = 0, sms = 0, dev = 0;
+    MBL_CUDA(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64)
+        if (const int64_t g = cache[dev].load()) return g;
+    MBL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fx_fwd_step, 256, FWD_SMEM));
+    MBL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t g = (int64_t)std::max(1, occ) * sms;
+    if (dev >= 0 && dev < 64) cache[dev].store(g);
+    return g;
+}
+
+}  // namespace
+
+void fx_pack_step(const Plan &pl, const SolveStep &ss, const double *G, int32_t *cex, int32_t *rex, double *out,
+                  cudaStream_t st) {
+    const SolveDesc *sd = pl.d_sdescs.data() + ss.d0;
+    const int64_t base = pl.sdescs[ss.d0].goff;
+    k_fx_colexp<<<dim3((unsigned)ss.nd, (ss.maxw + 15) / 16 * 2), 256, 0, st>>>(sd, G, base, cex);
+    MBL_LAUNCH_CHECK();
+    k_fx_pack<<<(unsigned)ss.nrb, 256, 0, st>>>(sd, pl.d_fblk_desc.data() + ss.fblk0, G, base, cex, rex, out);
+    MBL_LAUNCH_CHECK();
+}
+
+void fx_forward(const Plan &pl, const SolveStep &ss, const SolveBufs<double> *jb, unsigned K, int p, LaunchTrace *tr,
+                cudaStream_t st) {
+    const SolveDesc *sd = pl.d_sdescs.data() + ss.d0;
+    const int32_t *blk = pl.d_fblk_desc.data() + ss.fblk0;
+    if (ss.maxw <= 32) {
+        auto kern = ss.maxw <= 16 ? k_fx_fwd_narrow<1> : k_fx_fwd_narrow<2>;
+        launch_pdl(kern, dim3((unsigned)((ss.nrb + 7) / 8), 1, K), dim3(256), 0, st, sd, blk, (int)ss.nrb,
+                   pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, tr);
+        return;
+    }
+    const int64_t items = ss.nrb * (int64_t)K, cap = fwd_resident();
+    launch_pdl(k_fx_fwd_step, dim3((unsigned)std::min(items, cap)), dim3(256), FWD_SMEM, st, sd, blk, (int)ss.nrb, (int)K,
+               pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, tr);
+}
+
+void fx_backward_level(const Plan &pl, int l, const SolveBufs<double> *jb, unsigned K, int p, LaunchTrace *tr,
+                       cudaStream_t st) {
+    const SolveDesc *sdl = pl.d_sdescs.data() + pl.lvl_d0[l];
+    if (pl.lvl_maxw[l] <= 32 && pl.lvl_maxr[l] <= 1024) {  // the same rule as the FP32 narrow step
+        auto narrow = [&](auto kern, int nw) {
+            launch_pdl(kern, dim3((unsigned)((pl.lvl_nd[l] * nw + 7) / 8), 1, K), dim3(256), 0, st, sdl, pl.lvl_nd[l],
+                       pl.d_sn_zo.data(), pl.d_sn_nc.data(), pl.d_sn_start.data(), pl.d_sn_rows_off.data(),
+                       pl.d_rows.data(), jb, p, tr);
+        };
+        const bool two = pl.lvl_maxr[l] <= 160;
+        if (pl.lvl_maxw[l] <= 16) two ? narrow(k_fx_bwd_narrow<1, 2>, 2) : narrow(k_fx_bwd_narrow<1, 8>, 8);
+        else two ? narrow(k_fx_bwd_narrow<2, 2>, 2) : narrow(k_fx_bwd_narrow<2, 8>, 8);
+        return;
+    }
+    auto wide = [&](auto kern) {
+        launch_pdl(kern, dim3((unsigned)pl.lvl_nrbk[l], (pl.lvl_maxw[l] + RBB - 1) / RBB, K), dim3(256), BWD_SMEM, st,
+                   sdl, (const int32_t *)pl.d_lvl_bblk_desc.data() + pl.lvl_bblk0[l], pl.d_sn_zo.data(),
+                   pl.d_sn_nc.data(), pl.d_sn_start.data(), pl.d_sn_rows_off.data(), pl.d_rows.data(), jb,
+                   (int64_t)pl.lvl_d0[l] * SUBS, p, tr);
+    };
+    if (p <= 8) wide(k_fx_bwd_step<8>);
+    else if (p <= 16) wide(k_fx_bwd_step<16>);
+    else wide(k_fx_bwd_step<32>);
+}
+
+void fx_backward_update(const Plan &pl, const BwdUpd &bu, const SolveBufs<double> *jb, unsigned K, int p,
+                        LaunchTrace *tr, cudaStream_t st) {
+    launch_pdl(k_fx_bwd_update, dim3((unsigned)bu.nit, SUBS, K), dim3(256), BWD_SMEM, st,
+               (const SolveDesc *)pl.d_sdescs.data(), (const int32_t *)pl.d_bu_items.data() + 2 * bu.it0,
+               pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, tr);
+}
+
+void fx_prepare() {
+    smem_limit((const void *)k_fx_fwd_step, FWD_SMEM);
+    smem_limit((const void *)k_fx_bwd_update, BWD_SMEM);
+    smem_limit((const void *)k_fx_bwd_step<8>, BWD_SMEM);
+    smem_limit((const void *)k_fx_bwd_step<16>, BWD_SMEM);
+    smem_limit((const void *)k_fx_bwd_step<32>, BWD_SMEM);
+}
+
+}  // namespace mbl
