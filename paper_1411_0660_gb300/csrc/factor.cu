@@ -20,6 +20,7 @@
 
 #include "factor.h"
 #include "solve_tile.cuh"
+#include "fixed_digits.cuh"
 #include "tc_pieces.cuh"
 
 namespace mbl {
@@ -445,13 +446,13 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *de
                                                    const int32_t *fsz, const int32_t *sn_start, T *arena,
                                                    const T *Dg, const int32_t *piv, T *wscr,
                                                    unsigned long long *stats, void *pieces, int64_t prow,
-                                                   int pmode) {
+                                                   int pmode, int32_t *scales, int64_t srow) {
     static_assert(RB == NB && NB == 64, "a thread per row, a register per column");
     constexpr int E = 16 / sizeof(T);
     using V = typename Vec16<T>::type;
     __shared__ __align__(16) T Ls[NB * NB];  // L11 by columns; then W21 by rows
     __shared__ T Dinv[NB];
-    __shared__ int pv[NB];
+    __shared__ int pv[NB], hexp[NB];
     const int di = find_desc2(descs, nd, blockIdx.x);
     const PanelDesc d = descs[di];
     const int s = d.front, f = fsz[s], k0 = d.k0, w = d.w, m2 = d.m2;
@@ -467,6 +468,9 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *de
     if (tid < NB) {
         Dinv[tid] = tid < w ? T(1) / Dg[g0 + tid] : T(0);
         pv[tid] = tid < w ? piv[g0 + tid] : 0;
+        // a power of two near sqrt|d| (FP64: the columns' scaling of the digit operands)
+        if constexpr (sizeof(T) == 8)
+            hexp[tid] = tid < w ? (((__double2hiint(Dg[g0 + tid]) >> 20) & 0x7ff) - 1023) >> 1 : 0;
     }
     __syncthreads();
     const bool own = tid < nr;
@@ -487,15 +491,58 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *de
             }
         }
         if (own) {
-            T *W = wscr + d.woff + rb + tid;
+            [[maybe_unused]] T *W = wscr + d.woff + rb + tid;
 #pragma unroll
             for (int t = 0; t < NB; ++t) {
                 if (t >= w) break;
                 const T l = x[t] * Dinv[t];
                 F[(int64_t)(k0 + t) * f + r0 + tid] = l;
-                W[(int64_t)t * m2] = x[t];
+                if constexpr (sizeof(T) == 4) W[(int64_t)t * m2] = x[t];
                 lmax = fmaxf(lmax, (float)tabs(l));
             }
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // digits of L21 and W21 for the trailing update (layout: update_fx.cu), through shared memory so that
+        // they leave in whole lines; rows past the front are zero
+        uint32_t *sd = reinterpret_cast<uint32_t *>(Ls);
+        const int nk = (w + 15) / 16, gw = nk * 512;  // words of a 16-row group
+#pragma unroll
+        for (int op = 0; op < 2; ++op) {
+            __syncthreads();
+            if (tid < RB) {
+                const int sg = op ? -1 : 1;
+                int E = FX_NOZERO;
+#pragma unroll
+                for (int t = 0; t < NB; ++t)
+                    if (t < w) E = max(E, fx_exp(op ? x[t] : x[t] * Dinv[t], sg * hexp[t]));
+                scales[op * srow + (int64_t)blockIdx.x * RB + tid] = E >= FX_BAD ? FX_BAD : (E <= FX_NOZERO ? 0 : E - 1022);
+                uint32_t *o = sd + (tid >> 4) * gw + 16 * (tid & 7) + ((tid >> 3) & 1);
+#pragma unroll
+                for (int kb = 0; kb < NB / 16; ++kb) {
+                    if (kb >= nk) break;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        uint64_t y[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int t = 16 * kb + 2 * q + (e & 1) + 8 * (e >> 1);
+                            y[e] = fx_bytes(op ? x[t] : x[t] * Dinv[t], sg * hexp[t], E);
+                        }
+#pragma unroll
+                        for (int i = 0; i < FX_ND; ++i) {
+                            const int sh = 8 * (FX_ND - 1 - i);
+                            o[kb * 512 + (i >> 1) * 128 + 4 * q + 2 * (i & 1)] =
+                                (uint32_t)(y[0] >> sh & 255) | (uint32_t)(y[1] >> sh & 255) << 8 |
+                                (uint32_t)(y[2] >> sh & 255) << 16 | (uint32_t)(y[3] >> sh & 255) << 24;
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            uint4 *dst = reinterpret_cast<uint4 *>(static_cast<uint32_t *>(pieces) + op * prow +
+                                                   (d.xd + (int64_t)(rb / RB) * nk) * 2048);
+            for (int u = tid; u < gw; u += TRSM_THREADS) dst[u] = reinterpret_cast<const uint4 *>(sd)[u];
         }
     }
     if (sizeof(T) == 4 && pmode) {
@@ -1432,9 +1479,10 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                                                                                  p.d_sn_f.data(), p.d_sn_start.data(), arena,
                                                                                  Dg, fz.piv.data(), wscr,
                                                                                  fz.counters.data() + 3,
-                                                                                 fz.tma ? fz.pieces.m.p : nullptr,
+                                                                                 fz.tma || sizeof(T) == 8 ? fz.pieces.m.p : nullptr,
                                                                                  fz.prow,
-                                                                                 fz.tma && sizeof(T) == 4 ? fz.tc_mode : 0);
+                                                                                 fz.tma && sizeof(T) == 4 ? fz.tc_mode : 0,
+                                                                                 fz.uscale.data(), p.max_step_n2 * RB);
                     MBL_LAUNCH_CHECK();
                 }
             }
@@ -1457,9 +1505,13 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                                         fz.tc_mode == 2);
                 } else {
                     ProfScope ps(fz.ctx, sizeof(T) == 8 ? "schur_fp64" : "schur_fp32", fl, st);
-                    k_panel_update<T><<<(unsigned)stp.n3, 256, 0, st>>>(dd, stp.nd, p.d_sn_fo.data(), p.d_sn_f.data(),
-                                                                        arena, wscr);
-                    MBL_LAUNCH_CHECK();
+                    if constexpr (sizeof(T) == 8) {
+                        fx_update(stp, dd, p, arena, fz.pieces.m.p, fz.uscale.data(), st);
+                    } else {
+                        k_panel_update<T><<<(unsigned)stp.n3, 256, 0, st>>>(dd, stp.nd, p.d_sn_fo.data(),
+                                                                            p.d_sn_f.data(), arena, wscr);
+                        MBL_LAUNCH_CHECK();
+                    }
                 }
             }
             if (!lean && (stp.kk % SUBS == SUBS - 1 || si + 1 == p.lvl_step_ptr[l + 1])) {
@@ -1857,7 +1909,13 @@ void Factorization::allocate(bool lean_arena) {
     D.alloc(ctx, (size_t)pl.n * es);
     piv.alloc(ctx, pl.n);
     counters.alloc(ctx, 5);
-    wscr.alloc(ctx, (size_t)std::max<int64_t>(pl.wscratch_elems, 1) * es);
+    if (prec == MBL_PREC_FP64) {
+        prow = pl.max_step_xd * (XD_BYTES / 4);  // words of one operand's digits
+        pieces.alloc(ctx, (size_t)2 * std::max<int64_t>(pl.max_step_xd, 1) * XD_BYTES);
+        uscale.alloc(ctx, (size_t)2 * std::max<int64_t>(pl.max_step_n2, 1) * RB);
+    } else {
+        wscr.alloc(ctx, (size_t)std::max<int64_t>(pl.wscratch_elems, 1) * es);
+    }
     cmax.alloc(ctx, (size_t)std::max<int64_t>(pl.max_desc_per_step, 1) * NB * sizeof(unsigned int));
     M.alloc(ctx, (size_t)std::max<int64_t>(pl.m_elems, 1) * es);
     fx = prec == MBL_PREC_FP64 && !dataflow;
@@ -1892,6 +1950,7 @@ void reset_solve_counters(Factorization &fz, cudaStream_t st) {
 void Factorization::release_scratch() {
     wscr.release();
     pieces.release();
+    uscale.release();
     cmax.release();
     M.release();      // folded into G = [M; L21 M]
     gstep.release();
@@ -1909,7 +1968,7 @@ size_t Factorization::held_bytes() const {
     size_t b = 0;
     for (const DevMem *m : {&arena.m, &D.m, &wscr.m, &cmax.m, &M.m, &zwork.m, &zsolved.m, &ywork.m, &yfw.m, &pwork.m,
                             &gpk.m, &rex.m, &cex.m, &gstep.m, &piv.m, &scnt.m, &dfcnt.m, &counters.m, &trace.m, &dev_b.m, &dev_x.m, &dbufs.m,
-                            &pieces.m})
+                            &pieces.m, &uscale.m})
         b += m->bytes;
     return b;
 }

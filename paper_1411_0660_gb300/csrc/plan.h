@@ -32,6 +32,7 @@ struct PanelDesc {
     int64_t off3;    // prefix count of trailing tiles (stage 3) before this descriptor in its step
     int64_t woff;    // offset (elements) of this front's W21 scratch (m2 x NB column-major, ld m2)
     int64_t off3t;   // prefix count of 128 x 128 tensor-core tiles before this descriptor in its step
+    int64_t xd;      // prefix count of 64-row x 16-column digit blocks (FP64 fronts, one operand) in its step
 };
 
 struct PanelStep {
@@ -198,6 +199,7 @@ struct Plan {
     // digit form of the packed solve factor (FP64 fronts): 32 x 16 tiles, row scales, column scales; and the
     // most elements of one solve step's G (built in FP64 before its digits are taken)
     int64_t x_tiles = 0, x_rows = 0, x_cols = 0, max_step_g = 0;
+    int64_t max_step_xd = 0;  // most digit blocks of one operand in a panel step (PanelDesc::xd)
     int64_t arena_elems = 0, zwork_elems = 0, wscratch_elems = 0, max_desc_per_step = 0;
     int64_t max_step_n2 = 0;
     int64_t nnz_l = 0;
