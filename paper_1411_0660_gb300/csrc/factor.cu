@@ -445,7 +445,7 @@ template <class T>
 __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *descs, int nd, const int64_t *fo,
                                                    const int32_t *fsz, const int32_t *sn_start, T *arena,
                                                    const T *Dg, const int32_t *piv, T *wscr,
-                                                   unsigned long long *stats, void *pieces, int64_t prow,
+                                                   unsigned long long *stats, void *pieces, int64_t w_off,
                                                    int pmode, int32_t *scales, int64_t srow) {
     static_assert(RB == NB && NB == 64, "a thread per row, a register per column");
     constexpr int E = 16 / sizeof(T);
@@ -540,57 +540,49 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *de
                 }
             }
             __syncthreads();
-            uint4 *dst = reinterpret_cast<uint4 *>(static_cast<uint32_t *>(pieces) + op * prow +
+            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(pieces) + op * w_off) +
                                                    (d.xd + (int64_t)(rb / RB) * nk) * 2048);
             for (int u = tid; u < gw; u += TRSM_THREADS) dst[u] = reinterpret_cast<const uint4 *>(sd)[u];
         }
     }
-    if (sizeof(T) == 4 && pmode) {
-        // tensor-core operand pieces of this block's rows of L21 and W21 (pieces 0/1 and 2/3), row-major
-        // with NB per row, zero past the panel width; rows start at the descriptor's woff / NB.  W21 goes
-        // through shared memory (16-byte group g of row i at g ^ (i % 16): no bank conflicts) so that
-        // the pieces leave in whole rows.
-        __syncthreads();
-        V *Wv = reinterpret_cast<V *>(Ls);
-        if (tid < RB) {
+    if constexpr (sizeof(T) == 4) {
+        // tensor-core operand pieces of this block's rows (layout: schur_tc.cu): a thread's row, a 16-byte k group
+        // at a time, so that a warp's stores are whole lines; zero past the panel width
+        if (pmode && own) {
+            unsigned char *o = static_cast<unsigned char *>(pieces) + (d.pb + (int64_t)(rb / 128) * panel_kg(w)) * PB_BYTES +
+                               16 * (rb % 128 + tid);
+            const int kg = 2 * (pmode == 1 ? (w + 7) / 8 : (w + 15) / 16);
+            constexpr int G1 = NB / 4;
 #pragma unroll
-            for (int g = 0; g < NB / E; ++g) {
-                V v;
-                T *ve = reinterpret_cast<T *>(&v);
+            for (int g = 0; g < G1; ++g) {
+                if (pmode == 1 ? g >= kg : (g >= kg || g >= NB / 8)) break;
+                uint4 v[4];
+                if (pmode == 1) {
+                    uint32_t u[4][4];
 #pragma unroll
-                for (int e = 0; e < E; ++e) ve[e] = x[g * E + e];
-                Wv[tid * (NB / E) + (g ^ (tid % (NB / E)))] = v;
-            }
-        }
-        __syncthreads();
-        const int64_t p0 = d.woff / NB + rb;
-        for (int idx = tid; idx < nr * (NB / 4); idx += TRSM_THREADS) {
-            const int i = idx / (NB / 4), g = idx % (NB / 4);
-            const float *xr = reinterpret_cast<const float *>(Wv) + ((size_t)i * (NB / 4) + (g ^ (i % (NB / 4)))) * 4;
-            const int64_t e = (p0 + i) * NB + g * 4;
-            if (pmode == 1) {
-                uint32_t v[4][4];
+                    for (int e = 0; e < 4; ++e) {
+                        split_tf32((float)(x[4 * g + e] * Dinv[4 * g + e]), u[0][e], u[1][e]);
+                        split_tf32(x[4 * g + e], u[2][e], u[3][e]);
+                    }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    split_tf32((float)(xr[u] * (float)Dinv[g * 4 + u]), v[0][u], v[1][u]);
-                    split_tf32(xr[u], v[2][u], v[3][u]);
+                    for (int q = 0; q < 4; ++q) v[q] = make_uint4(u[q][0], u[q][1], u[q][2], u[q][3]);
+                } else {
+                    uint16_t u[4][8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int k = (8 * g + e) % NB;
+                        split_bf16((float)(x[k] * Dinv[k]), u[0][e], u[1][e]);
+                        split_bf16(x[k], u[2][e], u[3][e]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        v[q] = make_uint4(u[q][0] | (uint32_t)u[q][1] << 16, u[q][2] | (uint32_t)u[q][3] << 16,
+                                          u[q][4] | (uint32_t)u[q][5] << 16, u[q][6] | (uint32_t)u[q][7] << 16);
                 }
-                uint32_t *P = static_cast<uint32_t *>(pieces);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<uint4 *>(P + q * prow * NB + e) = make_uint4(v[q][0], v[q][1], v[q][2], v[q][3]);
-            } else {
-                uint16_t v[4][4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    split_bf16((float)(xr[u] * (float)Dinv[g * 4 + u]), v[0][u], v[1][u]);
-                    split_bf16(xr[u], v[2][u], v[3][u]);
-                }
-                uint16_t *P = static_cast<uint16_t *>(pieces);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<uint2 *>(P + q * prow * NB + e) =
-                        make_uint2(v[q][0] | (uint32_t)v[q][1] << 16, v[q][2] | (uint32_t)v[q][3] << 16);
+                *reinterpret_cast<uint4 *>(o + 2048 * g) = v[0];
+                *reinterpret_cast<uint4 *>(o + 2048 * (kg + g)) = v[1];
+                *reinterpret_cast<uint4 *>(o + w_off + 2048 * g) = v[2];
+                *reinterpret_cast<uint4 *>(o + w_off + 2048 * (kg + g)) = v[3];
             }
         }
     }
@@ -1480,7 +1472,7 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                                                                                  Dg, fz.piv.data(), wscr,
                                                                                  fz.counters.data() + 3,
                                                                                  fz.tma || sizeof(T) == 8 ? fz.pieces.m.p : nullptr,
-                                                                                 fz.prow,
+                                                                                 fz.w_off,
                                                                                  fz.tma && sizeof(T) == 4 ? fz.tc_mode : 0,
                                                                                  fz.uscale.data(), p.max_step_n2 * RB);
                     MBL_LAUNCH_CHECK();
@@ -1492,17 +1484,12 @@ static void factor_impl(Factorization &fz, cudaStream_t st) {
                     fl += (double)p.descs[q].m2 * (p.descs[q].m2 + 1) * p.descs[q].w;
                 // the autotuned tile shape of this step's size class (tensor cores unless the tuning found the
                 // CUDA-core tiles faster for it)
-                const bool tc = sizeof(T) == 4 && fz.tc_mode != 0 &&
+                const bool tc = sizeof(T) == 4 && fz.tma &&
                                 (!p.tuned[fz.tc_mode] || p.tune_tc[fz.tc_mode][p.step_class[si]]);
                 if (tc) {
                     ProfScope ps(fz.ctx, "schur_tc", fl, st);
-                    if (fz.tma)
-                        launch_schur_tma(stp, dd, p.d_sn_fo.data(), p.d_sn_f.data(), reinterpret_cast<float *>(arena),
-                                         fz.tmap, fz.counters.data() + 2, st, fz.tc_mode == 2);
-                    else
-                        launch_schur_tc(stp, dd, p, reinterpret_cast<float *>(arena),
-                                        reinterpret_cast<const float *>(wscr), fz.counters.data() + 2, st,
-                                        fz.tc_mode == 2);
+                    launch_schur(stp, dd, p.d_sn_fo.data(), p.d_sn_f.data(), reinterpret_cast<float *>(arena),
+                                 fz.pieces.m.p, fz.w_off, fz.counters.data() + 2, st, fz.tc_mode == 2);
                 } else {
                     ProfScope ps(fz.ctx, sizeof(T) == 8 ? "schur_fp64" : "schur_fp32", fl, st);
                     if constexpr (sizeof(T) == 8) {
@@ -1562,7 +1549,8 @@ void tune_schur(Factorization &fz, cudaStream_t st) {
         DVec<int32_t> fsz;
         F.alloc(fz.ctx, (size_t)f * f);
         W.alloc(fz.ctx, (size_t)m2 * NB);
-        pc.alloc(fz.ctx, (size_t)4 * m2 * NB * (mode == 2 ? 2 : 4));
+        const int64_t wo = (int64_t)((m2 + 127) / 128) * panel_kg(NB) * PB_BYTES;
+        pc.alloc(fz.ctx, (size_t)(2 * wo));
         dd.alloc(fz.ctx, 1);
         fo.alloc(fz.ctx, 1);
         fsz.alloc(fz.ctx, 1);
@@ -1571,13 +1559,11 @@ void tune_schur(Factorization &fz, cudaStream_t st) {
         k_fill_hash<<<(unsigned)(((int64_t)m2 * NB + 255) / 256), 256, 0, st>>>(W.data(), (int64_t)m2 * NB, 7u + c);
         MBL_LAUNCH_CHECK();
         MBL_CUDA(cudaMemsetAsync(pc.data(), 0, pc.size(), st));
-        const PanelDesc d{0, 0, NB, m2, 0, 0, 0, 0};
+        const PanelDesc d{0, 0, NB, m2, 0, 0, 0, 0, 0, 0};
         const int64_t z = 0;
         MBL_CUDA(cudaMemcpyAsync(dd.data(), &d, sizeof(d), cudaMemcpyHostToDevice, st));
         MBL_CUDA(cudaMemcpyAsync(fo.data(), &z, sizeof(z), cudaMemcpyHostToDevice, st));
         MBL_CUDA(cudaMemcpyAsync(fsz.data(), &f, sizeof(int), cudaMemcpyHostToDevice, st));
-        alignas(64) unsigned char map[128];
-        if (!encode_pieces_map(map, pc.data(), m2, mode == 2)) continue;
         PanelStep stp{};
         stp.nd = 1;
         const int64_t T64 = (m2 + TB - 1) / TB, T128 = (m2 + 127) / 128;
@@ -1589,7 +1575,7 @@ void tune_schur(Factorization &fz, cudaStream_t st) {
         for (int v = 0; v < 2; ++v) {
             auto run = [&] {
                 if (v == 0)
-                    launch_schur_tma(stp, dd.data(), fo.data(), fsz.data(), F.data(), map, err, st, mode == 2);
+                    launch_schur(stp, dd.data(), fo.data(), fsz.data(), F.data(), pc.data(), wo, err, st, mode == 2);
                 else {
                     k_panel_update<float><<<(unsigned)stp.n3, 256, 0, st>>>(dd.data(), 1, fo.data(), fsz.data(),
                                                                             F.data(), W.data());
@@ -1910,7 +1896,7 @@ void Factorization::allocate(bool lean_arena) {
     piv.alloc(ctx, pl.n);
     counters.alloc(ctx, 5);
     if (prec == MBL_PREC_FP64) {
-        prow = pl.max_step_xd * (XD_BYTES / 4);  // words of one operand's digits
+        w_off = pl.max_step_xd * XD_BYTES;
         pieces.alloc(ctx, (size_t)2 * std::max<int64_t>(pl.max_step_xd, 1) * XD_BYTES);
         uscale.alloc(ctx, (size_t)2 * std::max<int64_t>(pl.max_step_n2, 1) * RB);
     } else {
@@ -1931,12 +1917,10 @@ void Factorization::allocate(bool lean_arena) {
     dfcnt.alloc(ctx, (size_t)4 * pl.ns + 2);
     tma = false;
     if (prec == MBL_PREC_FP32 && tc_mode != 0 && pl.wscratch_elems > 0) {
-        // operand pieces of the TMA-fed Schur update: 4 arrays of prow rows x NB pieces
-        prow = pl.wscratch_elems / NB;
-        const size_t eb = tc_mode == 2 ? 2 : 4;
-        pieces.alloc(ctx, (size_t)4 * prow * NB * eb);
-        tma = encode_pieces_map(tmap, pieces.m.p, prow, tc_mode == 2);
-        if (!tma) pieces.release();
+        // operand pieces of the tensor-core trailing update
+        w_off = pl.max_step_pb * PB_BYTES;
+        pieces.alloc(ctx, (size_t)(2 * std::max<int64_t>(w_off, 1)));
+        tma = true;
     }
     MBL_CUDA(cudaMemset(scnt.data(), 0, std::max<size_t>(pl.sdescs.size() * SUBS, 1) * sizeof(unsigned int)));
 }

@@ -30,7 +30,7 @@ inline double solve_factor_scratch(const Plan &p, int prec) { return prec == MBL
 // and scales of L21 and W21 (FP64 fronts, update_fx.cu).
 constexpr int64_t XD_BYTES = 8192;  // one digit block
 inline double panel_scratch_bytes(const Plan &p, int prec) {
-    return prec == MBL_PREC_FP64 ? 2.0 * (double)(p.max_step_xd * XD_BYTES + 4 * p.max_step_n2 * RB) : 20.0 * (double)p.wscratch_elems;
+    return prec == MBL_PREC_FP64 ? 2.0 * (double)(p.max_step_xd * XD_BYTES + 4 * p.max_step_n2 * RB) : 4.0 * (double)p.wscratch_elems + 2.0 * (double)(p.max_step_pb * PB_BYTES);
 }
 
 // Trailing update of FP64 fronts (update_fx.cu): digits of L21 and W21 (each p.max_step_xd blocks), their row
@@ -91,8 +91,7 @@ struct Factorization {
     long long graph_nodes = 0;
     int tc_mode = 1;  // FP32 fronts' Schur updates: 0 CUDA cores, 1 tcgen05 3xTF32, 2 tcgen05 3xBF16
     DVec<char> pieces;                    // tensor-core operand pieces of the step's L21 and W21
-    int64_t prow = 0;                     // rows of each piece array
-    alignas(64) unsigned char tmap[128];  // tensor map over the pieces (TMA-fed Schur update)
+    int64_t w_off = 0;                    // bytes from L21's operands in `pieces` to W21's
     bool tma = false;                     // the pieces and their tensor map are ready
     // launch trace of the level-by-level solve (opt-in; recaptures the solve graph when switched)
     bool trace_on = false;
@@ -147,20 +146,14 @@ void batcher_stats(SolveBatcher *b, int64_t *batches, int64_t *solves, double *m
 template <class T>
 SolveBufs<T> solve_bufs(const Factorization &fz);
 
-// tcgen05 trailing update of one panel step (FP32 fronts); err counts bounded-wait time-outs.  The
-// TMA-fed form reads the operand pieces the panel's trsm wrote (tensor map from encode_pieces_map over
-// 4 x prow x NB pieces); the other form splits the raw operands itself.
-size_t schur_tc_smem(bool bf16);
-bool encode_pieces_map(void *map, void *pieces, int64_t prow, bool bf16);
-void launch_schur_tma(const PanelStep &stp, const PanelDesc *d_descs, const int64_t *fo, const int32_t *fsz,
-                      float *arena, const void *map, unsigned long long *err, cudaStream_t st, bool bf16);
 // Autotuning of the FP32 fronts' trailing update (once per plan and tensor-core mode): for every size
 // class of trailing block that the plan's panel steps have, time one update of a synthetic front of
-// that class with tcgen05 128 x 128 tiles (TMA-fed) and with CUDA-core 64 x 64 tiles, and keep the
-// faster in the plan.
+// that class with tcgen05 128 x 64 tiles and with CUDA-core 64 x 64 tiles, and keep the faster in the plan.
 void tune_schur(Factorization &fz, cudaStream_t st);
-void launch_schur_tc(const PanelStep &stp, const PanelDesc *d_descs, const Plan &p, float *arena, const float *wscr,
-                     unsigned long long *err, cudaStream_t st, bool bf16);
+// FP32 fronts' trailing update on the tensor cores (schur_tc.cu): 3xTF32, or 3xBF16, from the operand pieces that
+// the panel's trsm wrote (L21's, and w_off bytes further W21's).
+void launch_schur(const PanelStep &stp, const PanelDesc *d_descs, const int64_t *fo, const int32_t *fsz, float *arena,
+                  const void *pieces, int64_t w_off, unsigned long long *err, cudaStream_t st, bool bf16);
 
 // Both sweeps of a block solve as dataflow kernels (solve_df.cu), between the permutations.
 template <class T>

@@ -32,8 +32,17 @@ struct PanelDesc {
     int64_t off3;    // prefix count of trailing tiles (stage 3) before this descriptor in its step
     int64_t woff;    // offset (elements) of this front's W21 scratch (m2 x NB column-major, ld m2)
     int64_t off3t;   // prefix count of 128 x 128 tensor-core tiles before this descriptor in its step
+    int64_t pb;      // prefix count of operand-piece k groups (panel_kg per 128-row block) in its step
     int64_t xd;      // prefix count of 64-row x 16-column digit blocks (FP64 fronts, one operand) in its step
 };
+
+// 16-byte k groups of a 128-row block of tensor-core operand pieces (TF32; BF16 needs half), and the bytes
+// of one (two pieces of 128 rows): the unit of PanelDesc::pb
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int panel_kg(int w) { return 2 * ((w + 7) / 8); }
+constexpr int64_t PB_BYTES = 2 * 128 * 16;
 
 struct PanelStep {
     int32_t level, kk;
@@ -199,6 +208,7 @@ struct Plan {
     // digit form of the packed solve factor (FP64 fronts): 32 x 16 tiles, row scales, column scales; and the
     // most elements of one solve step's G (built in FP64 before its digits are taken)
     int64_t x_tiles = 0, x_rows = 0, x_cols = 0, max_step_g = 0;
+    int64_t max_step_pb = 0;  // most operand-piece k groups in a panel step (PanelDesc::pb)
     int64_t max_step_xd = 0;  // most digit blocks of one operand in a panel step (PanelDesc::xd)
     int64_t arena_elems = 0, zwork_elems = 0, wscratch_elems = 0, max_desc_per_step = 0;
     int64_t max_step_n2 = 0;

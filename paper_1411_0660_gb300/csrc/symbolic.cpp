@@ -843,14 +843,15 @@ std::shared_ptr<Plan> build_plan(int L, const std::vector<uint32_t> &states, con
         p.asm_ptr[l + 1] = (int32_t)p.asm_items.size();
         for (int32_t kk = 0; kk * NB < maxnc; ++kk) {
             PanelStep stp{l, kk, (int32_t)p.descs.size(), 0, 0, 0, 0, 0};
-            int64_t xd = 0;
+            int64_t pb = 0, xd = 0;
             for (int32_t q = p.lvl_ptr[l]; q < p.lvl_ptr[l + 1]; ++q) {
                 int32_t s = p.lvl_fronts[q];
                 int32_t k0 = kk * NB;
                 if (p.sn_nc[s] <= k0) continue;
                 int32_t w = std::min(NB, p.sn_nc[s] - k0);
                 int32_t m2 = p.sn_f[s] - k0 - w;
-                PanelDesc d{s, k0, w, m2, stp.n2, stp.n3, stp.wsize, stp.n3t, xd};
+                PanelDesc d{s, k0, w, m2, stp.n2, stp.n3, stp.wsize, stp.n3t, pb, xd};
+                pb += (int64_t)((m2 + 127) / 128) * panel_kg(w);
                 xd += (int64_t)((m2 + RB - 1) / RB) * ((w + 15) / 16);
                 fd_of[fd_off[s] + kk] = (int32_t)p.descs.size();
                 int64_t nb2 = (m2 + RB - 1) / RB;
@@ -870,6 +871,7 @@ std::shared_ptr<Plan> build_plan(int L, const std::vector<uint32_t> &states, con
             }
             p.max_desc_per_step = std::max<int64_t>(p.max_desc_per_step, stp.nd);
             p.max_step_n2 = std::max<int64_t>(p.max_step_n2, stp.n2);
+            p.max_step_pb = std::max(p.max_step_pb, pb);
             p.max_step_xd = std::max(p.max_step_xd, xd);
             p.wscratch_elems = std::max(p.wscratch_elems, stp.wsize);
             p.steps.push_back(stp);
