@@ -19,6 +19,7 @@
 #include <cfloat>
 
 #include "krylov.h"
+#include "sturm.cuh"
 
 namespace mbl {
 
@@ -1066,103 +1067,144 @@ __global__ void k_normalize_first(int64_t n, double *V, int ldv, const double *p
         V[i * ldv] *= inv;
 }
 
-// Plain Lanczos steps of the extremal bounds, over LZ_BLOCKS CTAs of 256 threads with grid-stride
-// loops.  Every CTA sums the previous kernel's LZ_BLOCKS partial sums itself, in the same order, so
-// all CTAs use identical coefficients and no single-thread launch sits between the steps.
-constexpr int LZ_BLOCKS = 304;
+// ---- plain Lanczos steps of the extremal bounds ----
+constexpr int LZ_THREADS = 512, LZ_TPR = 4;  // threads a CTA, lanes a row
+constexpr uint64_t LZ_WAIT_NS = 2000000000ull;
 
-__device__ double lz_block_sum(double s) {
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+// Sum over the CTA in a fixed order; every thread gets it.
+__device__ double lz_block_sum(double s, double *red) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    double t = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
+    double t = (threadIdx.x & 31) < LZ_THREADS / 32 ? red[threadIdx.x & 31] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     return t;
 }
 
-// sum of the LZ_BLOCKS partial sums in a fixed order (a warp per CTA, then across the lanes)
-__device__ double lz_total(const double *part) {
-    __shared__ double tot;
-    if (threadIdx.x < 32) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < LZ_BLOCKS; b += 32) s += part[b];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) tot = s;
+// Sum of s over the grid: the CTAs' sums meet in part[] (one slot each) and every CTA adds them in the same
+// order, so that all use the same bits.  Waits for the other CTAs (co-resident: a cooperative launch), at
+// most LZ_WAIT_NS; false on expiry, which is counted in *err.
+__device__ bool lz_grid_sum(double s, double *part, unsigned int *bar, unsigned int target, double *red,
+                            unsigned long long *err, double *total) {
+    __shared__ int ok;
+    const double b = lz_block_sum(s, red);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = b;
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const uint64_t t0 = global_ns();
+        unsigned int v;
+        ok = 1;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= target) break;
+            if (global_ns() - t0 > LZ_WAIT_NS) {
+                ok = 0;
+                atomicAdd(err, 1ull);
+                break;
+            }
+        }
     }
     __syncthreads();
-    return tot;
+    if (!ok) return false;
+    double t = 0.0;
+    for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    *total = t;
+    return true;
 }
 
-// dot[b] = partial sums of v^T (w - beta_{j-1} v_prev)
-__global__ void k_lz_dot(int64_t n, int j, const double *v, const double *vprev, const double *w, const double *beta,
-                         double *dot) {
-    const double b = j > 0 ? beta[j - 1] : 0.0;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += v[i] * (w[i] - b * vprev[i]);
-    s = lz_block_sum(s);
-    if (threadIdx.x == 0) dot[blockIdx.x] = s;
-}
-
-// alpha_j = sum(dot); w <- w - beta_{j-1} v_prev - alpha_j v; nrm[b] = partial sums of |w|^2
-__global__ void k_lz_update(int64_t n, int j, const double *v, const double *vprev, double *w, const double *dot,
-                            double *alpha, const double *beta, double *nrm) {
-    const double a = lz_total(dot), b = j > 0 ? beta[j - 1] : 0.0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) alpha[j] = a;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double x = w[i] - b * vprev[i] - a * v[i];
-        w[i] = x;
-        s += x * x;
+// Steps j0 .. j0 + steps - 1 of the three-term recurrence, one launch: w holds v_j times its norm beta_{j-1}
+// (1 for j = 0), vprev v_{j-1}.  Per step: u = H v_j - beta_{j-1} v_{j-1} and alpha_j = v_j . u, a grid-wide
+// sum; then w <- u - alpha_j v_j, vprev <- v_j and beta_j = |w|, another.  LZ_TPR lanes share a row; a thread
+// group's rows and every sum's order are fixed by the grid, which is fixed by n.
+// Bound by latency: a step is two grid-wide sums (some 2 us each) and one pass over H from L2.  As four
+// launches a step the bounds took 10.4 ms at L = 20 and 2.9 ms at L = 12, with the bisection below; @LZ@
+__global__ void __launch_bounds__(LZ_THREADS) k_lz_steps(int64_t n, const int64_t *__restrict__ rowptr,
+                                                         const int32_t *__restrict__ col,
+                                                         const double *__restrict__ val, int j0, int steps, double *w,
+                                                         double *vprev, double *u, double *alpha, double *beta,
+                                                         double *part, unsigned int *bar, unsigned long long *err) {
+    __shared__ double red[LZ_THREADS / 32];
+    const int sub = threadIdx.x % LZ_TPR;
+    const int64_t g0 = ((int64_t)blockIdx.x * LZ_THREADS + threadIdx.x) / LZ_TPR;
+    const int64_t gs = (int64_t)gridDim.x * LZ_THREADS / LZ_TPR;
+    double bprev = j0 > 0 ? beta[j0 - 1] : 0.0;
+    unsigned int target = 0;
+    for (int j = j0; j < j0 + steps; ++j) {
+        const double inv = j > 0 ? (bprev > 0.0 ? 1.0 / bprev : 0.0) : 1.0;
+        double dot = 0.0;
+        for (int64_t ib = g0 - g0 % (32 / LZ_TPR); ib < n; ib += gs) {  // the warp's rows (uniform: shuffles below)
+            const int64_t i = ib + g0 % (32 / LZ_TPR);
+            double s = 0.0;
+            if (i < n)
+                for (int64_t e = rowptr[i] + sub; e < rowptr[i + 1]; e += LZ_TPR) s = fma(val[e], __ldcg(w + col[e]), s);
+#pragma unroll
+            for (int o = 1; o < LZ_TPR; o *= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (i < n && sub == 0) {
+                const double x = s * inv - bprev * vprev[i];
+                u[i] = x;
+                dot += w[i] * inv * x;
+            }
+        }
+        double a, b2;
+        target += gridDim.x;
+        if (!lz_grid_sum(dot, part, bar, target, red, err, &a)) return;
+        double nr = 0.0;
+        for (int64_t i = g0; i < n; i += gs)
+            if (sub == 0) {
+                const double v = w[i] * inv, x = u[i] - a * v;
+                vprev[i] = v;
+                w[i] = x;
+                nr += x * x;
+            }
+        target += gridDim.x;
+        if (!lz_grid_sum(nr, part + gridDim.x, bar, target, red, err, &b2)) return;
+        bprev = sqrt(b2);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            alpha[j] = a;
+            beta[j] = bprev;
+        }
     }
-    s = lz_block_sum(s);
-    if (threadIdx.x == 0) nrm[blockIdx.x] = s;
 }
 
-// beta_j = sqrt(sum(nrm)); out = w / beta_j (out may be v_prev: every read of it is done)
-__global__ void k_lz_scale(int64_t n, int j, const double *w, const double *nrm, double *beta, double *out) {
-    const double b = sqrt(lz_total(nrm));
-    if (blockIdx.x == 0 && threadIdx.x == 0) beta[j] = b;
-    const double inv = b > 0.0 ? 1.0 / b : 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = w[i] * inv;
-}
-
-__device__ int tri_sturm(int m, const double *a, const double *b, double x) {
-    const double pivmin = 1e-300;
-    int c = 0;
-    double q = a[0] - x;
-    if (fabs(q) < pivmin) q = -pivmin;
-    c += q < 0.0;
-    for (int i = 1; i < m; ++i) {
-        q = (a[i] - x) - b[i - 1] * b[i - 1] / q;
-        if (fabs(q) < pivmin) q = -pivmin;
-        c += q < 0.0;
-    }
-    return c;
-}
-
-// Extreme eigenvalues of the Lanczos tridiagonal T (alpha, beta) by bisection, and the last component
-// of their unit eigenvectors by two steps of inverse iteration.  out = {lo, hi, z_lo, z_hi}.
-__global__ void k_tridiag_extremes(int m, const double *a, const double *b, double *scratch, double *out) {
-    // warp 0 finds the smallest eigenvalue, warp 1 the largest: multisection, each lane one Sturm
-    // count per round (32 points split the bracket into 33 parts), then lane 0 inverse-iterates
+// Extreme eigenvalues of the Lanczos tridiagonal T (alpha, beta), m <= LZ_MAX, and the last component of
+// their unit eigenvectors.  out = {lo, hi, z_lo, z_hi}.  Warp 0 the smallest, warp 1 the largest:
+// multisection, each lane one Sturm count per round (32 points split the bracket into 33 parts); then the
+// eigenvector by the twisted factorization of T - lambda (pivots from the top on one lane and from the bottom
+// on another; the twist where they match best), whose components come out by products of ratios, each with
+// a small relative error even where it is 1e-13 of the largest.
+constexpr int LZ_MAX = 1200;
+__global__ void __launch_bounds__(64) k_tridiag_extremes(int m, const double *a, const double *b, double *scratch,
+                                                         double *out) {
+    extern __shared__ double sm_tri[];
+    double *sa = sm_tri, *sb2 = sm_tri + LZ_MAX;  // scaled to a norm of about 1
     const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (which > 1) return;
-    double gl = a[0], gu = a[0];
-    for (int i = 0; i < m; ++i) {
-        double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < m ? fabs(b[i]) : 0.0);
+    double gl = INFINITY, gu = -INFINITY;
+    for (int i = lane; i < m; i += 32) {
+        const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < m ? fabs(b[i]) : 0.0);
         gl = fmin(gl, a[i] - r);
         gu = fmax(gu, a[i] + r);
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        gl = fmin(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+        gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+    }
+    const double tn = fmax(fabs(gl), fabs(gu));
+    const int ex = tn > 0.0 && tn < INFINITY ? ilogb(tn) : 0;
+    for (int i = threadIdx.x; i < m; i += 64) {
+        sa[i] = scalbn(a[i], -ex);
+        const double bs = i + 1 < m ? scalbn(b[i], -ex) : 0.0;
+        sb2[i] = bs * bs;
+    }
+    __syncthreads();
     const int j = which == 0 ? 0 : m - 1;
-    double lo = gl - 1e-12 * (fabs(gl) + fabs(gu)), hi = gu + 1e-12 * (fabs(gl) + fabs(gu));
+    double lo = scalbn(gl - 1e-12 * (fabs(gl) + fabs(gu)), -ex), hi = scalbn(gu + 1e-12 * (fabs(gl) + fabs(gu)), -ex);
     for (int it = 0; it < 64; ++it) {
         const double step = (hi - lo) / 33.0;
         const double x = lo + (lane + 1) * step;
-        const bool above = x < hi && tri_sturm(m, a, b, x) > j;  // x lies above eigenvalue j
+        const bool above = x < hi && sturm_count_minors(m, sa, sb2, x) > j;  // x lies above eigenvalue j
         const unsigned int mask = __ballot_sync(0xffffffffu, above);
         const int first = mask ? __ffs(mask) - 1 : 32;  // first point above it (32: none)
         const double nlo = first == 0 ? lo : lo + first * step;
@@ -1172,45 +1214,54 @@ __global__ void k_tridiag_extremes(int m, const double *a, const double *b, doub
         hi = fmin(nhi, hi);
         if (hi - lo <= 4.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi))) break;
     }
-    if (lane != 0) return;
     const double lam = 0.5 * (lo + hi);
-    // inverse iteration on T - lam I (LU with partial pivoting of the tridiagonal)
-    double *u1 = scratch + (size_t)which * 6 * m, *u2 = u1 + m, *u3 = u2 + m, *l = u3 + m, *x = l + m, *fl = x + m;
-    const double tiny = 1e-15 * (fabs(gl) + fabs(gu)) + 1e-300;
-    double aa = a[0] - lam, bb = m > 1 ? b[0] : 0.0;
-    for (int i = 0; i < m - 1; ++i) {
-        double c = b[i], an = a[i + 1] - lam, bn = (i + 1 < m - 1) ? b[i + 1] : 0.0;
-        if (fabs(aa) >= fabs(c)) {
-            if (aa == 0.0) aa = tiny;
-            double mult = c / aa;
-            u1[i] = aa; u2[i] = bb; u3[i] = 0.0; l[i] = mult; fl[i] = 0.0;
-            aa = an - mult * bb;
-            bb = bn;
-        } else {
-            double mult = aa / c;
-            u1[i] = c; u2[i] = an; u3[i] = bn; l[i] = mult; fl[i] = 1.0;
-            aa = bb - mult * an;
-            bb = -mult * bn;
+    // pivots from the top (lane 0) and from the bottom (lane 1) of T - lambda
+    double *dt = scratch + (size_t)which * 4 * m, *db = dt + m, *rt = db + m, *rb = rt + m;
+    const double tiny = 1e-30;
+    if (lane < 2) {
+        double q = 0.0;
+        for (int k = 0; k < m; ++k) {
+            const int i = lane == 0 ? k : m - 1 - k;
+            double x = sa[i] - lam;
+            if (k > 0) x -= sb2[lane == 0 ? i - 1 : i] / q;
+            if (fabs(x) < tiny) x = -tiny;
+            (lane == 0 ? dt : db)[i] = x;
+            q = x;
         }
     }
-    if (fabs(aa) < tiny) aa = aa >= 0.0 ? tiny : -tiny;
-    u1[m - 1] = aa;
-    for (int i = 0; i < m; ++i) x[i] = 1.0 / sqrt((double)m) * ((i & 1) ? 1.0 : 0.7);
-    for (int it = 0; it < 3; ++it) {
-        for (int i = 0; i < m - 1; ++i) {
-            if (fl[i] != 0.0) { double t = x[i]; x[i] = x[i + 1]; x[i + 1] = t; }
-            x[i + 1] -= l[i] * x[i];
-        }
-        x[m - 1] /= u1[m - 1];
-        if (m > 1) x[m - 2] = (x[m - 2] - u2[m - 2] * x[m - 1]) / u1[m - 2];
-        for (int i = m - 3; i >= 0; --i) x[i] = (x[i] - u2[i] * x[i + 1] - u3[i] * x[i + 2]) / u1[i];
-        double nrm = 0.0;
-        for (int i = 0; i < m; ++i) nrm += x[i] * x[i];
-        nrm = sqrt(nrm);
-        for (int i = 0; i < m; ++i) x[i] /= nrm;
+    __syncwarp();
+    double best = INFINITY;
+    int tw = 0;
+    for (int i = lane; i < m; i += 32) {
+        const double gm = fabs(dt[i] + db[i] - (sa[i] - lam));
+        if (gm < best) best = gm, tw = i;
+        const double bi = i + 1 < m ? scalbn(b[i], -ex) : 0.0;
+        rt[i] = -bi / dt[i];                          // z_i = rt_i z_{i+1} above the twist
+        rb[i] = i + 1 < m ? -bi / db[i + 1] : 0.0;    // z_{i+1} = rb_i z_i below it
     }
-    out[which] = lam;
-    out[2 + which] = x[m - 1];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int ot = __shfl_xor_sync(0xffffffffu, tw, o);
+        if (ob < best || (ob == best && ot < tw)) best = ob, tw = ot;
+    }
+    __syncwarp();
+    double z = 1.0, nrm = 0.0;
+    if (lane == 0)
+        for (int i = tw - 1; i >= 0; --i) {
+            z *= rt[i];
+            nrm = fma(z, z, nrm);
+        }
+    if (lane == 1)
+        for (int i = tw; i + 1 < m; ++i) {
+            z *= rb[i];
+            nrm = fma(z, z, nrm);
+        }
+    const double n2 = 1.0 + __shfl_sync(0xffffffffu, nrm, 0) + __shfl_sync(0xffffffffu, nrm, 1);
+    z = __shfl_sync(0xffffffffu, z, 1);
+    if (lane == 0) {
+        out[which] = scalbn(lam, ex);
+        out[2 + which] = z / sqrt(n2);
+    }
 }
 
 void extremal_bounds(mbl_sector *sec, double *emin, double *emax) {
@@ -1238,55 +1289,65 @@ void extremal_bounds(mbl_sector *sec, double *emin, double *emax) {
     // Plain Lanczos (three-term recurrence, no reorthogonalization): only the extreme Ritz values
     // are wanted, and in finite precision those still converge to the extreme eigenvalues; the lost
     // orthogonality only adds copies of converged Ritz values (Paige's analysis of the method).
-    const int mmax = (int)std::min<int64_t>(n - 1, 1200);
-    const int ldv = mmax + 1;
+    const int mmax = (int)std::min<int64_t>(n - 1, LZ_MAX);
+    const int grid = (int)std::min<int64_t>(ctx->sm_count, (n * LZ_TPR + LZ_THREADS - 1) / LZ_THREADS);
     DVec<double> V3, W, alpha, beta, part, scr, out;
+    DVec<unsigned long long> bar;  // [0] wait expiries, [1] the grid's arrivals
     V3.alloc(ctx, (size_t)2 * n);
     W.alloc(ctx, n);
-    alpha.alloc(ctx, ldv);
-    beta.alloc(ctx, ldv);
-    part.alloc(ctx, 2 * (size_t)LZ_BLOCKS);
-    scr.alloc(ctx, 12 * (size_t)ldv);
+    alpha.alloc(ctx, mmax + 1);
+    beta.alloc(ctx, mmax + 1);
+    part.alloc(ctx, std::max<size_t>(2 * (size_t)grid, 304));
+    scr.alloc(ctx, 8 * (size_t)(mmax + 1));
     out.alloc(ctx, 4);
-    double *v = V3.data(), *vprev = V3.data() + n, *dot = part.data(), *nrm = part.data() + LZ_BLOCKS;
+    bar.alloc(ctx, 2);
+    double *v = V3.data(), *vprev = V3.data() + n;
     // v_prev enters the first step multiplied by beta_{-1} = 0: it must hold numbers (0 * NaN is NaN,
     // and pool memory keeps whatever it held before)
     k_zero<<<nblk(2 * n), 256, 0, st>>>(V3.data(), 2 * n);
     MBL_LAUNCH_CHECK();
     k_random_block<<<nblk(n), 256, 0, st>>>(n, 1, 0xB0B5EEDull, v, 1, 0);
     MBL_LAUNCH_CHECK();
-    k_lanczos_norm_part<<<LZ_BLOCKS, 256, 0, st>>>(n, v, nrm);
+    k_lanczos_norm_part<<<304, 256, 0, st>>>(n, v, part.data());
     MBL_LAUNCH_CHECK();
-    k_normalize_first<<<LZ_BLOCKS, 256, 0, st>>>(n, v, 1, nrm, LZ_BLOCKS);
+    k_normalize_first<<<304, 256, 0, st>>>(n, v, 1, part.data(), 304);
     MBL_LAUNCH_CHECK();
+    smem_limit((const void *)k_tridiag_extremes, 2 * LZ_MAX * sizeof(double));
     double lo = 0, hi = 0;
     bool done = false;
-    for (int j = 0; j < mmax && !done; ++j) {
-        // w = H v; alpha_j = v^T (w - beta_{j-1} v_prev); w <- w - beta_{j-1} v_prev - alpha_j v;
-        // beta_j = |w|; v_prev <- w / beta_j, then the roles of v and v_prev swap
-        launch_spmv(sec, 0.0, v, 1, 1, W.data(), 1, 1, 1, st);
-        k_lz_dot<<<LZ_BLOCKS, 256, 0, st>>>(n, j, v, vprev, W.data(), beta.data(), dot);
-        MBL_LAUNCH_CHECK();
-        k_lz_update<<<LZ_BLOCKS, 256, 0, st>>>(n, j, v, vprev, W.data(), dot, alpha.data(), beta.data(), nrm);
-        MBL_LAUNCH_CHECK();
-        k_lz_scale<<<LZ_BLOCKS, 256, 0, st>>>(n, j, W.data(), nrm, beta.data(), vprev);
-        MBL_LAUNCH_CHECK();
-        std::swap(v, vprev);
-        const int m = j + 1;
+    for (int j = 0; j < mmax && !done;) {
         // convergence checks every 16 steps from m = 32: a check costs a bisection of T on one CTA,
         // several times the Lanczos steps it could save
-        if ((m >= 32 && m % 16 == 0) || m == mmax) {
-            k_tridiag_extremes<<<1, 64, 0, st>>>(m, alpha.data(), beta.data(), scr.data(), out.data());
+        const int steps = std::min(mmax - j, j == 0 ? 32 : 16 - j % 16);
+        MBL_CUDA(cudaMemsetAsync(bar.data(), 0, 2 * sizeof(unsigned long long), st));
+        {
+            int64_t n_ = n;
+            const int64_t *rp = sec->rowptr.data();
+            const int32_t *cl = sec->col.data();
+            const double *vl = sec->val.data();
+            double *u = W.data(), *al = alpha.data(), *be = beta.data(), *pt = part.data();
+            unsigned int *bc = reinterpret_cast<unsigned int *>(bar.data() + 1);
+            unsigned long long *er = bar.data();
+            int steps_ = steps;
+            void *args[] = {&n_, &rp, &cl, &vl, &j, &steps_, &v, &vprev, &u, &al, &be, &pt, &bc, &er};
+            MBL_CUDA(cudaLaunchCooperativeKernel((const void *)k_lz_steps, dim3(grid), dim3(LZ_THREADS), args, 0, st));
             MBL_LAUNCH_CHECK();
-            double h[4], bj;
-            MBL_CUDA(cudaMemcpyAsync(h, out.data(), 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
-            MBL_CUDA(cudaMemcpyAsync(&bj, beta.data() + j, sizeof(double), cudaMemcpyDeviceToHost, st));
-            MBL_CUDA(cudaStreamSynchronize(st));
-            lo = h[0];
-            hi = h[1];
-            double hn = std::max(std::fabs(lo), std::fabs(hi));
-            if ((std::fabs(bj * h[2]) <= 1e-13 * hn && std::fabs(bj * h[3]) <= 1e-13 * hn) || bj <= 1e-14 * hn) done = true;
         }
+        j += steps;
+        const int m = j;
+        k_tridiag_extremes<<<1, 64, 2 * LZ_MAX * sizeof(double), st>>>(m, alpha.data(), beta.data(), scr.data(), out.data());
+        MBL_LAUNCH_CHECK();
+        double h[4], bj;
+        unsigned long long expired = 0;
+        MBL_CUDA(cudaMemcpyAsync(h, out.data(), 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+        MBL_CUDA(cudaMemcpyAsync(&bj, beta.data() + m - 1, sizeof(double), cudaMemcpyDeviceToHost, st));
+        MBL_CUDA(cudaMemcpyAsync(&expired, bar.data(), sizeof(expired), cudaMemcpyDeviceToHost, st));
+        MBL_CUDA(cudaStreamSynchronize(st));
+        if (expired) fail(MBL_ERR_TIMEOUT, "a grid-wide wait of the extremal Lanczos steps expired");
+        lo = h[0];
+        hi = h[1];
+        const double hn = std::max(std::fabs(lo), std::fabs(hi));
+        if ((std::fabs(bj * h[2]) <= 1e-13 * hn && std::fabs(bj * h[3]) <= 1e-13 * hn) || bj <= 1e-14 * hn) done = true;
     }
     if (!done) fail(MBL_ERR_NOT_CONVERGED, "extremal Lanczos did not converge");
     sec->emin = lo;
