@@ -281,16 +281,7 @@ __device__ __forceinline__ float pdiv(float u, float d) {
     if (!(fabsf(d) > 1e-30f && fabsf(d) < 1e30f && fabsf(q) < 1e30f && (fabsf(q) > 1e-30f || u == 0.0f))) return u / d;
     return __fmaf_rn(__fmaf_rn(-q, d, u), r, q);
 }
-__device__ __forceinline__ double pdiv(double u, double d) {
-    const float df = (float)d;
-    if (!(fabsf(df) > 1e-30f && fabsf(df) < 1e30f)) return u / d;
-    double r = (double)(1.0f / df);
-    r = fma(fma(-d, r, 1.0), r, r);
-    r = fma(fma(-d, r, 1.0), r, r);
-    const double q = u * r;
-    const double l = fma(fma(-q, d, u), r, q);
-    return fabs(q) < 1e300 ? l : u / d;  // (also infinities and NaN)
-}
+__device__ __forceinline__ double pdiv(double u, double d) { return fx_div(u, d); }
 
 // LDL^T of a panel's w x w diagonal block with symmetric 1x1 pivoting, 256 threads.  The whole block
 // (both triangles) is kept in registers: thread (r, h) holds row r, columns [16 h, 16 h + 16).  Rows are
@@ -527,7 +518,8 @@ __global__ void __launch_bounds__(TRSM_THREADS) k_panel_trsm(const PanelDesc *de
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const int t = 16 * kb + 2 * q + (e & 1) + 8 * (e >> 1);
-                            y[e] = fx_bytes(op ? x[t] : x[t] * Dinv[t], sg * hexp[t], E);
+                            const double v = op ? x[t] : x[t] * Dinv[t];
+                            y[e] = fx_bytes(v, fx_exp(v, sg * hexp[t]), E);
                         }
 #pragma unroll
                         for (int i = 0; i < FX_ND; ++i) {
@@ -1913,7 +1905,7 @@ void Factorization::allocate(bool lean_arena) {
     } else {
         gpk.alloc(ctx, (size_t)std::max<int64_t>(pl.sg_elems, 1) * es);
     }
-    scnt.alloc(ctx, std::max<size_t>(pl.sdescs.size() * SUBS, 1));
+    scnt.alloc(ctx, std::max<size_t>(pl.sdescs.size() * BWD_CHUNKS, 1));
     dfcnt.alloc(ctx, (size_t)4 * pl.ns + 2);
     tma = false;
     if (prec == MBL_PREC_FP32 && tc_mode != 0 && pl.wscratch_elems > 0) {
@@ -1922,7 +1914,7 @@ void Factorization::allocate(bool lean_arena) {
         pieces.alloc(ctx, (size_t)(2 * std::max<int64_t>(w_off, 1)));
         tma = true;
     }
-    MBL_CUDA(cudaMemset(scnt.data(), 0, std::max<size_t>(pl.sdescs.size() * SUBS, 1) * sizeof(unsigned int)));
+    MBL_CUDA(cudaMemset(scnt.data(), 0, scnt.size() * sizeof(unsigned int)));
 }
 
 void reset_solve_counters(Factorization &fz, cudaStream_t st) {

@@ -5,8 +5,8 @@
 // [-128, 127].  Digits are exact in FP16, and a sum of products of digits stays an integer below 2^24, exact
 // in the tensor core's FP32 accumulator (the error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012, with
 // integer slices).  The products of digit i of one factor and digit j of the other are kept for i + j <= 8
-// (43 of 64): what is left out is of the size of the splittings' own 2^-63 of a scale, so that a term loses
-// 2^-62 of the product of the two scales, where FP64 arithmetic loses 2^-53 of the term: terms as small as 2^-9
+// (43 of 64): what is left out is of the size of the splittings' own 2^-62 of a scale, so that a term loses
+// 2^-61 of the product of the two scales, where FP64 arithmetic loses 2^-53 of the term: terms as small as 2^-8
 // of the largest keep FP64's accuracy, and a sum's error stays that of its largest terms.  The digit sums A_l
 // (l = i + j) are put together in integers:
 //   sum x y = (hi 2^40 + lo) 2^48 on the scale 2^-124, hi = sum_{l<4} A_l 256^(3-l), lo = sum_{l>=4} A_l 256^(8-l),
@@ -26,40 +26,32 @@ constexpr int FX_NOZERO = -(1 << 16);    // exponent of a zero
 constexpr int FX_BAD = 1 << 19;          // exponents from here on: an infinity or a NaN is among the numbers
 
 // biased exponent of v with an extra power of two e: |v| 2^e < 2^(result - 1022); FX_NOZERO for zero
-// (denormals count as zero: 2^-1022 is no size a sum here is accurate to)
+// (denormals count as zero: 2^-1022 is no size a sum here is accurate to); from FX_BAD / 2 on for infinities, NaN
+// and an e of FX_BAD
 __device__ __forceinline__ int fx_exp(double v, int e) {
     const int b = (__double2hiint(v) >> 20) & 0x7ff;
-    if (e >= FX_BAD / 2) return FX_BAD;
     return b == 0 ? FX_NOZERO : (b == 0x7ff ? FX_BAD : b + e);
 }
 
-// rint(v 2^e 2^(62 - (E - 1022))) + the bias that makes its base-256 digits' bytes d + 128; E: the largest
-// fx_exp of the block
-__device__ __forceinline__ uint64_t fx_bytes(double v, int e, int E) {
-    const uint64_t u = (uint64_t)__double_as_longlong(v);
-    const int b = (int)(u >> 52) & 0x7ff;
-    uint64_t m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
-    const int sh = 9 - (E - (b + e));
-    if (b == 0 || b == 0x7ff || sh < -53) m = 0;
-    else if (sh >= 0) m <<= sh;
-    else m = (m + (1ull << (-sh - 1))) >> -sh;
-    return 0x8080808080808080ull + (v < 0.0 ? (uint64_t)0 - m : m);
+// v on the scale 2^(E - 1022) (ev = fx_exp of v, E the block's largest) as a 62-bit integer, its magnitude
+// truncated, plus the bias that makes its base-256 digits' bytes d + 128
+__device__ __forceinline__ uint64_t fx_bytes(double v, int ev, int E) {
+    const int s = E - ev;
+    const uint64_t m = (((uint64_t)__double_as_longlong(v) << 9) & 0x1fffffffffffffffull) | 0x2000000000000000ull;
+    const uint64_t x = s < 64 && ev > FX_NOZERO / 2 ? m >> s : 0;
+    return __double2hiint(v) < 0 ? 0x8080808080808080ull - x : 0x8080808080808080ull + x;
 }
 
 // A block whose numbers span more than 2^FX_SPAN is taken in several passes: a number smaller than that share of
 // the scale keeps what its digits left out (and the others are done), so that every number counts with a
-// relative error below 2^-(63 - FX_SPAN) = 2^-43 whatever stands beside it.
+// relative error below 2^-(62 - FX_SPAN) = 2^-42 whatever stands beside it.
 constexpr int FX_SPAN = 20;
 
-// fx_bytes, and v becomes what the next pass takes
-__device__ __forceinline__ uint64_t fx_take(double &v, int e, int E, bool again) {
-    const uint64_t y = fx_bytes(v, e, E);
-    if (again) {
-        const int b = fx_exp(v, e);
-        const int64_t x = (int64_t)(y - 0x8080808080808080ull);
-        v = b != FX_NOZERO && b < FX_BAD && E - b > FX_SPAN ? v - scalbn((double)x, E - 1084 - e) : 0.0;
-    }
-    return y;
+// what the next pass takes of v, of which y = fx_bytes(v, ev, E) has been taken; e: v's extra power of two
+// (rare: kept out of line)
+static __device__ __noinline__ double fx_rest(double v, uint64_t y, int e, int ev, int E) {
+    const int64_t x = (int64_t)(y - 0x8080808080808080ull);
+    return ev != FX_NOZERO && ev < FX_BAD / 2 && E - ev > FX_SPAN ? v - scalbn((double)x, E - 1084 - e) : 0.0;
 }
 
 // FP16 pair (digits of the bytes selected by sel's nibbles 0 and 2; 0x64 in the others makes 1024 + byte)
@@ -88,16 +80,23 @@ __device__ __forceinline__ void fx_mma(float (&c)[4], const uint32_t (&a)[4], ui
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// exact integer of an accumulator
+// exact integer of an accumulator; the short form for at most 32 terms a digit sum (|a| <= 2^22)
 __device__ __forceinline__ int fx_int(float a) { return __float2int_rn(a); }
+__device__ __forceinline__ int fx_int_short(float a) { return __float_as_int(a + 12582912.0f) - 0x4B400000; }
 
-// hi and lo of one output from its digit sums acc[l][k]
-template <int N>
+// hi and lo of one output from its digit sums acc[l][k]; SHORT: at most 32 terms
+template <bool SHORT, int N>
 __device__ __forceinline__ void fx_collect(const float (&acc)[FX_NL][N], int k, int64_t &hi, int64_t &lo) {
-    hi = ((int64_t)fx_int(acc[0][k]) << 24) + ((int64_t)fx_int(acc[1][k]) << 16) + ((int64_t)fx_int(acc[2][k]) << 8) +
-         fx_int(acc[3][k]);
-    lo = ((int64_t)fx_int(acc[4][k]) << 32) + ((int64_t)fx_int(acc[5][k]) << 24) + ((int64_t)fx_int(acc[6][k]) << 16) +
-         ((int64_t)fx_int(acc[7][k]) << 8) + fx_int(acc[8][k]);
+    int a[FX_NL];
+#pragma unroll
+    for (int l = 0; l < FX_NL; ++l) a[l] = SHORT ? fx_int_short(acc[l][k]) : fx_int(acc[l][k]);
+    hi = (int64_t)a[0] * (1 << 24) + (int64_t)(a[1] * 256 + a[2]) * 256 + a[3];
+    lo = ((int64_t)a[4] << 32) + (int64_t)a[5] * (1 << 24) + (int64_t)(a[6] * 256 + a[7]) * 256 + a[8];
+}
+
+static __device__ __noinline__ double fx_scale(uint64_t m, int e, bool neg) {
+    const double v = scalbn((double)m, e);
+    return neg ? -v : v;
 }
 
 // (hi 2^40 + lo) 2^48 2^(ea - 62) 2^(eb - 62), rounded once: ea, eb the scales' powers of two.  In integers
@@ -113,8 +112,23 @@ __device__ __forceinline__ double fx_value(int64_t hi, int64_t lo, int ea, int e
     m = (m >> 11) + (m >> 10 & 1);  // 53 bits (a carry out of them lands in the exponent)
     const uint64_t sign = x < 0 ? 0x8000000000000000ull : 0ull;
     if (e > -1022 && e < 1023) return __longlong_as_double((int64_t)(sign | (((uint64_t)(e + 1022) << 52) + m)));
-    const double v = scalbn((double)m, e - 52);
-    return x < 0 ? -v : v;
+    return fx_scale(m, e - 52, x < 0);
+}
+
+// -v, and u / d (a reciprocal from FP32 by two Newton steps, the quotient corrected by its residual), with as few
+// instructions on the FP64 pipe as they need
+__device__ __forceinline__ double fx_neg(double v) {
+    return __hiloint2double(__double2hiint(v) ^ (int)0x80000000u, __double2loint(v));
+}
+__device__ __forceinline__ double fx_div(double u, double d) {
+    const float df = (float)d;
+    if (!(fabsf(df) > 1e-30f && fabsf(df) < 1e30f)) return u / d;
+    double r = (double)(1.0f / df);
+    r = fma(fma(-d, r, 1.0), r, r);
+    r = fma(fma(-d, r, 1.0), r, r);
+    const double q = u * r;
+    const double l = fma(fma(-q, d, u), r, q);
+    return fabs(q) < 1e300 ? l : u / d;  // (also infinities and NaN)
 }
 
 }  // namespace mbl

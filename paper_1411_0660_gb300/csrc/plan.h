@@ -55,6 +55,7 @@ struct PanelStep {
 constexpr int RBF = 32;  // rows per CTA of a forward solve step
 constexpr int RBB = 64;   // columns per chunk of a backward solve step; rows per CTA of the G = [M; L21 M] build
 constexpr int RBK = 256;  // rows per CTA of a backward solve step
+constexpr int BWD_CHUNKS = 8;  // most column chunks of a panel in a backward step (arrival counters of a descriptor)
 
 // One solve panel: columns [k0, k0 + w) of a front's fully-summed block (w <= SPW).  M (w x w) is
 // the composite of the factor panels' pivot permutations and unit-lower eliminations restricted

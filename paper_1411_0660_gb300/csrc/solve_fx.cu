@@ -4,8 +4,9 @@
 // x_panel <- G^T [y_panel; -x_below] backward, G = [M; L21 M] packed per 256-column solve panel), with the
 // products of G and a p-wide block formed from integer digits on the FP16 tensor cores (fixed_digits.cuh).
 // In FP64 arithmetic these steps are bound by the two FP64 FMAs a clock and SM: a whole L = 16 job of 43
-// block applications took 244 ms that way and takes 215 ms this way; the unrefined solve's error against a
-// dense 64-bit solve is 0.8 to 0.95 of what it was (geometric means over L = 10 to 14, 24 cases each).
+// block applications took 244 ms that way and takes 165 ms this way; the unrefined solve's error against a
+// dense 64-bit solve is 0.6 to 0.85 of what it was (geometric means over L = 10 to 14, 24 cases each).  Now
+// bound by latency: each step is a short chain of loads, one exchange of scales and some 170 products a warp.
 //
 // Packed form of one panel's G (R x w): column c is scaled by 2^-cex[c] and row r by 2^-rex[r] (powers of
 // two that put every column's, then every row's largest magnitude in [1/2, 1)), the entry becomes eight
@@ -91,9 +92,29 @@ __device__ __forceinline__ int min_over_t(int x) {
     x = min(x, __shfl_xor_sync(0xffffffffu, x, 1));
     return min(x, __shfl_xor_sync(0xffffffffu, x, 2));
 }
-// the smallest exponent leaves zeros out
-__device__ __forceinline__ int min_exp(int m, int e) { return e == FX_NOZERO ? m : min(m, e); }
 constexpr int FX_NOMIN = 1 << 20;
+// exponents ev of v with the powers of two e; largest, and smallest of the nonzero ones, over the lanes t of a group
+__device__ __forceinline__ void exponents(const double (&v)[8], const int (&e)[8], int (&ev)[8], int &em, int &el) {
+    em = FX_NOZERO, el = FX_NOMIN;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        ev[k] = fx_exp(v[k], e[k]);
+        em = max(em, ev[k]);
+        el = ev[k] == FX_NOZERO ? el : min(el, ev[k]);
+    }
+    em = max_over_t(em);
+    el = min_over_t(el);
+}
+// bytes of v on the scale E; with another pass to come v keeps what that takes
+__device__ __forceinline__ void take(double (&v)[8], const int (&e)[8], const int (&ev)[8], int E, bool again,
+                                     uint64_t (&y)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) y[k] = fx_bytes(v[k], ev[k], E);
+    if (again) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = fx_rest(v[k], y[k], e[k], ev[k], E);
+    }
+}
 
 __device__ __forceinline__ uint4 ld_tile(const double *G, int64_t tile, int plane, int lane) {
     return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint32_t *>(G) + tile * FT_WORDS) + plane * 32 +
@@ -111,7 +132,7 @@ __global__ void __launch_bounds__(256) k_fx_colexp(const SolveDesc *sdescs, cons
     if (c < d.w)
         for (int r = lane; r < R; r += 32) e = max(e, fx_exp(g[r], 0));
     for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if (lane == 0) cex[d.xcol + c] = e <= FX_NOZERO || e >= FX_BAD ? 0 : e - 1022;
+    if (lane == 0) cex[d.xcol + c] = e <= FX_NOZERO || e >= FX_BAD / 2 ? 0 : e - 1022;
 }
 
 // Row scales and digits of one 32-row block of a panel.
@@ -132,7 +153,7 @@ __global__ void __launch_bounds__(256) k_fx_pack(const SolveDesc *sdescs, const 
 #pragma unroll
         for (int i = 1; i < 8; ++i) e = max(e, wmax[i][lane]);
         rmax[lane] = e;
-        rex[d.xrow + r0 + lane] = e >= FX_BAD ? FX_BAD : (e <= FX_NOZERO ? 0 : e - 1022);
+        rex[d.xrow + r0 + lane] = e >= FX_BAD / 2 ? FX_BAD : (e <= FX_NOZERO ? 0 : e - 1022);
     }
     __syncthreads();
     const int gl = lane >> 2, t = lane & 3;
@@ -148,7 +169,8 @@ __global__ void __launch_bounds__(256) k_fx_pack(const SolveDesc *sdescs, const 
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = 4 * gl + i;
-                y[k][i] = fx_bytes(c < w && r0 + r < R ? g[(int64_t)c * ld + r] : 0.0, ce, E[i]);
+                const double v = c < w && r0 + r < R ? g[(int64_t)c * ld + r] : 0.0;
+                y[k][i] = fx_bytes(v, fx_exp(v, ce), E[i]);
             }
         }
         uint4 *o = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(out) +
@@ -228,15 +250,8 @@ __global__ void __launch_bounds__(256, 2)
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             double v = 0.0;
             for (bool again = true; again;) {  // one pass unless z spans more than 2^FX_SPAN
-                int em = FX_NOZERO, el = FX_NOMIN;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int e = fx_exp(z[k], ce[k]);
-                    em = max(em, e);
-                    el = min_exp(el, e);
-                }
-                em = max_over_t(em);
-                el = min_over_t(el);
+                int ev[8], em, el;
+                exponents(z, ce, ev, em, el);
                 if (t == 0) {
                     smax[wp][g] = em;
                     smin[wp][g] = el;
@@ -250,11 +265,10 @@ __global__ void __launch_bounds__(256, 2)
                     Eo = max(Eo, smax[i][oq]);
                 }
                 // (every warp holds all eight right-hand sides: the same answer in each)
-                again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+                again = __any_sync(0xffffffffu, E < FX_BAD / 2 && E - El > FX_SPAN);
                 if (wp < nw) {
                     uint64_t y[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) y[k] = fx_take(z[k], ce[k], E, again);
+                    take(z, ce, ev, E, again, y);
                     float acc[2][FX_NL][4];
 #pragma unroll
                     for (int m = 0; m < 2; ++m)
@@ -262,11 +276,15 @@ __global__ void __launch_bounds__(256, 2)
                         for (int l = 0; l < FX_NL; ++l)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) acc[m][l][k] = 0.f;
-#pragma unroll
+                    // (rolled, as the column blocks of the backward steps: straight code this long waits on its fetch)
+#pragma unroll 1
                     for (int kb = 0; kb < 2; ++kb) {
                         if (32 * wp + 16 * kb >= w) break;
+                        uint64_t yk[8];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) yk[k] = kb ? y[4 + k] : y[k];
                         uint32_t bq[FX_ND][2];
-                        fx_b_all(y, kb, bq);
+                        fx_b_all(yk, 0, bq);
                         const uint4 *tl = tiles + (size_t)(2 * wp + kb) * (FT_WORDS / 4) + lane;
                         tile_forward([&](int i) { return tl[i * 32]; }, bq, acc);
                     }
@@ -276,7 +294,7 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             int64_t hi, lo;
-                            fx_collect(acc[m], k, hi, lo);
+                            fx_collect<true>(acc[m], k, hi, lo);
                             const int row = 4 * g + 2 * m + (k >> 1), qq = 2 * t + (k & 1);
                             rw[qq * 32 + row] = hi;
                             rw[256 + qq * 32 + row] = lo;
@@ -298,7 +316,7 @@ __global__ void __launch_bounds__(256, 2)
                     // a panel row is final here: also its diagonal-scaled value for the backward sweep
                     const int64_t gr = (int64_t)sn_start[s] + k0 + rr;
                     J.Zs[(zb + rr) * p + q0 + oq] = v;
-                    J.yfw[gr * p + q0 + oq] = v / dg;
+                    J.yfw[gr * p + q0 + oq] = fx_div(v, dg);
                 } else {
                     J.Z[(zb + rr) * p + q0 + oq] = zold - v;
                 }
@@ -364,19 +382,11 @@ __global__ void __launch_bounds__(256) k_fx_fwd_narrow(const SolveDesc *sdescs, 
             }
         double sum[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
         for (bool again = true; again;) {  // one pass unless z spans more than 2^FX_SPAN
-            int E = FX_NOZERO, El = FX_NOMIN;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int e = fx_exp(z[k], ce[k]);
-                E = max(E, e);
-                El = min_exp(El, e);
-            }
-            E = max_over_t(E);
-            El = min_over_t(El);
-            again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+            int ev[8], E, El;
+            exponents(z, ce, ev, E, El);
+            again = __any_sync(0xffffffffu, E < FX_BAD / 2 && E - El > FX_SPAN);
             uint64_t y[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) y[k] = fx_take(z[k], ce[k], E, again);
+            take(z, ce, ev, E, again, y);
             float acc[2][FX_NL][4];
 #pragma unroll
             for (int m = 0; m < 2; ++m)
@@ -398,7 +408,7 @@ __global__ void __launch_bounds__(256) k_fx_fwd_narrow(const SolveDesc *sdescs, 
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     int64_t hi, lo;
-                    fx_collect(acc[m], k, hi, lo);
+                    fx_collect<true>(acc[m], k, hi, lo);
                     sum[m][k] += fx_value(hi, lo, re[2 * m + (k >> 1)], ((k & 1) ? e1 : e0) - 1022);
                 }
         }
@@ -411,7 +421,7 @@ __global__ void __launch_bounds__(256) k_fx_fwd_narrow(const SolveDesc *sdescs, 
                 const double v = sum[m][k];
                 if (rr < w) {
                     J.Zs[(zb + rr) * p + q] = v;
-                    J.yfw[(g0 + rr) * p + q] = v / dg[i];
+                    J.yfw[(g0 + rr) * p + q] = fx_div(v, dg[i]);
                 } else {
                     J.Z[(zb + rr) * p + q] = zold[i][k & 1] - v;
                 }
@@ -421,162 +431,126 @@ __global__ void __launch_bounds__(256) k_fx_fwd_narrow(const SolveDesc *sdescs, 
 
 // ---- backward ---------------------------------------------------------------------------------------
 
+constexpr int BC = 32;                    // columns of a CTA: more and smaller than the FP32 steps' 64
+constexpr int BCB = BC / FT_COLS;
 constexpr int BW_RB = RBK / FT_ROWS + 1;  // most row blocks of one tile (the first may start inside a block)
-constexpr size_t BWD_TILE = (size_t)BW_RB * (RBB / FT_COLS) * FT_WORDS * 4;
-constexpr size_t BWD_SMEM = BWD_TILE + (size_t)8 * 2 * 8 * RBB * 8;  // and the warps' sums [warp][hi, lo][q][column]
+constexpr size_t BWD_TILE = (size_t)BW_RB * BCB * FT_WORDS * 4;
+constexpr size_t BWD_SMEM = BWD_TILE + (size_t)8 * 2 * 8 * BC * 8;  // and the warps' sums [warp][hi, lo][q][column]
 
-// Copies row blocks [rb0, rb0 + nrb) of the 64 columns from 16 cb0 on.
+// Copies row blocks [rb0, rb0 + nrb) of the BC columns from 16 cb0 on.
 __device__ __forceinline__ void bwd_issue(uint4 *tiles, const double *G, const SolveDesc &d, int rb0, int nrb, int cb0) {
-    const int ncb = (d.w + FT_COLS - 1) / FT_COLS, nc = min(RBB / FT_COLS, ncb - cb0), per = nc * (FT_WORDS / 4);
+    const int ncb = (d.w + FT_COLS - 1) / FT_COLS, nc = min(BCB, ncb - cb0), per = nc * (FT_WORDS / 4);
     const uint32_t *src = reinterpret_cast<const uint32_t *>(G) + (d.xoff + (int64_t)rb0 * ncb + cb0) * FT_WORDS;
-    for (int u = threadIdx.x; u < nrb * per; u += 256) {
-        const int r = u / per, v = u - r * per;
-        cp_async16(tiles + (size_t)r * (RBB / FT_COLS) * (FT_WORDS / 4) + v,
-                   reinterpret_cast<const uint4 *>(src + (int64_t)r * ncb * FT_WORDS) + v);
-    }
+    for (int r = 0; r < nrb; ++r)
+        for (int u = threadIdx.x; u < per; u += 256)
+            cp_async16(tiles + (size_t)r * BCB * (FT_WORDS / 4) + u,
+                       reinterpret_cast<const uint4 *>(src + (int64_t)r * ncb * FT_WORDS) + u);
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Digit sums of the tiles' columns for right-hand sides q0 .. q0 + 7, added over the CTA: thread o returns
-// the products of outputs o and o + 256 (column c = o % RBB, q = q0 + o / RBB).  vf(r, q): entry of v at row r
-// (relative to the first row block), zero outside.  rexp: the rows' scales, from the first row block on.
+// Products of the tiles' columns with right-hand sides q0 .. q0 + 7, added over the CTA: thread o returns output o
+// (column c = o % BC, q = q0 + o / BC).  Eight row blocks at a time, one a warp, on one scale of v.  vf(r, q): entry of
+// v at row r (relative to the first row block), zero outside.  rexp: the rows' scales, from the first row block on.
 template <class VF>
-__device__ __forceinline__ void bwd_products(uint4 *tiles, const SolveDesc &d, int nrb, int cb0, const int32_t *rexp,
-                                             const int32_t *cexp, int q0, int p, VF &&vf, double out[2]) {
+__device__ __forceinline__ double bwd_products(uint4 *tiles, const SolveDesc &d, int nrb, int cb0, const int32_t *rexp,
+                                               const int32_t *cexp, int q0, int p, VF &&vf) {
     __shared__ int smax[8][8], smin[8][8];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int nc = min(RBB / FT_COLS, (d.w + FT_COLS - 1) / FT_COLS - cb0);
-    // (at most two row blocks a warp: wp and, of nine, the last one for warp 0)
-    double v[2][8];
-    int re[2][8];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
+    const int nc = min(BCB, (d.w + FT_COLS - 1) / FT_COLS - cb0);
+    const int oc = threadIdx.x % BC, oq = threadIdx.x / BC;
+    const int ce = 16 * cb0 + oc < d.w ? cexp[16 * cb0 + oc] : 0;
+    int64_t *red = reinterpret_cast<int64_t *>(tiles) + BWD_TILE / 8, *rw = red + (size_t)wp * 16 * BC;
+    double out = 0.0;
+#pragma unroll 1
+    for (int r8 = 0; r8 < nrb; r8 += 8) {
+        const int rbk = r8 + wp, nwp = min(8, nrb - r8);
+        double v[8];
+        int re[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const int rbk = wp + 8 * h, r = 32 * rbk + 8 * t + 2 * (k >> 2) + (k & 1) + 4 * ((k >> 1) & 1);
+            const int r = 32 * rbk + 8 * t + 2 * (k >> 2) + (k & 1) + 4 * ((k >> 1) & 1);
             const bool in = rbk < nrb && q0 + g < p;
-            v[h][k] = in ? vf(r, q0 + g) : 0.0;
-            re[h][k] = in ? rexp[r] : 0;
+            v[k] = in ? vf(r, q0 + g) : 0.0;
+            re[k] = in ? rexp[r] : 0;
         }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    out[0] = out[1] = 0.0;
-    for (bool again = true; again;) {  // one pass unless v spans more than 2^FX_SPAN
-        int em = FX_NOZERO, el = FX_NOMIN;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int e = fx_exp(v[h][k], re[h][k]);
-                em = max(em, e);
-                el = min_exp(el, e);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        for (bool again = true; again;) {  // one pass unless v spans more than 2^FX_SPAN
+            int ev[8], em, el;
+            exponents(v, re, ev, em, el);
+            if (t == 0) {
+                smax[wp][g] = em;
+                smin[wp][g] = el;
             }
-        em = max_over_t(em);
-        el = min_over_t(el);
-        if (t == 0) {
-            smax[wp][g] = em;
-            smin[wp][g] = el;
-        }
-        __syncthreads();
-        int E = smax[0][g], El = smin[0][g];
+            __syncthreads();
+            int E = smax[0][g], El = smin[0][g];
 #pragma unroll
-        for (int i = 1; i < 8; ++i) {
-            E = max(E, smax[i][g]);
-            El = min(El, smin[i][g]);
-        }
-        // (every warp holds all eight right-hand sides: the same answer in each)
-        again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
-        int64_t hi[RBB / FT_COLS][4], lo[RBB / FT_COLS][4];
-#pragma unroll
-        for (int cb = 0; cb < RBB / FT_COLS; ++cb)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) hi[cb][k] = lo[cb][k] = 0;
+            for (int i = 1; i < 8; ++i) {
+                E = max(E, smax[i][g]);
+                El = min(El, smin[i][g]);
+            }
+            // (every warp holds all eight right-hand sides: the same answer in each)
+            again = __any_sync(0xffffffffu, E < FX_BAD / 2 && E - El > FX_SPAN);
+            if (rbk < nrb) {
+                uint32_t b[2][FX_ND][2];
+                {
+                    uint64_t y[8];
+                    take(v, re, ev, E, again, y);
+                    fx_b_all(y, 0, b[0]);
+                    fx_b_all(y, 1, b[1]);
+                }
+                // (rolled, as the k blocks of the forward step: straight code this long waits on its fetch)
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            const int rbk = wp + 8 * h;
-            if (rbk >= nrb) break;
-            uint32_t b[2][FX_ND][2];
-            {
-                uint64_t y[8];
+                for (int cb = 0; cb < nc; ++cb) {
+                    float acc[FX_NL][4];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    double vk = h ? v[1][k] : v[0][k];
-                    y[k] = fx_take(vk, h ? re[1][k] : re[0][k], E, again);
-                    if (h) v[1][k] = vk;
-                    else v[0][k] = vk;
-                }
-                fx_b_all(y, 0, b[0]);
-                fx_b_all(y, 1, b[1]);
-            }
+                    for (int l = 0; l < FX_NL; ++l)
 #pragma unroll
-            for (int cb = 0; cb < RBB / FT_COLS; ++cb) {
-                if (cb >= nc) break;
-                float acc[FX_NL][4];
+                        for (int k = 0; k < 4; ++k) acc[l][k] = 0.f;
+                    const uint4 *tl = tiles + (size_t)(rbk * BCB + cb) * (FT_WORDS / 4) + lane;
+                    tile_backward([&](int i) { return tl[i * 32]; }, b, acc);
 #pragma unroll
-                for (int l = 0; l < FX_NL; ++l)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[l][k] = 0.f;
-                const uint4 *tl = tiles + (size_t)(rbk * (RBB / FT_COLS) + cb) * (FT_WORDS / 4) + lane;
-                tile_backward([&](int i) { return tl[i * 32]; }, b, acc);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    int64_t a, c;
-                    fx_collect(acc, k, a, c);
-                    hi[cb][k] += a;
-                    lo[cb][k] += c;
+                    for (int k = 0; k < 4; ++k) {
+                        int64_t hi, lo;
+                        fx_collect<true>(acc, k, hi, lo);
+                        int64_t *o = rw + (2 * t + (k & 1)) * BC + 16 * cb + g + 8 * (k >> 1);
+                        o[0] = hi;
+                        o[8 * BC] = lo;
+                    }
                 }
             }
-        }
-        int64_t *red = reinterpret_cast<int64_t *>(tiles) + BWD_TILE / 8;
-        const int nwp = min(8, nrb);
-        if (wp < nwp) {
-            int64_t *rw = red + (size_t)wp * 16 * RBB;
-#pragma unroll
-            for (int cb = 0; cb < RBB / FT_COLS; ++cb)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int c = 16 * cb + g + 8 * (k >> 1), q = 2 * t + (k & 1);
-                    rw[q * RBB + c] = hi[cb][k];
-                    rw[8 * RBB + q * RBB + c] = lo[cb][k];
-                }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, c = o % RBB, q = o / RBB;
-            int64_t a = 0, b = 0;
+            __syncthreads();
+            int64_t hi = 0, lo = 0;
             for (int i = 0; i < nwp; ++i) {
-                a += red[(size_t)i * 16 * RBB + q * RBB + c];
-                b += red[(size_t)i * 16 * RBB + 8 * RBB + q * RBB + c];
+                hi += red[(size_t)i * 16 * BC + oq * BC + oc];
+                lo += red[(size_t)i * 16 * BC + 8 * BC + oq * BC + oc];
             }
-            int Eo = smax[0][q];
+            int Eo = smax[0][oq];
 #pragma unroll
-            for (int i = 1; i < 8; ++i) Eo = max(Eo, smax[i][q]);
-            if (16 * cb0 + c < d.w) out[h] += fx_value(a, b, cexp[16 * cb0 + c], Eo - 1022);
+            for (int i = 1; i < 8; ++i) Eo = max(Eo, smax[i][oq]);
+            if (16 * cb0 + oc < d.w) out += fx_value(hi, lo, ce, Eo - 1022);
+            __syncthreads();  // red, smax and smin are used again
         }
-        __syncthreads();  // red, smax and smin are used again
     }
+    return out;
 }
 
-// Start of the backward sweep of one level: see k_bwd_step in factor.cu (same blocks, same partial sums).
-// Block b >= 1 of a panel takes an even share of the 32-row blocks from the contribution block's first row on
-// (rows of the front's later panels in the first of them meet a zero v).
-template <int PB>
-__global__ void __launch_bounds__(256) k_fx_bwd_step(const SolveDesc *sdescs, const int32_t *blk_desc,
-                                                     const int64_t *zo, const int32_t *nc, const int32_t *sn_start,
-                                                     const int64_t *rows_off, const int32_t *rows,
-                                                     const SolveBufs<double> *jb, int64_t cnt_off, int p,
-                                                     LaunchTrace *tr) {
+// Start of the backward sweep of one level: see k_bwd_step in factor.cu (same row blocks; BC columns).  Block
+// b >= 1 of a panel takes an even share of the 32-row blocks from the contribution block's first row on (rows
+// of the front's later panels in the first of them meet a zero v).  Partial sums: [block][column chunk][q][column].
+__global__ void __launch_bounds__(256, 2)
+    k_fx_bwd_step(const SolveDesc *sdescs, const int32_t *blk_desc, const int64_t *zo, const int32_t *nc,
+                  const int32_t *sn_start, const int64_t *rows_off, const int32_t *rows, const SolveBufs<double> *jb,
+                  int64_t cnt_off, int p, int pad, LaunchTrace *tr) {
     TraceScope trace_scope(tr);
     extern __shared__ __align__(16) unsigned char smraw[];
     uint4 *tiles = reinterpret_cast<uint4 *>(smraw);
     __shared__ int s_last;
     __shared__ const double *vrow[BW_RB * FT_ROWS];  // row of v (null: zero)
-    __shared__ double vsgn[BW_RB * FT_ROWS];
     const SolveBufs<double> J = jb[blockIdx.z];
     unsigned int *cnt = J.cnt + cnt_off;
     const int di = blk_desc[blockIdx.x];
     const SolveDesc d = sdescs[di];
-    const int cc = blockIdx.y * RBB;
+    const int cc = blockIdx.y * BC;
     if (cc >= d.w) {
         pdl_wait();
         return;
@@ -589,7 +563,7 @@ __global__ void __launch_bounds__(256) k_fx_bwd_step(const SolveDesc *sdescs, co
         rb0 = f0 + (b - 1) * per;
         nrb = max(0, min(per, n32 - (b - 1) * per));
     }
-    const int wc = min(RBB, w - cc);
+    const int wc = min(BC, w - cc);
     const int64_t zb = zo[s] + k0;
     if (nrb > 0) bwd_issue(tiles, J.G, d, rb0, nrb, cc / FT_COLS);
     for (int i = threadIdx.x; i < BW_RB * FT_ROWS; i += 256) {
@@ -600,63 +574,69 @@ __global__ void __launch_bounds__(256) k_fx_bwd_step(const SolveDesc *sdescs, co
             else if (rr >= cb0 && rr < R) sp = J.y + (int64_t)rows[rows_off[s] + k0 + rr] * p;
         }
         vrow[i] = sp;
-        vsgn[i] = b == 0 ? 1.0 : -1.0;
     }
     __syncthreads();
     pdl_wait();
     pdl_trigger();
-    const int64_t tile = (int64_t)RBB * PB;
-    double *out = J.P + ((d.offk_l + b) * SUBS + blockIdx.y) * tile;
+    const int64_t tile = (int64_t)BC * pad;
+    double *out = J.P + ((d.offk_l + b) * (SPW / BC) + blockIdx.y) * tile;
     double *zsp = J.Zs + (zb + cc) * p;
     double *xp = k0 + w >= ncs ? J.y + ((int64_t)sn_start[s] + k0 + cc) * p : nullptr;
-    for (int q0 = 0; q0 < PB; q0 += 8) {
-        double o2[2];
-        bwd_products(tiles, d, nrb, cc / FT_COLS, J.rex + d.xrow + rb0 * FT_ROWS, J.cex + d.xcol, q0, p,
-                     [&](int r, int q) { return vrow[r] ? vsgn[r] * __ldcg(vrow[r] + q) : 0.0; }, o2);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
-            if (nb == 1) {
-                if (c < wc && q < p) {
-                    zsp[c * p + q] = o2[h];
-                    if (xp) xp[c * p + q] = o2[h];
-                }
-            } else {
-                out[q * RBB + c] = o2[h];
-            }
+    const int c = threadIdx.x % BC;
+    for (int q0 = 0; q0 < p; q0 += 8) {
+        const double o = bwd_products(tiles, d, nrb, cc / FT_COLS, J.rex + d.xrow + rb0 * FT_ROWS, J.cex + d.xcol, q0, p,
+                                      [&](int r, int q) {
+                                          const double x = vrow[r] ? __ldcg(vrow[r] + q) : 0.0;
+                                          return b == 0 ? x : fx_neg(x);
+                                      });
+        const int q = q0 + threadIdx.x / BC;
+        if (nb > 1) {
+            out[q * BC + c] = o;
+        } else if (c < wc && q < p) {
+            zsp[c * p + q] = o;
+            if (xp) xp[c * p + q] = o;
         }
     }
     if (nb == 1) return;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned int prev = atomicAdd(&cnt[(size_t)di * SUBS + blockIdx.y], 1u);
+        const unsigned int prev = atomicAdd(&cnt[(size_t)di * (SPW / BC) + blockIdx.y], 1u);
         s_last = prev == (unsigned int)(nb - 1);
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    bwd_finish<double, PB>(J.P + (d.offk_l * SUBS + blockIdx.y) * tile, (int64_t)SUBS * tile, nb, wc, p, zsp, xp,
-                           reinterpret_cast<double *>(smraw));
-    if (threadIdx.x == 0) cnt[(size_t)di * SUBS + blockIdx.y] = 0u;
+    // the last block adds the partial sums in a fixed order
+    const double *src = J.P + (d.offk_l * (SPW / BC) + blockIdx.y) * tile;
+    for (int q = threadIdx.x / BC; q < p; q += 8) {
+        double v = 0.0;
+#pragma unroll 8
+        for (int i = 0; i < nb; ++i) v += __ldcg(src + (int64_t)i * (SPW / BC) * tile + q * BC + c);
+        if (c < wc) {
+            zsp[c * p + q] = v;
+            if (xp) xp[c * p + q] = v;
+        }
+    }
+    if (threadIdx.x == 0) cnt[(size_t)di * (SPW / BC) + blockIdx.y] = 0u;
 }
 
 // Backward update: see k_bwd_update in factor.cu.
-__global__ void __launch_bounds__(256) k_fx_bwd_update(const SolveDesc *sdescs, const int32_t *items, const int64_t *zo,
-                                                       const int32_t *sn_start, const SolveBufs<double> *jb, int p,
-                                                       LaunchTrace *tr) {
+__global__ void __launch_bounds__(256, 2)
+    k_fx_bwd_update(const SolveDesc *sdescs, const int32_t *items, const int64_t *zo, const int32_t *sn_start,
+                    const SolveBufs<double> *jb, int p, LaunchTrace *tr) {
     static_assert(SPW % FT_ROWS == 0, "later panels start on a row block");
     TraceScope trace_scope(tr);
     extern __shared__ __align__(16) unsigned char smraw[];
     uint4 *tiles = reinterpret_cast<uint4 *>(smraw);
     const SolveBufs<double> J = jb[blockIdx.z];
     const SolveDesc di = sdescs[items[2 * blockIdx.x]], dj = sdescs[items[2 * blockIdx.x + 1]];
-    const int cc = blockIdx.y * RBB;
+    const int cc = blockIdx.y * BC;
     if (cc >= di.w) {
         pdl_wait();
         return;
     }
-    const int s = di.front, wc = min(RBB, di.w - cc), wj = dj.w, rb0 = (dj.k0 - di.k0) / FT_ROWS;
+    const int s = di.front, wc = min(BC, di.w - cc), wj = dj.w, rb0 = (dj.k0 - di.k0) / FT_ROWS;
     const int nrb = (wj + FT_ROWS - 1) / FT_ROWS;
     bwd_issue(tiles, J.G, di, rb0, nrb, cc / FT_COLS);
     const int64_t zi = zo[s] + di.k0 + cc, zj = zo[s] + dj.k0;
@@ -664,23 +644,16 @@ __global__ void __launch_bounds__(256) k_fx_bwd_update(const SolveDesc *sdescs, 
     pdl_wait();
     pdl_trigger();
     double *xp = J.y + ((int64_t)sn_start[s] + di.k0 + cc) * p;
+    const int c = threadIdx.x % BC;
     for (int q0 = 0; q0 < p; q0 += 8) {
-        double old[2], o2[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
-            old[h] = c < wc && q < p ? J.Zs[(zi + c) * p + q] : 0.0;
-        }
-        bwd_products(tiles, di, nrb, cc / FT_COLS, J.rex + di.xrow + rb0 * FT_ROWS, J.cex + di.xcol, q0, p,
-                     [&](int r, int q) { return r < wj ? J.Zs[(zj + r) * p + q] : 0.0; }, o2);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
-            if (c < wc && q < p) {
-                const double v = old[h] - o2[h];
-                J.Zs[(zi + c) * p + q] = v;
-                if (fin) xp[c * p + q] = v;
-            }
+        const int q = q0 + threadIdx.x / BC;
+        const bool own = c < wc && q < p;
+        const double old = own ? J.Zs[(zi + c) * p + q] : 0.0;
+        const double o = bwd_products(tiles, di, nrb, cc / FT_COLS, J.rex + di.xrow + rb0 * FT_ROWS, J.cex + di.xcol, q0, p,
+                                      [&](int r, int q_) { return r < wj ? J.Zs[(zj + r) * p + q_] : 0.0; });
+        if (own) {
+            J.Zs[(zi + c) * p + q] = old - o;
+            if (fin) xp[c * p + q] = old - o;
         }
     }
 }
@@ -742,24 +715,16 @@ __global__ void __launch_bounds__(256) k_fx_bwd_narrow(const SolveDesc *sdescs, 
                 v[k] = 0.0;
                 if (r < R && q0 + g < p)
                     v[k] = r < w ? J.yfw[(g0 + r) * p + q0 + g]
-                                 : -(k0 + r < ncs ? J.Zs[(zb + r) * p + q0 + g] : J.y[(int64_t)rowx[k] * p + q0 + g]);
+                                 : fx_neg(k0 + r < ncs ? J.Zs[(zb + r) * p + q0 + g] : J.y[(int64_t)rowx[k] * p + q0 + g]);
             }
             for (bool again = true; again;) {  // one pass unless v spans more than 2^FX_SPAN
-                int E = FX_NOZERO, El = FX_NOMIN;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int e = fx_exp(v[k], re[k]);
-                    E = max(E, e);
-                    El = min_exp(El, e);
-                }
-                E = max_over_t(E);
-                El = min_over_t(El);
-                again = __any_sync(0xffffffffu, E < FX_BAD && E - El > FX_SPAN);
+                int ev[8], E, El;
+                exponents(v, re, ev, E, El);
+                again = __any_sync(0xffffffffu, E < FX_BAD / 2 && E - El > FX_SPAN);
                 uint32_t b[2][FX_ND][2];
                 {
                     uint64_t y[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) y[k] = fx_take(v[k], re[k], E, again);
+                    take(v, re, ev, E, again, y);
                     fx_b_all(y, 0, b[0]);
                     fx_b_all(y, 1, b[1]);
                 }
@@ -776,7 +741,7 @@ __global__ void __launch_bounds__(256) k_fx_bwd_narrow(const SolveDesc *sdescs, 
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         int64_t hi, lo;
-                        fx_collect(acc, k, hi, lo);
+                        fx_collect<true>(acc, k, hi, lo);
                         sum[cb][k] += fx_value(hi, lo, ce[cb][k >> 1], ((k & 1) ? e1 : e0) - 1022);
                     }
                 }
@@ -856,20 +821,15 @@ void fx_backward_level(const Plan &pl, int l, const SolveBufs<double> *jb, unsig
         else two ? narrow(k_fx_bwd_narrow<2, 2>, 2) : narrow(k_fx_bwd_narrow<2, 8>, 8);
         return;
     }
-    auto wide = [&](auto kern) {
-        launch_pdl(kern, dim3((unsigned)pl.lvl_nrbk[l], (pl.lvl_maxw[l] + RBB - 1) / RBB, K), dim3(256), BWD_SMEM, st,
-                   sdl, (const int32_t *)pl.d_lvl_bblk_desc.data() + pl.lvl_bblk0[l], pl.d_sn_zo.data(),
-                   pl.d_sn_nc.data(), pl.d_sn_start.data(), pl.d_sn_rows_off.data(), pl.d_rows.data(), jb,
-                   (int64_t)pl.lvl_d0[l] * SUBS, p, tr);
-    };
-    if (p <= 8) wide(k_fx_bwd_step<8>);
-    else if (p <= 16) wide(k_fx_bwd_step<16>);
-    else wide(k_fx_bwd_step<32>);
+    launch_pdl(k_fx_bwd_step, dim3((unsigned)pl.lvl_nrbk[l], (pl.lvl_maxw[l] + BC - 1) / BC, K), dim3(256), BWD_SMEM, st,
+               sdl, (const int32_t *)pl.d_lvl_bblk_desc.data() + pl.lvl_bblk0[l], pl.d_sn_zo.data(), pl.d_sn_nc.data(),
+               pl.d_sn_start.data(), pl.d_sn_rows_off.data(), pl.d_rows.data(), jb,
+               (int64_t)pl.lvl_d0[l] * (SPW / BC), p, p <= 8 ? 8 : (p <= 16 ? 16 : 32), tr);
 }
 
 void fx_backward_update(const Plan &pl, const BwdUpd &bu, const SolveBufs<double> *jb, unsigned K, int p,
                         LaunchTrace *tr, cudaStream_t st) {
-    launch_pdl(k_fx_bwd_update, dim3((unsigned)bu.nit, SUBS, K), dim3(256), BWD_SMEM, st,
+    launch_pdl(k_fx_bwd_update, dim3((unsigned)bu.nit, SPW / BC, K), dim3(256), BWD_SMEM, st,
                (const SolveDesc *)pl.d_sdescs.data(), (const int32_t *)pl.d_bu_items.data() + 2 * bu.it0,
                pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, tr);
 }
@@ -877,9 +837,7 @@ void fx_backward_update(const Plan &pl, const BwdUpd &bu, const SolveBufs<double
 void fx_prepare() {
     smem_limit((const void *)k_fx_fwd_step, FWD_SMEM);
     smem_limit((const void *)k_fx_bwd_update, BWD_SMEM);
-    smem_limit((const void *)k_fx_bwd_step<8>, BWD_SMEM);
-    smem_limit((const void *)k_fx_bwd_step<16>, BWD_SMEM);
-    smem_limit((const void *)k_fx_bwd_step<32>, BWD_SMEM);
+    smem_limit((const void *)k_fx_bwd_step, BWD_SMEM);
 }
 
 }  // namespace mbl

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(UF_THREADS, 2)
                 const int gi = i0 + ri, gj = j0 + rj;
                 if (gi >= f || gj > gi) continue;
                 int64_t hi, lo;
-                fx_collect(acc[m][n], k, hi, lo);
+                fx_collect<false>(acc[m][n], k, hi, lo);
                 F[(int64_t)gj * f + gi] = c[m][k] - fx_value(hi, lo, el[ri], ew[rj]);
             }
     }
