@@ -17,6 +17,7 @@
 #include <cfloat>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "factor.h"
 #include "solve_tile.cuh"
@@ -272,7 +273,8 @@ __device__ __forceinline__ unsigned int mag_bits(float x) { return __float_as_ui
 __device__ __forceinline__ unsigned int mag_bits(double x) { return (unsigned int)__double2hiint(x) & 0x7fffffffu; }
 template <class T>
 __device__ __forceinline__ float mag_float(unsigned int b) {
-    return sizeof(T) == 4 ? __uint_as_float(b) : (float)__hiloint2double((int)b, 0);
+    if (sizeof(T) == 4) return __uint_as_float(b);
+    return b < 0x38100000u ? 0.f : (b >= 0x47e00000u ? 3.0e38f : __uint_as_float((b - 0x38000000u) << 3));
 }
 // u / d by a reciprocal and the quotient's own residual (a shorter chain than the division's).  FP64: the
 // reciprocal from FP32 by two Newton steps, nine FP64 operations where the division takes some thirty.
@@ -284,35 +286,37 @@ __device__ __forceinline__ float pdiv(float u, float d) {
 __device__ __forceinline__ double pdiv(double u, double d) { return fx_div(u, d); }
 
 // LDL^T of a panel's w x w diagonal block with symmetric 1x1 pivoting, 256 threads.  The whole block
-// (both triangles) is kept in registers: thread (r, h) holds row r, columns [16 h, 16 h + 16).  Rows are
-// never exchanged: a pivot row is marked done, its column of the remaining rows becomes zero by the update
-// itself (its multiplier is 1), and the order of the pivots is applied when the factor is written.  Per
-// step: the candidates' scores go to shared memory, every warp finds the best one, the threads that hold
-// the pivot's column publish it with its multipliers, and the block updates its registers; the largest
-// off-diagonal magnitude that the next choice needs falls out of the update.  Both mirror entries of the
-// update subtract u_a l_b with one rounding (a the larger index, u the unscaled pivot column, l = u / d),
-// so the block stays exactly symmetric.
-// Bound by the chain of w dependent steps on one SM (FP64: by the SM's two FMAs a clock too).  With the
-// block in shared memory, rows exchanged and a thread pair a row, a step took 1.2 us (79 us a launch inside
-// an L = 19 factorization); this one takes 0.75 us (50), with FP64 fronts 409 -> 230 us.
+// (both triangles) is kept in registers: lane l of warp (half, h) holds row 32 half + l, columns
+// [16 h, 16 h + 16).  Rows are never exchanged: a pivot row is marked done, its column of the remaining rows
+// becomes zero by the update itself (its multiplier is 1), and the order of the pivots is applied when the
+// factor is written.  Per step: the rows' largest off-diagonal magnitudes go to shared memory, every warp
+// finds the best candidate (a lane scores two), the two warps that hold the pivot's column publish it with
+// its multipliers, and the block updates its registers (entry (r, c) by u_r l_c, u the unscaled pivot column,
+// l = u / d, one rounding); the magnitudes of the next choice fall out of the update.
+// Bound by the chain of w dependent steps on one SM (FP64: by the SM's FP64 rate too).  With the block in
+// shared memory, rows exchanged and a thread pair a row, a launch took 79 us (409 with FP64 fronts); in
+// registers, four threads of a warp on a row, 50 (230); now 36 at L = 14, where it is alone, and 42 (209 to 231)
+// beside the building of G at L = 18 and 19.
 template <class T>
 __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, const int64_t *fo, const int32_t *fsz,
                                                     const int32_t *sn_start, T *arena, T *Dg, int32_t *piv,
                                                     double tiny, unsigned long long *counters,
                                                     const unsigned int *cmax) {
-    static_assert(NB == 64, "four threads per row of a 64-wide block on 256 threads");
+    static_assert(NB == 64, "two warps of rows, four of columns");
     constexpr int CPT = NB / 4;
     constexpr int E = 16 / sizeof(T);
     using V = typename Vec16<T>::type;
-    __shared__ __align__(16) T ucol[NB], lcol[NB];
+    __shared__ __align__(16) T lcol[NB];
+    __shared__ T ucol[NB];
     __shared__ T Ls[NB][NB + 1];  // Ls[t][r]: multiplier of row r in step t
     __shared__ T dcand[NB], dvec[NB];
     __shared__ int order[NB];
-    __shared__ unsigned int s_k1[NB], s_k2[NB];
+    __shared__ unsigned int s_om[4][NB];
     const PanelDesc d = descs[blockIdx.x];
     const int s = d.front, f = fsz[s], k0 = d.k0, w = d.w;
     T *F = arena + fo[s];
-    const int tid = threadIdx.x, lane = tid & 31, r = tid >> 2, h = tid & 3, c0 = h * CPT;
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, h = wp & 3, r = (wp >> 2) * 32 + lane, c0 = h * CPT;
+    const bool has_diag = h / 2 == wp >> 2;  // some row of the warp has its diagonal entry here
     T B[CPT];
 #pragma unroll
     for (int k = 0; k < CPT; ++k) {
@@ -320,7 +324,14 @@ __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, cons
         B[k] = hi < w ? F[(int64_t)(k0 + lo) * f + k0 + hi] : T(0);
     }
     T dr = r < w ? F[(int64_t)(k0 + r) * f + k0 + r] : T(0);  // the row's diagonal entry
-    const float cm = r < w ? __uint_as_float(cmax[(size_t)blockIdx.x * NB + r]) : 0.f;
+    // this lane's two candidates: the column maxima below the panel, and whether they are still to come
+    float cm[2];
+    bool cand[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        cand[u] = lane + 32 * u < w;
+        cm[u] = cand[u] ? __uint_as_float(cmax[(size_t)blockIdx.x * NB + lane + 32 * u]) : 0.f;
+    }
     bool active = r < w;
     unsigned int om = 0u;  // largest off-diagonal magnitude of the thread's part of the row
 #pragma unroll
@@ -328,29 +339,36 @@ __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, cons
         if (c0 + k != r) om = max(om, mag_bits(B[k]));
     unsigned int npert = 0u, nneg = 0u;
     for (int t = 0; t < w; ++t) {
+        s_om[h][r] = om;
+        if (h == 0) dcand[r] = dr;
+        __syncthreads();
         // pivot: the candidate whose diagonal is largest relative to the rest of its column (inside the
         // block and, from before this panel, in the rows below), which bounds the multipliers; order:
         // largest score, then largest |d|, then the smallest index.  Scores and |d| are non-negative
         // floats, so their bit patterns order like their values.
-        om = max(om, __shfl_xor_sync(0xffffffffu, om, 1));
-        om = max(om, __shfl_xor_sync(0xffffffffu, om, 2));
-        if (h == 0) {
-            const float o = fmaxf(mag_float<T>(om), cm);
-            const unsigned int db = mag_bits(dr);
-            const float sc = o > 0.f ? pdiv(mag_float<T>(db), o) : 3.0e38f;
-            s_k1[r] = active ? __float_as_uint(sc) + 1u : 0u;  // 0 marks a row that is no candidate
-            s_k2[r] = db;
-            dcand[r] = dr;
-        }
-        __syncthreads();
         int j;
         {
-            const unsigned int a1 = s_k1[lane], b1 = s_k1[lane + 32];
-            const unsigned int m1 = __reduce_max_sync(0xffffffffu, max(a1, b1));
-            const unsigned int a2 = a1 == m1 ? s_k2[lane] : 0u, b2 = b1 == m1 ? s_k2[lane + 32] : 0u;
-            const unsigned int m2 = __reduce_max_sync(0xffffffffu, max(a2, b2));
-            const unsigned int ja = a1 == m1 && a2 == m2 ? lane : NB, jb = b1 == m1 && b2 == m2 ? lane + 32 : NB;
-            j = (int)__reduce_min_sync(0xffffffffu, min(ja, jb));
+            unsigned int k1[2], k2[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int c = lane + 32 * u;
+                const unsigned int ob = max(max(s_om[0][c], s_om[1][c]), max(s_om[2][c], s_om[3][c]));
+                const float o = fmaxf(mag_float<T>(ob), cm[u]);
+                k2[u] = mag_bits(dcand[c]);
+                const float sc = o > 0.f ? fminf(__fdividef(mag_float<T>(k2[u]), o), 3.0e38f) : 3.0e38f;
+                k1[u] = cand[u] ? __float_as_uint(sc) + 1u : 0u;  // 0 marks a row that is no candidate
+            }
+            const unsigned int m1 = __reduce_max_sync(0xffffffffu, max(k1[0], k1[1]));
+            const unsigned int va = __ballot_sync(0xffffffffu, k1[0] == m1), vb = __ballot_sync(0xffffffffu, k1[1] == m1);
+            if (__popc(va) + __popc(vb) == 1) {
+                j = va ? __ffs(va) - 1 : __ffs(vb) + 31;
+            } else {
+                const unsigned int a2 = k1[0] == m1 ? k2[0] : 0u, b2 = k1[1] == m1 ? k2[1] : 0u;
+                const unsigned int m2 = __reduce_max_sync(0xffffffffu, max(a2, b2));
+                const unsigned int ja = k1[0] == m1 && a2 == m2 ? lane : NB, jb = k1[1] == m1 && b2 == m2 ? lane + 32 : NB;
+                j = (int)__reduce_min_sync(0xffffffffu, min(ja, jb));
+            }
+            if (lane == (j & 31)) (j >> 5 ? cand[1] : cand[0]) = false;
         }
         // the pivot (a tiny one replaced by +-tiny, statically)
         T dv = dcand[j];
@@ -367,20 +385,10 @@ __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, cons
             T u = j & 1 ? ub : ua;
             if (!active) u = T(0);
             if (r == j) u = dv;
+            const T l = pdiv(u, dv);
             ucol[r] = u;
-            if (sizeof(T) == 4) {
-                const T l = pdiv(u, dv);
-                lcol[r] = l;
-                Ls[t][r] = l;
-            }
-        }
-        if (sizeof(T) == 8) {  // the divisions on two full warps: FP64 instructions cost the same half empty
-            __syncthreads();
-            if (tid < NB) {
-                const T l = pdiv(ucol[tid], dv);
-                lcol[tid] = l;
-                Ls[t][tid] = l;
-            }
+            lcol[r] = l;
+            Ls[t][r] = l;
         }
         if (tid == 0) {
             dvec[t] = dv;
@@ -393,36 +401,42 @@ __global__ void __launch_bounds__(256) k_panel_diag(const PanelDesc *descs, cons
         const T ur = active ? ucol[r] : T(0), lr = active ? lcol[r] : T(0);
         dr = fnms(ur, lr, dr);
         om = 0u;
+        auto update = [&](auto diag) {
 #pragma unroll
-        for (int k0v = 0; k0v < CPT; k0v += E) {
-            const V uv = *reinterpret_cast<const V *>(ucol + c0 + k0v), lv = *reinterpret_cast<const V *>(lcol + c0 + k0v);
+            for (int k0v = 0; k0v < CPT; k0v += E) {
+                const V lv = *reinterpret_cast<const V *>(lcol + c0 + k0v);
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int k = k0v + e, c = c0 + k;
-                const T uc = Vec16<T>::get(uv, e), lc = Vec16<T>::get(lv, e);
-                const T v = fnms(c <= r ? ur : uc, c <= r ? lc : lr, B[k]);
-                B[k] = v;
-                if (c != r) om = max(om, mag_bits(v));
+                for (int e = 0; e < E; ++e) {
+                    const int k = k0v + e;
+                    B[k] = fnms(ur, Vec16<T>::get(lv, e), B[k]);
+                    const unsigned int mb = mag_bits(B[k]);
+                    om = max(om, decltype(diag)::value && c0 + k == r ? 0u : mb);
+                }
             }
-        }
+        };
+        if (has_diag) update(std::true_type());  // (the diagonal entry is kept in dr)
+        else update(std::false_type());
     }
     __syncthreads();
     if (tid == 0) {
         if (npert) atomicAdd(&counters[0], (unsigned long long)npert);
         if (nneg) atomicAdd(&counters[1], (unsigned long long)nneg);
     }
-    // write L11 (strictly lower) in pivot order, D on the diagonal, pivots
-    for (int idx = tid; idx < w * w; idx += 256) {
-        const int i = idx % w, c = idx / w;
-        if (i >= c) F[(int64_t)(k0 + c) * f + k0 + i] = i == c ? dvec[c] : Ls[c][order[i]];
-    }
+    // write L11 (strictly lower) in pivot order, D on the diagonal, pivots: a warp per column
+    float lmax = 0.f;
+    for (int c = wp; c < w; c += 8)
+        for (int i = lane; i < w; i += 32) {
+            if (i < c) continue;
+            const T l = i == c ? dvec[c] : Ls[c][order[i]];
+            F[(int64_t)(k0 + c) * f + k0 + i] = l;
+            if (i > c) lmax = fmaxf(lmax, (float)tabs(l));
+        }
+    for (int o = 16; o > 0; o >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    if (lane == 0) atomicMax(reinterpret_cast<unsigned int *>(counters + 3), __float_as_uint(lmax));
     const int64_t g0 = (int64_t)sn_start[s] + k0;
     if (tid < w) {
         Dg[g0 + tid] = dvec[tid];
         piv[g0 + tid] = k0 + order[tid];
-        float lmax = 0.f;
-        for (int i = tid + 1; i < w; ++i) lmax = fmaxf(lmax, (float)tabs(Ls[tid][order[i]]));
-        atomicMax(reinterpret_cast<unsigned int *>(counters + 3), __float_as_uint(lmax));
         atomicMin(reinterpret_cast<unsigned int *>(counters + 4), __float_as_uint((float)tabs(dvec[tid])));
     }
 }
