@@ -177,48 +177,81 @@ void copy_cols(int64_t n, const double *src, int lds, int s0, double *dst, int l
     MBL_LAUNCH_CHECK();
 }
 
-// Cholesky of the p x p Gram matrix G = R^T R (R upper, row-major); flag = 0 if not positive.
-__global__ void k_chol(int p, const double *G, double *R, int *flag) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double maxd = 0.0;
-    for (int j = 0; j < p; ++j) maxd = fmax(maxd, G[j * p + j]);
-    for (int i = 0; i < p * p; ++i) R[i] = 0.0;
-    for (int j = 0; j < p; ++j) {
-        double s = G[j * p + j];
-        for (int l = 0; l < j; ++l) s -= R[l * p + j] * R[l * p + j];
-        if (!(s > 1e-28 * maxd) || !(maxd > 0.0)) {
-            *flag = 0;
-            s = fmax(maxd, 1e-300);  // keep going with a harmless value
-        }
-        double rjj = sqrt(s);
-        R[j * p + j] = rjj;
-        for (int c = j + 1; c < p; ++c) {
-            double t = G[j * p + c];
-            for (int l = 0; l < j; ++l) t -= R[l * p + j] * R[l * p + c];
-            R[j * p + c] = t / rjj;
-        }
-    }
+// 1 / sqrt(s) from FP32 by three Newton steps (relative error below 2^-51): the FP64 square root and division are
+// chains of some thousand clocks on GB300
+__device__ __forceinline__ double inv_sqrt(double s) {
+    const float f = (float)s;
+    if (!(f > 1e-30f && f < 1e30f)) return 1.0 / sqrt(s);
+    double r = (double)rsqrtf(f);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r = fma(0.5 * r, fma(-s * r, r, 1.0), r);
+    return r;
 }
 
-// x_row <- x_row R^{-1} for every row
-__global__ void k_trsm_rows(int64_t n, double *X, int p, const double *R) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double x[32];
-    for (int j = 0; j < p; ++j) x[j] = X[i * p + j];
+// Cholesky of the p x p Gram matrix G = R^T R (R upper, row-major); flag = 0 if not positive.  One warp,
+// a lane per column of the trailing block in shared memory.
+__global__ void __launch_bounds__(32) k_chol(int p, const double *G, double *R, int *flag) {
+    __shared__ double A[32][33];
+    const int c = threadIdx.x;
+    for (int i = 0; i < p; ++i) A[i][c] = c < p ? G[i * p + c] : 0.0;
+    double maxd = c < p ? G[c * p + c] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) maxd = fmax(maxd, __shfl_xor_sync(0xffffffffu, maxd, o));
+    maxd = fmax(maxd, 0.0);
+    __syncwarp();
     for (int j = 0; j < p; ++j) {
-        double s = x[j];
-        for (int l = 0; l < j; ++l) s -= x[l] * R[l * p + j];
-        x[j] = s / R[j * p + j];
+        double s = A[j][j];
+        if (!(s > 1e-28 * maxd) || !(maxd > 0.0)) {
+            if (c == 0) *flag = 0;
+            s = fmax(maxd, 1e-300);  // keep going with a harmless value
+        }
+        const double ir = inv_sqrt(s);
+        const double r = c > j ? A[j][c] * ir : (c == j ? s * ir : 0.0);
+        __syncwarp();
+        A[j][c] = r;
+        __syncwarp();
+        if (c > j)
+            for (int i = j + 1; i <= c; ++i) A[i][c] = fma(-A[j][i], r, A[i][c]);
+        __syncwarp();
     }
-    for (int j = 0; j < p; ++j) X[i * p + j] = x[j];
+    for (int i = 0; i < p; ++i)
+        if (c < p) R[i * p + c] = A[i][c] * (c >= i ? 1.0 : 0.0);
+}
+
+// x_row <- x_row R^{-1} for every row (P columns or fewer, in registers)
+template <int P>
+__global__ void k_trsm_rows(int64_t n, double *X, int p, const double *R) {
+    __shared__ double Rs[P][P + 1], inv[P];
+    for (int u = threadIdx.x; u < P * P; u += blockDim.x) {
+        const int i = u / P, j = u % P;
+        Rs[i][j] = i < p && j < p ? R[i * p + j] : 0.0;
+        if (i == j) inv[i] = i < p ? 1.0 / R[i * p + i] : 0.0;
+    }
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double x[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) x[j] = j < p ? X[i * p + j] : 0.0;
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        double s = x[j];
+#pragma unroll
+        for (int l = 0; l < j; ++l) s -= x[l] * Rs[l][j];
+        x[j] = s * inv[j];
+    }
+#pragma unroll
+    for (int j = 0; j < P; ++j)
+        if (j < p) X[i * p + j] = x[j];
 }
 
 void chol_qr(int64_t n, double *X, int p, double *R, double *G, double *work, int *d_flag, cudaStream_t st) {
     dense_tn(n, X, p, 0, p, X, p, 0, p, G, work, st);
     k_chol<<<1, 32, 0, st>>>(p, G, R, d_flag);
     MBL_LAUNCH_CHECK();
-    k_trsm_rows<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(n, X, p, R);
+    const unsigned g = (unsigned)((n + 127) / 128);
+    if (p <= 8) k_trsm_rows<8><<<g, 128, 0, st>>>(n, X, p, R);
+    else if (p <= 16) k_trsm_rows<16><<<g, 128, 0, st>>>(n, X, p, R);
+    else k_trsm_rows<32><<<g, 128, 0, st>>>(n, X, p, R);
     MBL_LAUNCH_CHECK();
 }
 
@@ -359,58 +392,82 @@ __device__ void ql_sweep_record(int lo, int hi, R *d, R *e, R *cs, R *sn) {
     d[lo] = dk1;
 }
 
-// Householder reduction of the symmetric m x m matrix a (column-major, leading dimension lda) to
-// tridiagonal form, by the whole block: afterwards the diagonal and subdiagonal are on a's diagonals, the
-// reflectors' tails below the subdiagonal and their scalings in beta.  red: 64 entries.  Bound by the chain
-// of m steps: four barriers a step (the norm, the reflector, the product, the update); four lanes share a
-// row of the product.
+// Householder reduction of the symmetric m x m matrix a (column-major, leading dimension lda, lower triangle
+// used and kept) to tridiagonal form, by the whole block: afterwards the diagonal and subdiagonal are on a's
+// diagonals, the reflectors' tails below the subdiagonal and their scalings in beta.  red: 64 entries.  FP64:
+// bound by the SM's FP64 rate, so the scalars of a reflector come from one warp (every warp computing its own
+// sums, root and divisions took a third of the time) and only the lower triangle is updated.
 template <class R>
 __device__ void householder_tridiag(R *a, int lda, int m, R *beta, R *vv, R *pp, R *red) {
     for (int k = 0; k + 2 < m; ++k) {
         const int len = m - k - 1;
         R *x = a + (size_t)k * lda + (k + 1);
-        R loc = R(0);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) loc += x[i] * x[i];
-        const R alpha2 = block_sum1(loc, red);
-        if (alpha2 == R(0)) {
+        if (threadIdx.x < 32) {
+            R loc = R(0);
+            for (int i = threadIdx.x; i < len; i += 32) loc += x[i] * x[i];
+            for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+            if (threadIdx.x == 0) {
+                const R x0 = x[0], alpha = sqrt(loc);
+                const R v0 = x0 >= R(0) ? x0 + alpha : x0 - alpha;
+                red[32] = loc;
+                red[33] = loc == R(0) ? R(0) : R(1) / v0;
+                red[34] = x0 >= R(0) ? -alpha : alpha;
+                // v = x / v0 with v_0 = 1: 2 / |v|^2 = |v0| / alpha
+                red[35] = loc == R(0) ? R(0) : fabs(v0) / alpha;
+            }
+        }
+        __syncthreads();
+        const R iv0 = red[33], bk = red[35];
+        if (red[32] == R(0)) {
             if (threadIdx.x == 0) beta[k] = R(0);
             __syncthreads();
             continue;
         }
-        const R x0 = x[0];
-        const R sgn = x0 >= R(0) ? R(1) : R(-1);
-        const R alpha = sqrt(alpha2);
-        const R v0 = x0 + sgn * alpha;
-        const R iv0 = R(1) / v0;
-        // v = x / v0 with v_0 = 1: 2 / |v|^2 = |v0| / alpha
-        const R bk = fabs(v0) / alpha;
         for (int i = threadIdx.x; i < len; i += blockDim.x) vv[i] = i == 0 ? R(1) : x[i] * iv0;
         __syncthreads();
+        // p = bk A22 v, four lanes a row: entries (i, j) of the lower triangle, mirrored above it
         R *A22 = a + (size_t)(k + 1) * lda + (k + 1);
         const int part = threadIdx.x & 3, step = blockDim.x >> 2;
-        loc = R(0);
         for (int i0 = 0; i0 < len; i0 += step) {
             const int i = i0 + (int)(threadIdx.x >> 2);
             R s = R(0);
-            if (i < len)
-                for (int j = part; j < len; j += 4) s = fma(A22[(size_t)j * lda + i], vv[j], s);
+            if (i < len) {
+                int j = part;
+                for (; j <= i; j += 4) s = fma(A22[(size_t)j * lda + i], vv[j], s);
+                for (; j < len; j += 4) s = fma(A22[(size_t)i * lda + j], vv[j], s);
+            }
             s += __shfl_xor_sync(0xffffffffu, s, 1);
             s += __shfl_xor_sync(0xffffffffu, s, 2);
-            if (i < len && part == 0) {
-                s *= bk;
-                pp[i] = s;
-                loc += s * vv[i];
+            if (i < len && part == 0) pp[i] = s * bk;
+        }
+        __syncthreads();
+        // w = p - (bk / 2) (p . v) v, by one warp
+        if (threadIdx.x < 32) {
+            R loc = R(0);
+            for (int i = threadIdx.x; i < len; i += 32) loc += pp[i] * vv[i];
+            for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+            const R K = R(0.5) * bk * loc;
+            for (int i = threadIdx.x; i < len; i += 32) pp[i] -= K * vv[i];
+        } else {
+            for (int i = (int)threadIdx.x - 32; i < len; i += (int)blockDim.x - 32) x[i] = i == 0 ? red[34] : vv[i];
+            if (threadIdx.x == 32) beta[k] = bk;
+        }
+        __syncthreads();
+        // A22 -= v w^T + w v^T, lower triangle: a warp per column pair (j, len - 1 - j), len + 1 entries in all
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int q = threadIdx.x >> 5; q < (len + 1) / 2; q += nw) {
+            const int j2 = len - 1 - q;
+            const R v1 = vv[q], w1 = pp[q], v2 = vv[j2], w2 = pp[j2];
+            R *c1 = A22 + (size_t)q * lda, *c2 = A22 + (size_t)j2 * lda;
+            const int n1 = len - q;  // entries q .. len - 1 of column q, then j2 .. len - 1 of column j2
+            for (int e = lane; e < (j2 > q ? len + 1 : n1); e += 32) {
+                const bool first = e < n1;
+                const int i = first ? q + e : j2 + e - n1;
+                R *c = first ? c1 : c2;
+                const R vj = first ? v1 : v2, wj = first ? w1 : w2;
+                c[i] -= vv[i] * wj + pp[i] * vj;
             }
         }
-        const R K = R(0.5) * bk * block_sum1(loc, red + 32);
-        // A22 -= v w^T + w v^T with w = p - K v
-        for (int t = threadIdx.x; t < len * len; t += blockDim.x) {
-            const int i = t % len, j = t / len;
-            const R vi = vv[i], vj = vv[j];
-            A22[(size_t)j * lda + i] -= vi * (pp[j] - K * vj) + (pp[i] - K * vi) * vj;
-        }
-        for (int i = threadIdx.x; i < len; i += blockDim.x) x[i] = (i == 0) ? -sgn * alpha : vv[i];
-        if (threadIdx.x == 0) beta[k] = bk;
         __syncthreads();
     }
 }
@@ -694,7 +751,6 @@ __global__ void __launch_bounds__(EIG_THREADS) k_bi_tridiag(int m, double *A, R 
 template <class R>
 __global__ void k_bi_values(int m, const R *work, double *W) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
     const R *d = work, *e = work + m, *e2 = work + 2 * m;
     R gl = d[0], gu = d[0], emax2 = R(0);
     for (int i = 0; i < m; ++i) {
@@ -707,13 +763,26 @@ __global__ void k_bi_values(int m, const R *work, double *W) {
     gl -= R(2) * eps * tn * (R)m + tiny;
     gu += R(2) * eps * tn * (R)m + tiny;
     const R pivmin = tiny * fmax(R(1), emax2), atol = R(2) * eps * tn;  // absolute accuracy 2 eps ||T||
+    __shared__ double sd[EIG_SMEM_MAX_M], se2[EIG_SMEM_MAX_M];
+    const double sc = tn > R(0) && tn < R(INFINITY) ? scalbn(1.0, -ilogb((double)tn)) : 1.0;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        sd[i] = (double)d[i] * sc;
+        se2[i] = i + 1 < m ? ((double)e[i] * sc) * ((double)e[i] * sc) : 0.0;
+    }
+    __syncthreads();
+    if (j >= m) return;
     R lo = gl, hi = gu;
     for (int it = 0; it < 200; ++it) {
         const R mid = R(0.5) * (lo + hi);
         if (hi - lo <= R(2) * eps * fmax(fabs(lo), fabs(hi)) + R(4) * pivmin || hi - lo <= atol || mid == lo ||
             mid == hi)
             break;
-        if (sturm_count<R>(m, d, e2, mid, pivmin) > j) hi = mid; else lo = mid;
+        if constexpr (sizeof(R) == 8) {
+            // counts from the minors, on T scaled to a norm of about 1
+            if (sturm_count_minors(m, sd, se2, mid * sc) > j) hi = mid; else lo = mid;
+        } else {
+            if (sturm_count<R>(m, d, e2, mid, pivmin) > j) hi = mid; else lo = mid;
+        }
     }
     W[j] = (double)(R(0.5) * (lo + hi));
 }

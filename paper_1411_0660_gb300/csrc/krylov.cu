@@ -96,21 +96,26 @@ __global__ void k_pack_sym(const double *T, int ldt, int mm, double *A) {
 // lambda_i = S_ii / G_ii and X <- X (I + E) with E_ii = r_ii / 2 and, for |lambda_i - lambda_j| > delta,
 // E_ij = (S_ij + lambda_j r_ij) / (lambda_j - lambda_i), where r = I - G; closer pairs (a cluster
 // at the current accuracy) take E_ij = r_ij / 2, which refines the cluster's subspace.  delta =
-// 2 (||S - diag(lambda)|| + ||A|| ||r||), Frobenius norms and ||A|| ~ max |lambda|.  One CTA.
-__global__ void __launch_bounds__(1024) k_oa_step(int m, const double *G, const double *S, double *lam, double *E) {
-    __shared__ double red[3][32];
-    __shared__ double s_delta;
+// 2 (||S - diag(lambda)|| + ||A|| ||r||), Frobenius norms and ||A|| ~ max |lambda|.  OA_CTAS CTAs: each sums
+// a share of the norms (k_oa_norms), then every one of k_oa_step adds the shares in the same order and
+// writes a share of E -- its divisions, in FP64, kept one CTA busy for 83 us at m = 116.
+constexpr int OA_CTAS = 32;
+__global__ void __launch_bounds__(256) k_oa_norms(int m, const double *G, const double *S, double *lam, double *part) {
+    __shared__ double red[3][8];
     const int t = threadIdx.x;
-    for (int i = t; i < m; i += blockDim.x) lam[i] = S[(size_t)i * m + i] / G[(size_t)i * m + i];
-    __syncthreads();
     double off = 0.0, rr = 0.0, amax = 0.0;
-    for (int idx = t; idx < m * m; idx += blockDim.x) {
+    for (int idx = blockIdx.x * 256 + t; idx < m * m; idx += OA_CTAS * 256) {
         const int i = idx % m, j = idx / m;
         const double r = (i == j ? 1.0 : 0.0) - G[idx];
-        const double sv = S[idx] - (i == j ? lam[i] : 0.0);
+        double sv = S[idx];
+        if (i == j) {
+            const double l = sv / G[idx];
+            lam[i] = l;
+            amax = fmax(amax, fabs(l));
+            sv -= l;
+        }
         off += sv * sv;
         rr += r * r;
-        if (i == j) amax = fmax(amax, fabs(lam[i]));
     }
     for (int o = 16; o > 0; o >>= 1) {
         off += __shfl_xor_sync(0xffffffffu, off, o);
@@ -125,16 +130,27 @@ __global__ void __launch_bounds__(1024) k_oa_step(int m, const double *G, const 
     __syncthreads();
     if (t == 0) {
         double a = 0.0, b = 0.0, c = 0.0;
-        for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) {
+        for (int w = 0; w < 8; ++w) {
             a += red[0][w];
             b += red[1][w];
             c = fmax(c, red[2][w]);
         }
-        s_delta = 2.0 * (sqrt(a) + c * sqrt(b));
+        part[3 * blockIdx.x] = a;
+        part[3 * blockIdx.x + 1] = b;
+        part[3 * blockIdx.x + 2] = c;
     }
-    __syncthreads();
-    const double delta = s_delta;
-    for (int idx = t; idx < m * m; idx += blockDim.x) {
+}
+
+__global__ void __launch_bounds__(256) k_oa_step(int m, const double *G, const double *S, const double *lam,
+                                                 const double *part, double *E) {
+    double a = 0.0, b = 0.0, c = 0.0;
+    for (int w = 0; w < OA_CTAS; ++w) {
+        a += part[3 * w];
+        b += part[3 * w + 1];
+        c = fmax(c, part[3 * w + 2]);
+    }
+    const double delta = 2.0 * (sqrt(a) + c * sqrt(b));
+    for (int idx = blockIdx.x * 256 + threadIdx.x; idx < m * m; idx += OA_CTAS * 256) {
         const int i = idx % m, j = idx / m;
         const double r = (i == j ? 1.0 : 0.0) - G[idx];
         double e = 0.5 * r;
@@ -166,7 +182,10 @@ static void refine_eig(int m, const double *A, double *X, double *lam, int steps
         gemm_small(true, false, m, m, m, 1.0, X, m, X, m, 0.0, G, m, st);
         gemm_small(false, false, m, m, m, 1.0, A, m, X, m, 0.0, Q, m, st);
         gemm_small(true, false, m, m, m, 1.0, X, m, Q, m, 0.0, S, m, st);
-        k_oa_step<<<1, 1024, 0, st>>>(m, G, S, lam, Q);  // E into Q
+        // (the norms' shares go behind the eigenvalues; E into Q)
+        k_oa_norms<<<OA_CTAS, 256, 0, st>>>(m, G, S, lam, lam + m);
+        MBL_LAUNCH_CHECK();
+        k_oa_step<<<OA_CTAS, 256, 0, st>>>(m, G, S, lam, lam + m, Q);
         MBL_LAUNCH_CHECK();
         MBL_CUDA(cudaMemcpyAsync(G, X, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, st));
         gemm_small(false, false, m, m, m, 1.0, G, m, Q, m, 1.0, X, m, st);  // X += X E
@@ -359,7 +378,7 @@ KrylovSchur::KrylovSchur(Ctx *c, int64_t n_, int p_, int ncv_) : ctx(c), n(n_), 
     flag.alloc(ctx, 1);
     work.alloc(ctx, std::max(dense_tn_work(n, ldv, p), dense_tn_work(n, ldv, 32)) + 64);
     eigA.alloc(ctx, (size_t)ldv * ldv);
-    eigW.alloc(ctx, ldv);
+    eigW.alloc(ctx, ldv + 3 * OA_CTAS);  // and the norms' shares of a refinement step
     eigWork.alloc(ctx, syev_work_doubles(ldv));
     eigInfo.alloc(ctx, 1);
     eigM.alloc(ctx, 1);
@@ -724,16 +743,23 @@ __global__ void __launch_bounds__(512) k_small_inverse(int k, double *A, int *fl
     if (t == 0) *flag = 1;
     __syncthreads();
     for (int j = 0; j < k; ++j) {
-        if (t == 0) {
+        if (t < 32) {  // the largest entry of the column, the first of equals
+            double best = -1.0;
             int p = j;
-            double best = fabs(sa[j * k + j]);
-            for (int i = j + 1; i < k; ++i)
+            for (int i = j + t; i < k; i += 32)
                 if (fabs(sa[i * k + j]) > best) {
                     best = fabs(sa[i * k + j]);
                     p = i;
                 }
-            s_p = p;
-            perm[j] = p;
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int op = __shfl_xor_sync(0xffffffffu, p, o);
+                if (ob > best || (ob == best && op < p)) best = ob, p = op;
+            }
+            if (t == 0) {
+                s_p = p;
+                perm[j] = p;
+            }
         }
         __syncthreads();
         const int p = s_p;
@@ -756,10 +782,11 @@ __global__ void __launch_bounds__(512) k_small_inverse(int k, double *A, int *fl
         const double ip = 1.0 / s_piv;
         for (int c = t; c < k; c += blockDim.x) sa[j * k + c] *= ip;
         __syncthreads();
-        for (int idx = t; idx < k * k; idx += blockDim.x) {
-            const int i = idx / k, c = idx % k;
-            if (i == j || c == j) continue;
-            sa[i * k + c] -= sa[i * k + j] * sa[j * k + c];
+        for (int i = t >> 5; i < k; i += 16) {  // a warp per row
+            if (i == j) continue;
+            const double f = sa[i * k + j];
+            for (int c = t & 31; c < k; c += 32)
+                if (c != j) sa[i * k + c] -= f * sa[j * k + c];
         }
         __syncthreads();
         for (int i = t; i < k; i += blockDim.x)
@@ -789,7 +816,7 @@ __global__ void k_cols_to_f32(int64_t n, const double *src, int lds, int k, floa
 }
 
 // ---- deflation products: tall-skinny products with the FP32 copies U32, AU32 (n x kd, kd <= 90) ----
-constexpr int DEFL_ROWS = 256;  // rows per CTA of k_defl_tn
+constexpr int DEFL_ROWS = 64;  // rows per CTA of k_defl_tn (short enough that a small sector still fills the SMs)
 
 // part[b][a][q] = sum over the block's rows r of U[r][a] V[r][q] (FP32 arithmetic, V converted): thread
 // a of the CTA owns column a of U (coalesced row reads), the block's rows of V are staged in shared
@@ -811,6 +838,7 @@ __global__ void __launch_bounds__(128) k_defl_tn(int64_t n, int kd, int p, const
 #pragma unroll
     for (int q = 0; q < PB; ++q) acc[q] = 0.f;
     const float *u = U + r0 * kd + a;
+#pragma unroll 8
     for (int r = 0; r < nr; ++r) {
         const float ur = u[(int64_t)r * kd];
 #pragma unroll
@@ -1675,7 +1703,7 @@ RitzH::RitzH(Ctx *c, int64_t n_, int ldv, int nev_) : ctx(c), n(n_), nev(nev_) {
     Gr2.alloc(ctx, (size_t)ldv * ldv);
     Gr3.alloc(ctx, (size_t)ldv * ldv);
     M2.alloc(ctx, (size_t)ldv * ldv);
-    Gw.alloc(ctx, ldv);
+    Gw.alloc(ctx, ldv + 3 * OA_CTAS);
     Gwork.alloc(ctx, syev_work_doubles(ldv));
     if (ldv <= EIG_SMEM_MAX_M) Bwork.alloc(ctx, syev_bisect_work(ldv));
     Ctmp.alloc(ctx, (size_t)ldv * 32);

@@ -19,31 +19,38 @@
 
 namespace mbl {
 
-__global__ void k_gap_ratio(int nev, const double *ev, double *r, double *rmean) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One warp: a lane per ratio; the mean sums them in order.
+__global__ void __launch_bounds__(32) k_gap_ratio(int nev, const double *ev, double *r, double *rmean) {
     double s = 0.0;
     int cnt = 0;
-    for (int k = 1; k + 1 < nev; ++k) {
-        double d0 = ev[k] - ev[k - 1], d1 = ev[k + 1] - ev[k];
-        double mx = d0 > d1 ? d0 : d1, mn = d0 > d1 ? d1 : d0;
-        if (mx == 0.0) {
-            r[k - 1] = NAN;
-            continue;
+    for (int k0 = 1; k0 + 1 < nev; k0 += 32) {
+        const int k = k0 + (int)threadIdx.x;
+        double x = NAN;
+        if (k + 1 < nev) {
+            const double d0 = ev[k] - ev[k - 1], d1 = ev[k + 1] - ev[k];
+            const double mx = d0 > d1 ? d0 : d1, mn = d0 > d1 ? d1 : d0;
+            if (mx != 0.0) x = mn / mx;
+            r[k - 1] = x;
         }
-        r[k - 1] = mn / mx;
-        s += r[k - 1];
-        ++cnt;
+        const bool live = k + 1 < nev && x == x;
+        for (int l = 0; l < 32; ++l) {
+            const double y = __shfl_sync(0xffffffffu, x, l);
+            if (__shfl_sync(0xffffffffu, (int)live, l)) s += y, ++cnt;
+        }
     }
-    if (rmean) *rmean = cnt > 0 ? s / cnt : NAN;
+    if (rmean && threadIdx.x == 0) *rmean = cnt > 0 ? s / cnt : NAN;
 }
 
-// One CTA per vector: A = sum y^2, B = sum y^2 ln y^2; S = ln A - B / A.
-__global__ void k_s1p(int64_t n, const double *Y, double *s1p, double *nrm2) {
-    __shared__ double ra[32], rb[32];
-    const double *y = Y + (int64_t)blockIdx.x * n;
+// A = sum y^2, B = sum y^2 ln y^2 over chunk c of vector j (CTA (c, j)): part[(j * nch + c) * 2 + {0, 1}].  Bound by
+// the logarithms in FP64, so the chunks fill the SMs whatever the number of vectors.
+__global__ void __launch_bounds__(256) k_s1p_part(int64_t n, int nch, const double *Y, double *part) {
+    __shared__ double ra[8], rb[8];
+    const int j = blockIdx.y, c = blockIdx.x;
+    const int64_t per = (n + nch - 1) / nch, r0 = (int64_t)c * per, r1 = min(n, r0 + per);
+    const double *y = Y + (int64_t)j * n;
     double a = 0.0, b = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        double v = y[i] * y[i];
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+        const double v = y[i] * y[i];
         a += v;
         if (v > 0.0) b += v * log(v);
     }
@@ -51,15 +58,34 @@ __global__ void k_s1p(int64_t n, const double *Y, double *s1p, double *nrm2) {
         a += __shfl_down_sync(0xffffffffu, a, o);
         b += __shfl_down_sync(0xffffffffu, b, o);
     }
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) { ra[w] = a; rb[w] = b; }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane == 0) {
+        ra[w] = a;
+        rb[w] = b;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double A = 0.0, B = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { A += ra[i]; B += rb[i]; }
-        s1p[blockIdx.x] = log(A) - B / A;
-        nrm2[blockIdx.x] = A;
+        for (int i = 0; i < 8; ++i) {
+            A += ra[i];
+            B += rb[i];
+        }
+        part[((int64_t)j * nch + c) * 2] = A;
+        part[((int64_t)j * nch + c) * 2 + 1] = B;
     }
+}
+
+// S = ln A - B / A of vector j, a thread each, the chunks in order.
+__global__ void k_s1p_fin(int nev, int nch, const double *part, double *s1p, double *nrm2) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nev) return;
+    double A = 0.0, B = 0.0;
+    for (int c = 0; c < nch; ++c) {
+        A += part[((int64_t)j * nch + c) * 2];
+        B += part[((int64_t)j * nch + c) * 2 + 1];
+    }
+    s1p[j] = log(A) - B / A;
+    nrm2[j] = A;
 }
 
 // Gram matrices: CTA (vector j, block q) writes G_q (dA x dA, column-major) normalized by |y|^2.
@@ -77,9 +103,12 @@ __global__ void k_gram(int64_t n, int nblk, const double *Y, const double *nrm2,
         for (int t = threadIdx.x; t < da * db; t += blockDim.x) Ms[t] = y[ix[t]];
         __syncthreads();
     }
-    for (int t = threadIdx.x; t < da * da; t += blockDim.x) {
-        int r = t % da, c = t / da;
-        if (r < c) continue;
+    for (int t = threadIdx.x; t < da * (da + 1) / 2; t += blockDim.x) {
+        // row r, column c <= r of the lower triangle, row by row (no lanes idle above the diagonal)
+        int r = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while ((r + 1) * (r + 2) / 2 <= t) ++r;
+        while (r * (r + 1) / 2 > t) --r;
+        const int c = t - r * (r + 1) / 2;
         double s = 0.0;
         if (in_smem)
             for (int b = 0; b < db; ++b) s += Ms[r * db + b] * Ms[c * db + b];
@@ -93,19 +122,21 @@ __global__ void k_gram(int64_t n, int nblk, const double *Y, const double *nrm2,
 
 // S_E of vector j from the Schmidt weights of its nblk blocks; NaN if the eigensolver reported a
 // block it did not converge (info != 0), so that a wrong value is never returned silently.
+// (A warp per vector, lanes over a block's weights, in a fixed order.)
 __global__ void k_entropy_sum(int nev, int nblk, const int32_t *dA, const int64_t *woff, const double *lam,
                               const int *info, double *se) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= nev) return;
     double S = 0.0;
     bool bad = false;
     for (int q = 0; q < nblk; ++q) {
         bad = bad || info[(int64_t)j * nblk + q] != 0;
         const double *l = lam + woff[(int64_t)j * nblk + q];
-        for (int i = 0; i < dA[q]; ++i)
+        for (int i = lane; i < dA[q]; i += 32)
             if (l[i] > 1e-15) S -= l[i] * log(l[i]);
     }
-    se[j] = bad ? nan("") : S;
+    for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
+    if (lane == 0) se[j] = bad ? nan("") : S;
 }
 
 static int64_t host_rank(uint32_t s) {
@@ -341,7 +372,13 @@ void observables_dev(Ctx *ctx, int L, int nup, int nev, const double *d_evals, c
     }
     DVec<double> nrm2;
     nrm2.alloc(ctx, nev);
-    k_s1p<<<nev, 256, 0, st>>>(n, d_evecs, d_s1p, nrm2.data());
+    // about four CTAs per SM over all vectors, chunks of at least 1024 rows
+    const int nch = (int)std::max<int64_t>(1, std::min<int64_t>((4 * ctx->sm_count + nev - 1) / nev, n / 1024));
+    DVec<double> spart;
+    spart.alloc(ctx, (size_t)nev * nch * 2);
+    k_s1p_part<<<dim3(nch, nev), 256, 0, st>>>(n, nch, d_evecs, spart.data());
+    MBL_LAUNCH_CHECK();
+    k_s1p_fin<<<(nev + 127) / 128, 128, 0, st>>>(nev, nch, spart.data(), d_s1p, nrm2.data());
     MBL_LAUNCH_CHECK();
     EntTables &E = ent_tables(ctx, L, nup);
     int nb = E.nblk;
@@ -387,7 +424,7 @@ void observables_dev(Ctx *ctx, int L, int nup, int nev, const double *d_evals, c
     MBL_LAUNCH_CHECK();
     syev_batched((int)batch, dm.data(), dgo.data(), dwo.data(), G.data(), lam.data(), 0, nullptr, E.dAmax,
                  work.data(), info.data(), st);
-    k_entropy_sum<<<(nev + 63) / 64, 64, 0, st>>>(nev, nb, E.d_dA.data(), dwo.data(), lam.data(), info.data(),
+    k_entropy_sum<<<(nev + 3) / 4, 128, 0, st>>>(nev, nb, E.d_dA.data(), dwo.data(), lam.data(), info.data(),
                                                    d_se);
     MBL_LAUNCH_CHECK();
     MBL_CUDA(cudaStreamSynchronize(st));
