@@ -117,6 +117,25 @@ static cudaMemPool_t device_pool(int device) {
 
 void trim_device_pool(int device) { cudaMemPoolTrimTo(device_pool(device), 0); }
 
+void ReadBack::add(void *dst, const void *src, size_t bytes) {
+    if (!ctx->pin) MBL_CUDA(cudaMallocHost(&ctx->pin, PIN_BYTES));
+    if (bytes > PIN_BYTES) {  // too large for the buffer: straight to its place
+        MBL_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st));
+        return;
+    }
+    if (used + bytes > PIN_BYTES) done();
+    MBL_CUDA(cudaMemcpyAsync(ctx->pin + used, src, bytes, cudaMemcpyDeviceToHost, st));
+    items.push_back({dst, used, bytes});
+    used += (bytes + 15) & ~(size_t)15;
+}
+
+void ReadBack::done() {
+    MBL_CUDA(cudaStreamSynchronize(st));
+    for (const Item &i : items) std::memcpy(i.dst, ctx->pin + i.off, i.bytes);
+    items.clear();
+    used = 0;
+}
+
 void DevMem::alloc(Ctx *c, size_t nbytes) {
     release();
     if (nbytes == 0) nbytes = 16;
@@ -365,6 +384,7 @@ void mbl_ctx_destroy(mbl_ctx *ctx) {
     ctx->ent.clear();
     cudaStreamSynchronize(ctx->stream);
     cudaStreamDestroy(ctx->stream);
+    if (ctx->pin) cudaFreeHost(ctx->pin);
     if (ctx->side_ev) cudaEventDestroy(ctx->side_ev);
     if (ctx->side) cudaStreamDestroy(ctx->side);
     {

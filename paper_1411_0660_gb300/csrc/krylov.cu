@@ -404,15 +404,13 @@ void KrylovSchur::orthonormalize_new_block(int m, cudaStream_t st, bool *deflate
         dense_tn(n, Vd, ldv, 0, m, W.data(), p, 0, p, C2.data(), work.data(), st);
         dense_nn_sub(n, Vd, ldv, 0, m, C2.data(), p, W.data(), st);
     }
-    int one = 1;
-    MBL_CUDA(cudaMemcpyAsync(flag.data(), &one, sizeof(int), cudaMemcpyHostToDevice, st));
+    MBL_CUDA(cudaMemsetAsync(flag.data(), 1, sizeof(int), st));  // any nonzero value: no deflation seen
     chol_qr(n, W.data(), p, R1.data(), G.data(), work.data(), flag.data(), st);
     chol_qr(n, W.data(), p, R2.data(), G.data(), work.data(), flag.data(), st);
     k_upper_mul<<<1, 1024, 0, st>>>(p, R2.data(), R1.data(), Rm.data());
     MBL_LAUNCH_CHECK();
     int ok = 1;
-    MBL_CUDA(cudaMemcpyAsync(&ok, flag.data(), sizeof(int), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaStreamSynchronize(st));
+    read_back(ctx, st, &ok, flag.data(), sizeof(int));
     *deflated = (ok == 0);
 }
 
@@ -494,8 +492,7 @@ void KrylovSchur::ritz(cudaStream_t st, std::vector<double> &theta, std::vector<
             syev_batched(1, eigM.data(), eigOff.data(), eigOff.data(), eigA.data(), eigW.data(), 1, nullptr, ldv,
                          eigWork.data(), eigInfo.data(), st, fp32);
         }
-        MBL_CUDA(cudaMemcpyAsync(&info, eigInfo.data(), sizeof(int), cudaMemcpyDeviceToHost, st));
-        MBL_CUDA(cudaStreamSynchronize(st));
+        read_back(ctx, st, &info, eigInfo.data(), sizeof(int));
         if (fp32 && info != 0) {  // QL did not converge in FP32: redo in FP64
             ProfScope ps2(ctx, "syev_fallback", (double)mm, st);
             k_pack_sym<<<nblk((int64_t)mm * mm), 256, 0, st>>>(T.data(), ldv, mm, eigA.data());
@@ -512,9 +509,10 @@ void KrylovSchur::ritz(cudaStream_t st, std::vector<double> &theta, std::vector<
     MBL_LAUNCH_CHECK();
     theta.resize(mm);
     rnorm.resize(mm);
-    MBL_CUDA(cudaMemcpyAsync(theta.data(), eigW.data(), mm * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaMemcpyAsync(rnorm.data(), res.data(), mm * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaStreamSynchronize(st));
+    ReadBack rb(ctx, st);
+    rb.add(theta.data(), eigW.data(), mm * sizeof(double));
+    rb.add(rnorm.data(), res.data(), mm * sizeof(double));
+    rb.done();
 }
 
 void KrylovSchur::restart(const std::vector<int> &keep_idx, cudaStream_t st) {
@@ -568,8 +566,7 @@ double RefinedSolve::residual(const double *X, int ldx, double *Y, int p, cudaSt
     k_reduce_parts<<<reduce_grid(3 * p), 256, 0, st>>>((int)nb, 3 * p, part.data(), norms.data());
     MBL_LAUNCH_CHECK();
     std::vector<double> h(3 * p);
-    MBL_CUDA(cudaMemcpyAsync(h.data(), norms.data(), 3 * p * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaStreamSynchronize(st));
+    read_back(sec->ctx, st, h.data(), norms.data(), 3 * p * sizeof(double));
     double worst = 0.0, rmax = 0.0;
     if (rn) rn->assign(p, 0.0);
     if (lim) lim->assign(p, 0.0);
@@ -613,99 +610,167 @@ void RefinedSolve::apply_plain(const double *X, int ldx, double *Y, int p, cudaS
     }
 }
 
+// Waits until every CTA of the launch (co-resident: a cooperative launch) has come here as often as this one:
+// *bar counts the arrivals, `target` is the count to wait for (modulo 2^32).  At most GRID_WAIT_NS; false on
+// expiry, which is counted in *err.  The CTAs' writes before it are visible after it (read them with ld.cg).
+constexpr uint64_t GRID_WAIT_NS = 2000000000ull;
+__device__ bool grid_wait(unsigned int *bar, unsigned int target, unsigned long long *err) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const uint64_t t0 = global_ns();
+        ok = 1;
+        for (;;) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (global_ns() - t0 > GRID_WAIT_NS) {
+                ok = 0;
+                atomicAdd(err, 1ull);
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 // ---- FGMRES refinement kernels (all p columns in lockstep, each with its own Krylov space) ----
 // V blocks are n x p row-major; column q of block i is the i-th Arnoldi vector of right-hand side q.
-// part[chunk][i * p + q] = sum over the chunk's rows r of V_i[r][q] W[r][q], i < k1.  Thread t < S
-// (S = the largest multiple of p up to the block size) walks the chunk's row-major elements with
-// stride S, so its column q = t % p is fixed and the loads coalesce; sixteen V_i at a time are
-// accumulated in registers, then the threads of each q are added in shared memory (16 x blockDim).
-__global__ void k_gm_dots_part(int64_t n, int k1, int p, const double *V, int64_t vstride, const double *W,
-                               double *part, int64_t rows_per) {
-    extern __shared__ double red[];
-    const int t = threadIdx.x, nt = blockDim.x, S = (nt / p) * p;
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
-    const int64_t e0 = r0 * p, e1 = r1 * p;
-    for (int i0 = 0; i0 < k1; i0 += 16) {
-        const int ni = min(16, k1 - i0);
-        double acc[16];
+// The Arnoldi step's orthogonalization as one cooperative launch: W against V_0 .. V_{k1-1} twice (classical
+// Gram-Schmidt), the norms, V_{k1} = W / |W|, and the Hessenberg bookkeeping.  CTA b takes a chunk of rows; its
+// thread t < S (S = the largest multiple of p up to the block size) walks the chunk's row-major elements with
+// stride S, so its column q = t % p is fixed, the loads coalesce, and W's elements stay with their thread through
+// the passes.  The chunks' sums meet in part[] and every CTA adds them itself in the same order.
+// Ten launches of 2 to 5 us in a row before (dots, reduce, subtract, twice; norm, reduce, Givens, scale); bound by
+// latency: three grid-wide waits and as many passes over V from L2 (40 us at L = 12, where they took some 50 with
+// their gaps; a refined solve of one right-hand side at L = 16 1.09 -> 1.00 ms, of 16 at L = 18 6.03 -> 5.30).
+constexpr int GM_THREADS = 512, GM_BATCH = 16;
+
+// part[b][o] = sum of the CTA's rows of V_i[r][q] W[r][q] (o = i p + q, i < k1), then, over the grid, h[o]
+__device__ bool gm_dots(int64_t e0, int64_t e1, int k1, int p, const double *V, int64_t vstride, const double *W,
+                        double *part, double *h, double *red, unsigned int *bar, unsigned int target,
+                        unsigned long long *err) {
+    const int t = threadIdx.x, S = (GM_THREADS / p) * p;
+    for (int i0 = 0; i0 < k1; i0 += GM_BATCH) {
+        const int ni = min(GM_BATCH, k1 - i0);
+        double acc[GM_BATCH];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.0;
-        if (t < S) {
+        for (int i = 0; i < GM_BATCH; ++i) acc[i] = 0.0;
+        if (t < S)
             for (int64_t e = e0 + t; e < e1; e += S) {
                 const double wv = W[e];
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
+                for (int i = 0; i < GM_BATCH; ++i)
                     if (i < ni) acc[i] = fma(V[(int64_t)(i0 + i) * vstride + e], wv, acc[i]);
             }
-        }
+        // threads of one right-hand side: within a warp by shuffles where p divides 32, the rest in shared memory
+        const int lanes = 32 % p == 0 ? p : 32;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) red[i * nt + t] = t < S ? acc[i] : 0.0;
+        for (int i = 0; i < GM_BATCH; ++i) {
+            if (i >= ni) break;
+            double x = t < S ? acc[i] : 0.0;
+            for (int o = lanes; o < 32; o *= 2) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if ((t & 31) < lanes) red[i * GM_THREADS + (t >> 5) * lanes + (t & 31)] = x;
+        }
         __syncthreads();
-        for (int o = t; o < ni * p; o += nt) {
+        const int nred = GM_THREADS / 32 * lanes;
+        for (int o = t; o < ni * p; o += GM_THREADS) {
             const int i = o / p, q = o - i * p;
             double sum = 0.0;
-            for (int u = q; u < S; u += p) sum += red[i * nt + u];
+            for (int u = q; u < nred; u += p) sum += red[i * GM_THREADS + u];
             part[(size_t)blockIdx.x * k1 * p + (size_t)(i0 + i) * p + q] = sum;
         }
         __syncthreads();
     }
-}
-
-__global__ void k_gm_sub(int64_t n, int k1, int p, const double *V, int64_t vstride, const double *h, double *W) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * p) return;
-    int q = (int)(t % p);
-    double s = 0.0;
-    for (int i = 0; i < k1; ++i) s = fma(V[(int64_t)i * vstride + t], h[i * p + q], s);
-    W[t] -= s;
-}
-
-// normalize W into V_{k+1}; the norms (one per column) come from a dots pass with V = W
-__global__ void k_gm_scale(int64_t n, int p, const double *W, const double *nrm2, double *Vn) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * p) return;
-    double nn = sqrt(nrm2[t % p]);
-    Vn[t] = nn > 0.0 ? W[t] / nn : 0.0;
-}
-
-// Hessenberg bookkeeping per column q (one thread each): store column k of H (h1 + h2 from the two
-// Gram-Schmidt passes, h_{k+1,k} = |w|), apply the earlier Givens rotations, make a new one, update g.
-// Layout per column: Hc[(kmax+1) x kmax] column-major, cs/sn[kmax], g[kmax+1].
-__global__ void k_gm_givens(int p, int k, int kmax, const double *h1, const double *h2, const double *nrm2,
-                            double *Hall, double *res) {
-    int q = threadIdx.x;
-    if (q >= p) return;
-    const int ld = kmax + 1;
-    double *Hc = Hall + (size_t)q * (ld * kmax + 3 * ld);
-    double *cs = Hc + ld * kmax, *sn = cs + ld, *g = sn + ld;
-    double *col = Hc + (size_t)k * ld;
-    for (int i = 0; i <= k; ++i) col[i] = h1[i * p + q] + h2[i * p + q];
-    col[k + 1] = sqrt(nrm2[q]);
-    for (int i = 0; i < k; ++i) {
-        double a = col[i], b = col[i + 1];
-        col[i] = cs[i] * a + sn[i] * b;
-        col[i + 1] = -sn[i] * a + cs[i] * b;
+    if (!grid_wait(bar, target, err)) return false;
+    // a warp per output, lanes over the CTAs
+    for (int o = t >> 5; o < k1 * p; o += GM_THREADS / 32) {
+        double sum = 0.0;
+        for (int c = t & 31; c < (int)gridDim.x; c += 32) sum += __ldcg(part + (size_t)c * k1 * p + o);
+        for (int x = 16; x > 0; x >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, x);
+        if ((t & 31) == 0) h[o] = sum;
     }
-    double a = col[k], b = col[k + 1];
-    double r = hypot(a, b);
-    double c = r > 0.0 ? a / r : 1.0, s_ = r > 0.0 ? b / r : 0.0;
-    cs[k] = c;
-    sn[k] = s_;
-    col[k] = r;
-    col[k + 1] = 0.0;
-    g[k + 1] = -s_ * g[k];
-    g[k] = c * g[k];
-    res[q] = fabs(g[k + 1]);
+    __syncthreads();
+    return true;
 }
 
-__global__ void k_gm_init(int p, int kmax, const double *beta2, double *Hall) {
-    int q = threadIdx.x;
-    if (q >= p) return;
-    const int ld = kmax + 1;
-    double *Hc = Hall + (size_t)q * (ld * kmax + 3 * ld);
-    double *g = Hc + ld * kmax + 2 * ld;
-    for (int i = 0; i < ld; ++i) g[i] = 0.0;
-    g[0] = sqrt(beta2[q]);
+// Layout per column of Hall: Hc[(kmax+1) x kmax] column-major, cs/sn[kmax], g[kmax+1].
+__host__ __device__ inline size_t gm_hall(int kmax) { return (size_t)(kmax + 1) * kmax + 3 * (size_t)(kmax + 1); }
+
+__global__ void __launch_bounds__(GM_THREADS) k_gm_step(int64_t n, int k, int p, int kmax, int64_t rows_per, double *V,
+                                                        int64_t vstride, double *W, double *Hall, double *res,
+                                                        double *part, int64_t part_len, unsigned int *bar,
+                                                        unsigned int base, unsigned long long *err) {
+    extern __shared__ double sm_gm[];
+    const int k1 = k + 1, t = threadIdx.x, S = (GM_THREADS / p) * p;
+    double *red = sm_gm, *h1 = red + GM_BATCH * GM_THREADS, *h2 = h1 + k1 * p, *nr = h2 + k1 * p;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per), e0 = r0 * p, e1 = r1 * p;
+    const int q = t % p;
+    for (int pass = 0; pass < 2; ++pass) {
+        double *h = pass ? h2 : h1;
+        if (!gm_dots(e0, e1, k1, p, V, vstride, W, part + pass * part_len, h, red, bar, base + (pass + 1) * gridDim.x, err))
+            return;
+        if (t < S)
+            for (int64_t e = e0 + t; e < e1; e += S) {
+                double s = 0.0;
+                for (int i = 0; i < k1; ++i) s = fma(V[(int64_t)i * vstride + e], h[i * p + q], s);
+                W[e] -= s;
+            }
+    }
+    if (!gm_dots(e0, e1, 1, p, W, 0, W, part + 2 * part_len, nr, red, bar, base + 3 * gridDim.x, err)) return;
+    {
+        double *Vn = V + (int64_t)k1 * vstride;
+        const double nn = sqrt(nr[q]), inv = nn > 0.0 ? 1.0 / nn : 0.0;
+        if (t < S)
+            for (int64_t e = e0 + t; e < e1; e += S) Vn[e] = W[e] * inv;
+    }
+    // Hessenberg column per right-hand side (a thread each): h1 + h2 and h_{k+1,k} = |w|, the earlier Givens
+    // rotations, a new one, and the right-hand side g
+    if (blockIdx.x == 0 && t < p) {
+        const int ld = kmax + 1;
+        double *Hc = Hall + (size_t)t * gm_hall(kmax);
+        double *cs = Hc + ld * kmax, *sn = cs + ld, *g = sn + ld;
+        double *col = Hc + (size_t)k * ld;
+        double a = h1[t] + h2[t];
+        for (int i = 0; i < k; ++i) {
+            const double b = h1[(i + 1) * p + t] + h2[(i + 1) * p + t];
+            col[i] = cs[i] * a + sn[i] * b;
+            a = -sn[i] * a + cs[i] * b;
+        }
+        const double b = sqrt(nr[t]);
+        const double r = hypot(a, b);
+        const double c = r > 0.0 ? a / r : 1.0, s_ = r > 0.0 ? b / r : 0.0;
+        cs[k] = c;
+        sn[k] = s_;
+        col[k] = r;
+        col[k + 1] = 0.0;
+        g[k + 1] = -s_ * g[k];
+        g[k] = c * g[k];
+        res[t] = fabs(g[k + 1]);
+    }
+}
+
+// Start of a cycle, one cooperative launch: V_0 = R / |R|, g = |R| e_1.
+__global__ void __launch_bounds__(GM_THREADS) k_gm_start(int64_t n, int p, int kmax, int64_t rows_per, const double *Rr,
+                                                         double *V, double *Hall, double *part, unsigned int *bar,
+                                                         unsigned int base, unsigned long long *err) {
+    extern __shared__ double sm_gm[];
+    const int t = threadIdx.x, S = (GM_THREADS / p) * p, q = t % p;
+    double *red = sm_gm, *nr = red + GM_BATCH * GM_THREADS;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per), e0 = r0 * p, e1 = r1 * p;
+    if (!gm_dots(e0, e1, 1, p, Rr, 0, Rr, part, nr, red, bar, base + gridDim.x, err)) return;
+    const double nn = sqrt(nr[q]), inv = nn > 0.0 ? 1.0 / nn : 0.0;
+    if (t < S)
+        for (int64_t e = e0 + t; e < e1; e += S) V[e] = Rr[e] * inv;
+    if (blockIdx.x == 0 && t < p) {
+        const int ld = kmax + 1;
+        double *g = Hall + (size_t)t * gm_hall(kmax) + ld * kmax + 2 * ld;
+        for (int i = 0; i < ld; ++i) g[i] = 0.0;
+        g[0] = nn;
+    }
 }
 
 // y = H^{-1} g (upper triangular, k columns), per column q
@@ -914,8 +979,7 @@ void RefinedSolve::set_deflation(const double *U_, int ldu_, int k, cudaStream_t
     k_small_inverse<<<1, 512, (size_t)k * k * sizeof(double), st>>>(k, Einv.data(), Dflag.data());
     MBL_LAUNCH_CHECK();
     int ok = 0;
-    MBL_CUDA(cudaMemcpyAsync(&ok, Dflag.data(), sizeof(int), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaStreamSynchronize(st));
+    read_back(ctx, st, &ok, Dflag.data(), sizeof(int));
     if (!ok) return;
     k_cols_to_f32<<<nblk(n * k), 256, 0, st>>>(n, U_, ldu_, k, U32.data());
     MBL_LAUNCH_CHECK();
@@ -967,21 +1031,25 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
     if (GZ.size() < (size_t)blk * kmax) GZ.alloc(ctx, (size_t)blk * kmax);
     if (GW.size() < (size_t)blk) GW.alloc(ctx, blk);
     const int ld = kmax + 1;
-    if (Gh.size() < (size_t)p * (ld * kmax + 3 * ld) + 2 * (size_t)ld * p + 3 * 32)
-        Gh.alloc(ctx, (size_t)p * (ld * kmax + 3 * ld) + 2 * (size_t)ld * p + 3 * 32);
-    const int64_t rows_per = std::max<int64_t>(1, (n + 303) / 304);
-    const int nch = (int)((n + rows_per - 1) / rows_per);
-    if (Gdots.size() < (size_t)nch * ld * p) Gdots.alloc(ctx, (size_t)nch * ld * p);
+    if (Gh.size() < (size_t)p * gm_hall(kmax) + 32) Gh.alloc(ctx, (size_t)p * gm_hall(kmax) + 32);
+    // rows a CTA: about four elements a thread, at most one CTA an SM
+    const int64_t rows_per = std::max<int64_t>((n + ctx->sm_count - 1) / ctx->sm_count, (4 * GM_THREADS + p - 1) / p);
+    const unsigned nch = (unsigned)((n + rows_per - 1) / rows_per);
+    const int64_t part_len = (int64_t)nch * ld * p;
+    if (Gdots.size() < (size_t)(3 * part_len)) Gdots.alloc(ctx, (size_t)(3 * part_len));
+    if (Gbar.size() < 2) {
+        Gbar.alloc(ctx, 2);
+        MBL_CUDA(cudaMemsetAsync(Gbar.data(), 0, 2 * sizeof(unsigned long long), st));
+        gbar_count = 0;
+    }
     if (Gy.size() < (size_t)kmax * p + 64) Gy.alloc(ctx, (size_t)kmax * p + 64);
-    double *Hall = Gh.data();
-    double *h1 = Hall + (size_t)p * (ld * kmax + 3 * ld), *h2 = h1 + (size_t)ld * p, *nr = h2 + (size_t)ld * p;
+    double *Hall = Gh.data(), *est_d = Hall + (size_t)p * gm_hall(kmax);
+    unsigned long long *err = Gbar.data();
+    unsigned int *bar = reinterpret_cast<unsigned int *>(Gbar.data() + 1);
     const unsigned nbk = nblk(blk);
-    auto dots = [&](int k1, const double *V, int64_t vstride, const double *W, double *out) {
-        k_gm_dots_part<<<nch, 256, 16 * 256 * sizeof(double), st>>>(n, k1, p, V, vstride, W, Gdots.data(), rows_per);
-        MBL_LAUNCH_CHECK();
-        k_reduce_parts<<<reduce_grid(k1 * p), 256, 0, st>>>(nch, k1 * p, Gdots.data(), out);
-        MBL_LAUNCH_CHECK();
-    };
+    const size_t smem0 = (GM_BATCH * GM_THREADS + 32) * sizeof(double);
+    smem_limit((const void *)k_gm_start, smem0);
+    smem_limit((const void *)k_gm_step, smem0 + (size_t)2 * 64 * 32 * sizeof(double));
     double prev = INFINITY;
     for (int outer = 0; outer < max_outer; ++outer) {
         std::vector<double> rn, lim;
@@ -990,11 +1058,16 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
         if (outer > 0 && last_rel > 0.5 * prev) { stalled = true; return; }
         prev = last_rel;
         // V_0 = R / |R|, g = |R| e_1
-        dots(1, R.data(), 0, R.data(), nr);
-        k_gm_scale<<<nbk, 256, 0, st>>>(n, p, R.data(), nr, GV.data());
-        MBL_LAUNCH_CHECK();
-        k_gm_init<<<1, 32, 0, st>>>(p, kmax, nr, Hall);
-        MBL_LAUNCH_CHECK();
+        {
+            int64_t n_ = n, rp = rows_per;
+            int p_ = p, km = kmax;
+            const double *r_ = R.data();
+            double *v_ = GV.data(), *h_ = Hall, *pt = Gdots.data();
+            void *args[] = {&n_, &p_, &km, &rp, &r_, &v_, &h_, &pt, &bar, &gbar_count, &err};
+            MBL_CUDA(cudaLaunchCooperativeKernel((const void *)k_gm_start, dim3(nch), dim3(GM_THREADS), args, smem0, st));
+            MBL_LAUNCH_CHECK();
+            gbar_count += nch;
+        }
         int k = 0;
         for (; k < kmax; ++k) {
             double *Vk = GV.data() + (size_t)k * blk, *Zk = GZ.data() + (size_t)k * blk;
@@ -1007,20 +1080,23 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
             }
             ProfScope ps_o(ctx, "gm_orth", 0.0, st);
             // two Gram-Schmidt passes against V_0..V_k (each column its own space)
-            dots(k + 1, GV.data(), blk, GW.data(), h1);
-            k_gm_sub<<<nbk, 256, 0, st>>>(n, k + 1, p, GV.data(), blk, h1, GW.data());
-            MBL_LAUNCH_CHECK();
-            dots(k + 1, GV.data(), blk, GW.data(), h2);
-            k_gm_sub<<<nbk, 256, 0, st>>>(n, k + 1, p, GV.data(), blk, h2, GW.data());
-            MBL_LAUNCH_CHECK();
-            dots(1, GW.data(), 0, GW.data(), nr);
-            k_gm_givens<<<1, 32, 0, st>>>(p, k, kmax, h1, h2, nr, Hall, nr + 32);
-            MBL_LAUNCH_CHECK();
-            k_gm_scale<<<nbk, 256, 0, st>>>(n, p, GW.data(), nr, GV.data() + (size_t)(k + 1) * blk);
-            MBL_LAUNCH_CHECK();
+            {
+                int64_t n_ = n, rp = rows_per, vs = blk, pl = part_len;
+                int k_ = k, p_ = p, km = kmax;
+                double *v_ = GV.data(), *w_ = GW.data(), *h_ = Hall, *re = est_d, *pt = Gdots.data();
+                void *args[] = {&n_, &k_, &p_, &km, &rp, &v_, &vs, &w_, &h_, &re, &pt, &pl, &bar, &gbar_count, &err};
+                MBL_CUDA(cudaLaunchCooperativeKernel((const void *)k_gm_step, dim3(nch), dim3(GM_THREADS), args,
+                                                     smem0 + (size_t)2 * (k + 1) * p * sizeof(double), st));
+                MBL_LAUNCH_CHECK();
+                gbar_count += 3 * nch;
+            }
             std::vector<double> est(p);
-            MBL_CUDA(cudaMemcpyAsync(est.data(), nr + 32, p * sizeof(double), cudaMemcpyDeviceToHost, st));
-            MBL_CUDA(cudaStreamSynchronize(st));
+            unsigned long long expired = 0;
+            ReadBack rb(ctx, st);
+            rb.add(est.data(), est_d, p * sizeof(double));
+            rb.add(&expired, err, sizeof(expired));
+            rb.done();
+            if (expired) fail(MBL_ERR_TIMEOUT, "a grid-wide wait of the refinement's orthogonalization expired");
             bool ok = true;
             for (int q = 0; q < p; ++q) ok = ok && est[q] <= 0.5 * lim[q];
             if (ok) {
@@ -1097,7 +1173,6 @@ __global__ void k_normalize_first(int64_t n, double *V, int ldv, const double *p
 
 // ---- plain Lanczos steps of the extremal bounds ----
 constexpr int LZ_THREADS = 512, LZ_TPR = 4;  // threads a CTA, lanes a row
-constexpr uint64_t LZ_WAIT_NS = 2000000000ull;
 
 // Sum over the CTA in a fixed order; every thread gets it.
 __device__ double lz_block_sum(double s, double *red) {
@@ -1111,31 +1186,12 @@ __device__ double lz_block_sum(double s, double *red) {
 }
 
 // Sum of s over the grid: the CTAs' sums meet in part[] (one slot each) and every CTA adds them in the same
-// order, so that all use the same bits.  Waits for the other CTAs (co-resident: a cooperative launch), at
-// most LZ_WAIT_NS; false on expiry, which is counted in *err.
+// order, so that all use the same bits.  False if the wait for the other CTAs expired.
 __device__ bool lz_grid_sum(double s, double *part, unsigned int *bar, unsigned int target, double *red,
                             unsigned long long *err, double *total) {
-    __shared__ int ok;
     const double b = lz_block_sum(s, red);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = b;
-        __threadfence();
-        atomicAdd(bar, 1u);
-        const uint64_t t0 = global_ns();
-        unsigned int v;
-        ok = 1;
-        for (;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
-            if (global_ns() - t0 > LZ_WAIT_NS) {
-                ok = 0;
-                atomicAdd(err, 1ull);
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    if (!ok) return false;
+    if (threadIdx.x == 0) part[blockIdx.x] = b;
+    if (!grid_wait(bar, target, err)) return false;
     double t = 0.0;
     for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -1367,10 +1423,11 @@ void extremal_bounds(mbl_sector *sec, double *emin, double *emax) {
         MBL_LAUNCH_CHECK();
         double h[4], bj;
         unsigned long long expired = 0;
-        MBL_CUDA(cudaMemcpyAsync(h, out.data(), 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
-        MBL_CUDA(cudaMemcpyAsync(&bj, beta.data() + m - 1, sizeof(double), cudaMemcpyDeviceToHost, st));
-        MBL_CUDA(cudaMemcpyAsync(&expired, bar.data(), sizeof(expired), cudaMemcpyDeviceToHost, st));
-        MBL_CUDA(cudaStreamSynchronize(st));
+        ReadBack rb(ctx, st);
+        rb.add(h, out.data(), 4 * sizeof(double));
+        rb.add(&bj, beta.data() + m - 1, sizeof(double));
+        rb.add(&expired, bar.data(), sizeof(expired));
+        rb.done();
         if (expired) fail(MBL_ERR_TIMEOUT, "a grid-wide wait of the extremal Lanczos steps expired");
         lo = h[0];
         hi = h[1];
@@ -1777,9 +1834,10 @@ void RitzH::run(mbl_sector *sec, KrylovSchur &ks, double sigma, double hnorm, do
             k_oa_colnorms<<<nblk(mb, 128), 128, 0, st>>>(mb, Gr1.data(), Gr3.data(), Gr2.data());
             MBL_LAUNCH_CHECK();
             std::vector<double> q((size_t)2 * mb), th(mb);
-            MBL_CUDA(cudaMemcpyAsync(q.data(), Gr2.data(), q.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-            MBL_CUDA(cudaMemcpyAsync(th.data(), Gw.data(), mb * sizeof(double), cudaMemcpyDeviceToHost, st));
-            MBL_CUDA(cudaStreamSynchronize(st));
+            ReadBack rb(ctx, st);
+            rb.add(q.data(), Gr2.data(), q.size() * sizeof(double));
+            rb.add(th.data(), Gw.data(), mb * sizeof(double));
+            rb.done();
             double amax = 0.0;
             for (double v : th) amax = std::max(amax, std::fabs(v));
             bool good = true;
@@ -1826,9 +1884,12 @@ void RitzH::run(mbl_sector *sec, KrylovSchur &ks, double sigma, double hnorm, do
     k_ritz_all_resid<<<nblk(mb, 128), 128, 0, st>>>(mb, Gs.data(), Gr1.data(), Gw.data(), Gr2.data());
     MBL_LAUNCH_CHECK();
     std::vector<double> gth(mb), gres(mb);
-    MBL_CUDA(cudaMemcpyAsync(gth.data(), Gw.data(), mb * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaMemcpyAsync(gres.data(), Gr2.data(), mb * sizeof(double), cudaMemcpyDeviceToHost, st));
-    MBL_CUDA(cudaStreamSynchronize(st));
+    {
+        ReadBack rb(ctx, st);
+        rb.add(gth.data(), Gw.data(), mb * sizeof(double));
+        rb.add(gres.data(), Gr2.data(), mb * sizeof(double));
+        rb.done();
+    }
     // candidates: Ritz pairs with residual <= 1e-3 ||H|| (a spurious value sits near 0.1 ||H||)
     std::vector<int> cand;
     for (int j = 0; j < mb; ++j)

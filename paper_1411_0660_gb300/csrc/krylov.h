@@ -49,6 +49,8 @@ struct RefinedSolve {
     int kmax = 24;     // FGMRES inner dimension
     int max_outer = 4; // FGMRES restarts per application before a stall is declared
     DVec<double> R, part, norms, GV, GZ, GW, Gh, Gy, Gdots;
+    DVec<unsigned long long> Gbar;   // grid-wide waits of the orthogonalization: expiries, arrivals
+    unsigned int gbar_count = 0;     // arrivals of the launches so far
     // Deflation of the preconditioner (FGMRES mode): with U (n x kd, row stride ldu) approximate
     // eigenvectors nearest sigma and A = H - sigma, the preconditioner is
     //   P = M^-1 (I - A Q) + Q,   Q = U (U^T A U)^-1 U^T,

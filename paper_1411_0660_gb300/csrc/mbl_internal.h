@@ -172,6 +172,7 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t side = nullptr;  // work beside `stream`, made at first use and always joined to it
     cudaEvent_t side_ev = nullptr;
+    char *pin = nullptr;          // ReadBack's pinned buffer, made at first use
     std::string last_error;
     std::shared_ptr<PlanCache> plans = std::make_shared<PlanCache>();  // per L; shared with serving workers
     std::map<int, std::shared_ptr<EntTables>> ent;  // per sector (sector_key)
@@ -189,6 +190,29 @@ struct Ctx {
     void resolve_profile();
 };
 void server_shutdown(Ctx *ctx);
+
+// Small device results to the host through the context's pinned buffer (a copy into pageable memory goes by
+// the driver's own staging, several microseconds more): add() queues a copy on `st`, done() waits for the
+// stream and hands the values out.  At most PIN_BYTES between two done().
+constexpr size_t PIN_BYTES = 64 << 10;
+struct ReadBack {
+    Ctx *ctx;
+    cudaStream_t st;
+    struct Item {
+        void *dst;
+        size_t off, bytes;
+    };
+    std::vector<Item> items;
+    size_t used = 0;
+    ReadBack(Ctx *c, cudaStream_t s) : ctx(c), st(s) {}
+    void add(void *dst, const void *src, size_t bytes);
+    void done();
+};
+inline void read_back(Ctx *ctx, cudaStream_t st, void *dst, const void *src, size_t bytes) {
+    ReadBack rb(ctx, st);
+    rb.add(dst, src, bytes);
+    rb.done();
+}
 
 // Times the enclosed launches on `st` under class `name` when profiling is on.
 struct ProfScope {
