@@ -317,22 +317,16 @@ __device__ int sturm_count(int m, const R *d, const R *e2, R x, R pivmin) {
 // c, s, r of the rotation that takes (x, z) to (r, 0): FP32 by the reciprocal square root and one Newton
 // step (a chain of some 60 clocks against 200 of hypotf and a division)
 __device__ __forceinline__ void ql_rotation(float x, float z, float &c, float &s, float &r) {
+    // (no branch on the chain: the pair is far below the matrix' rounding where r2 underflows; the matrices solved
+    // here, projections of (H - sigma)^-1 and H, are far from the overflow of their squares)
     const float r2 = fmaf(x, x, z * z);
-    if (r2 > 1e-30f && r2 < 1e30f) {
-        float ir = rsqrtf(r2);
-        ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.0f), ir);
-        c = x * ir;
-        s = z * ir;
-        r = r2 * ir;
-        return;
-    }
-    r = hypotf(x, z);
-    c = 1.0f;
-    s = 0.0f;
-    if (r != 0.0f) {
-        c = x / r;
-        s = z / r;
-    }
+    float ir;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(fmaxf(r2, 1e-37f)));
+    ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.0f), ir);
+    const bool in = r2 > 1e-37f;
+    c = in ? x * ir : 1.0f;
+    s = in ? z * ir : 0.0f;
+    r = in ? r2 * ir : 0.0f;
 }
 __device__ __forceinline__ void ql_rotation(double x, double z, double &c, double &s, double &r) {
     r = hypot(x, z);
@@ -354,7 +348,7 @@ __device__ __forceinline__ void ql_rotation(double x, double z, double &c, doubl
 // entries it meets for the first time, d[k] and e[k - 1], one rotation ahead, and stores each final
 // value once.  The arithmetic, and so every result, is the same as with d and e updated in place.
 template <class R>
-__device__ void ql_sweep_record(int lo, int hi, R *d, R *e, R *cs, R *sn) {
+__device__ __forceinline__ void ql_sweep_record(int lo, int hi, R *d, R *e, R *cs, R *sn) {
     R delta = R(0.5) * (d[lo + 1] - d[lo]);
     R b = e[lo];
     R mu = d[lo] - b * b / (delta + copysign(hypot(delta, b), delta));
@@ -599,83 +593,88 @@ __global__ void __launch_bounds__(EIG_THREADS) k_syev(const int *mv, const int64
                 q_d[i] = d[i];
                 q_e[i] = e[i];
             }
-            d = q_d;
-            e = q_e;
         }
-        R *csb[2] = {qsm ? q_cs[0] : work + 3 * m, qsm ? q_cs[1] : work + 5 * m};  // (vv and e2 are free now)
-        R *snb[2] = {qsm ? q_sn[0] : work + 6 * m, qsm ? q_sn[1] : work + 7 * m};
         for (int t = threadIdx.x; t < m * m; t += blockDim.x) Z[t] = ((t / m) == (t % m)) ? R(1) : R(0);
         if (threadIdx.x == 0) s_fail = 0;
         __syncthreads();
-        const int lane = threadIdx.x & 31;
-        int iter = 0, nlo = 0;  // (warp 0)
-        for (int buf = 0;; buf ^= 1) {
-            if (threadIdx.x < 32) {
-                // first entry of e at or after `from` that is negligible (want = true) or not, else m - 1
-                auto scan = [&](int from, bool want) {
-                    for (int k0 = from; k0 < m - 1; k0 += 32) {
-                        const int k = k0 + lane;
-                        const bool small = k < m - 1 && fabs(e[k]) <= Num<R>::eps() * (fabs(d[k]) + fabs(d[k + 1]));
-                        const unsigned int hit = __ballot_sync(0xffffffffu, k < m - 1 && small == want);
-                        if (hit) return k0 + __ffs(hit) - 1;
+        // (inlined with the shared arrays themselves, so that the chain's accesses are shared-memory ones)
+        auto sweeps = [&](R *d, R *e, R *cs0, R *cs1, R *sn0, R *sn1) {
+            const int lane = threadIdx.x & 31;
+            int iter = 0, nlo = 0;  // (warp 0)
+            for (int buf = 0;; buf ^= 1) {
+                if (threadIdx.x < 32) {
+                    // first entry of e at or after `from` that is negligible (want = true) or not, else m - 1
+                    auto scan = [&](int from, bool want) {
+                        for (int k0 = from; k0 < m - 1; k0 += 32) {
+                            const int k = k0 + lane;
+                            const bool small = k < m - 1 && fabs(e[k]) <= Num<R>::eps() * (fabs(d[k]) + fabs(d[k + 1]));
+                            const unsigned int hit = __ballot_sync(0xffffffffu, k < m - 1 && small == want);
+                            if (hit) return k0 + __ffs(hit) - 1;
+                        }
+                        return m - 1;
+                    };
+                    const int lo = scan(nlo, false);
+                    if (lo != nlo) {
+                        for (int k = nlo + lane; k < lo; k += 32) e[k] = R(0);
+                        iter = 0;
+                        nlo = lo;
                     }
-                    return m - 1;
-                };
-                const int lo = scan(nlo, false);
-                if (lo != nlo) {
-                    for (int k = nlo + lane; k < lo; k += 32) e[k] = R(0);
-                    iter = 0;
-                    nlo = lo;
+                    int hi = -1;
+                    bool done = lo >= m - 1;
+                    if (!done) {
+                        hi = scan(lo + 1, true);
+                        if (++iter > 100) {
+                            done = true;
+                            hi = -1;
+                            if (lane == 0) s_fail = 1;
+                        } else if (lane == 0) {
+                            if (hi < m - 1) e[hi] = R(0);
+                            ql_sweep_record(lo, hi, d, e, buf ? cs1 : cs0, buf ? sn1 : sn0);
+                        }
+                    }
+                    if (lane == 0) {
+                        s_lo[buf] = lo;
+                        s_hi[buf] = hi;
+                        s_done[buf] = done;
+                    }
+                    __syncwarp();
                 }
-                int hi = -1;
-                bool done = lo >= m - 1;
-                if (!done) {
-                    hi = scan(lo + 1, true);
-                    if (++iter > 100) {
-                        done = true;
-                        hi = -1;
-                        if (lane == 0) s_fail = 1;
-                    } else if (lane == 0) {
-                        if (hi < m - 1) e[hi] = R(0);
-                        ql_sweep_record(lo, hi, d, e, csb[buf], snb[buf]);
+                __syncthreads();
+                // this sweep is applied while warp 0 generates the next one into the other list (which the
+                // previous sweep's application left before this barrier)
+                const int lo = s_lo[buf], hi = s_hi[buf];
+                if (threadIdx.x >= 32 && hi >= 0) {
+                    const R *c_ = buf ? cs1 : cs0, *s_ = buf ? sn1 : sn0;
+                    // Z is column-major (column k contiguous): a thread walks its row down the sweep,
+                    // carrying the rotated entry of column k + 1; accesses coalesce across threads
+                    // (the next rotation's inputs are loaded before this one's store, which the compiler
+                    // could not otherwise move ahead of it: Z and the rotation list might alias)
+                    for (int r = (int)threadIdx.x - 32; r < m; r += (int)blockDim.x - 32) {
+                        R a1 = Z[(size_t)hi * m + r];
+                        R a0 = Z[(size_t)(hi - 1) * m + r];
+                        R c = c_[hi - 1], sv = s_[hi - 1];
+                        for (int k = hi - 1; k >= lo; --k) {
+                            const bool more = k > lo;
+                            const R a0n = more ? Z[(size_t)(k - 1) * m + r] : R(0);
+                            const R cn = more ? c_[k - 1] : R(0), svn = more ? s_[k - 1] : R(0);
+                            Z[(size_t)(k + 1) * m + r] = sv * a0 + c * a1;
+                            a1 = c * a0 - sv * a1;
+                            a0 = a0n;
+                            c = cn;
+                            sv = svn;
+                        }
+                        Z[(size_t)lo * m + r] = a1;
                     }
                 }
-                if (lane == 0) {
-                    s_lo[buf] = lo;
-                    s_hi[buf] = hi;
-                    s_done[buf] = done;
-                }
-                __syncwarp();
+                if (s_done[buf]) break;  // (no sweep was recorded with it; uniform: written before the barrier,
+                                         // and next rewritten two sweeps later)
             }
-            __syncthreads();
-            // this sweep is applied while warp 0 generates the next one into the other list (which the
-            // previous sweep's application left before this barrier)
-            const int lo = s_lo[buf], hi = s_hi[buf];
-            if (threadIdx.x >= 32 && hi >= 0) {
-                const R *c_ = csb[buf], *s_ = snb[buf];
-                // Z is column-major (column k contiguous): a thread walks its row down the sweep,
-                // carrying the rotated entry of column k + 1; accesses coalesce across threads
-                // (the next rotation's inputs are loaded before this one's store, which the compiler
-                // could not otherwise move ahead of it: Z and the rotation list might alias)
-                for (int r = (int)threadIdx.x - 32; r < m; r += (int)blockDim.x - 32) {
-                    R a1 = Z[(size_t)hi * m + r];
-                    R a0 = Z[(size_t)(hi - 1) * m + r];
-                    R c = c_[hi - 1], sv = s_[hi - 1];
-                    for (int k = hi - 1; k >= lo; --k) {
-                        const bool more = k > lo;
-                        const R a0n = more ? Z[(size_t)(k - 1) * m + r] : R(0);
-                        const R cn = more ? c_[k - 1] : R(0), svn = more ? s_[k - 1] : R(0);
-                        Z[(size_t)(k + 1) * m + r] = sv * a0 + c * a1;
-                        a1 = c * a0 - sv * a1;
-                        a0 = a0n;
-                        c = cn;
-                        sv = svn;
-                    }
-                    Z[(size_t)lo * m + r] = a1;
-                }
-            }
-            if (s_done[buf]) break;  // (no sweep was recorded with it; uniform: written before the barrier,
-                                     // and next rewritten two sweeps later)
+        };
+        if (qsm) {
+            sweeps(q_d, q_e, q_cs[0], q_cs[1], q_sn[0], q_sn[1]);
+            d = q_d;
+        } else {
+            sweeps(d, e, work + 3 * m, work + 5 * m, work + 6 * m, work + 7 * m);  // (vv and e2 are free now)
         }
         __syncthreads();
         // ascending order: the rank of each eigenvalue (ties by index); cs[rank] = its column of Z
