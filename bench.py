@@ -118,6 +118,8 @@ _ordering = 3
 
 def _context(device):
     """A library context whose symbolic analyses use the ordering chosen on the command line."""
+    import paper_1411_0660_gb300 as g
+
     ctx = g.Context(device)
     ctx.set_ordering(_ordering)
     return ctx
