@@ -1818,10 +1818,11 @@ void RitzH::run(mbl_sector *sec, KrylovSchur &ks, double sigma, double hnorm, do
     MBL_LAUNCH_CHECK();
     MBL_CUDA(cudaMemcpyAsync(gm.data(), &mb, sizeof(int), cudaMemcpyHostToDevice, st));
     {
-        // FP32 eigensolve (the parallel Jacobi method) refined by three Ogita-Aishima steps and
-        // re-orthonormalized (Newton-Schulz) in FP64; accepted only if the nev wanted columns are
-        // orthonormal and diagonalize G to FP64 accuracy, otherwise FP64 bisection and inverse
-        // iteration run.  The pairs' residuals on H are recomputed below.
+        // FP32 eigensolve (the QL sweeps; 1.6 ms at m = 124, the parallel Jacobi method took 2.8) refined by three
+        // Ogita-Aishima steps and re-orthonormalized (Newton-Schulz) in FP64; accepted only if the nev
+        // wanted columns are orthonormal and diagonalize G to FP64 accuracy, otherwise refined again and then
+        // FP64 bisection and inverse iteration run.  The pairs' residuals on H are recomputed below.
+        // (An FP32 Jacobi start, unchecked here, left an L = 16 job at 48 of 50 pairs.)
         ProfScope ps(ctx, "syev_rr", (double)mb, st);
         const bool fp32 = ks.ldv <= EIG_SMEM_MAX_M;
         // accept eigenvectors X (in Gs) only if the nev wanted columns are orthonormal and diagonalize
@@ -1848,15 +1849,19 @@ void RitzH::run(mbl_sector *sec, KrylovSchur &ks, double sigma, double hnorm, do
         if (fp32) {
             MBL_CUDA(cudaMemcpyAsync(Gsym.data(), Gs.data(), (size_t)mb * mb * sizeof(double), cudaMemcpyDeviceToDevice,
                                      st));
-            syev_jacobi32(1, gm.data(), goff.data(), goff.data(), Gs.data(), Gw.data(), ks.ldv, ginfo.data(), st);
-            refine_eig(mb, Gsym.data(), Gs.data(), Gw.data(), 3, Gr1.data(), Gr2.data(), Gr3.data(), st);
-            for (int it = 0; it < 2; ++it) {  // X <- 1.5 X - 0.5 X (X^T X)
-                gemm_small(true, false, mb, mb, mb, 1.0, Gs.data(), mb, Gs.data(), mb, 0.0, Gr1.data(), mb, st);
-                MBL_CUDA(cudaMemcpyAsync(Gr2.data(), Gs.data(), (size_t)mb * mb * sizeof(double),
-                                         cudaMemcpyDeviceToDevice, st));
-                gemm_small(false, false, mb, mb, mb, -0.5, Gr2.data(), mb, Gr1.data(), mb, 1.5, Gs.data(), mb, st);
+            syev_batched(1, gm.data(), goff.data(), goff.data(), Gs.data(), Gw.data(), 1, nullptr, ks.ldv, Gwork.data(),
+                         ginfo.data(), st, true);
+            // (two more steps where eigenvalues closer than the start's error needed the first to part)
+            for (int steps = 3; steps >= 2 && !ok; --steps) {
+                refine_eig(mb, Gsym.data(), Gs.data(), Gw.data(), steps, Gr1.data(), Gr2.data(), Gr3.data(), st);
+                for (int it = 0; it < 2; ++it) {  // X <- 1.5 X - 0.5 X (X^T X)
+                    gemm_small(true, false, mb, mb, mb, 1.0, Gs.data(), mb, Gs.data(), mb, 0.0, Gr1.data(), mb, st);
+                    MBL_CUDA(cudaMemcpyAsync(Gr2.data(), Gs.data(), (size_t)mb * mb * sizeof(double),
+                                             cudaMemcpyDeviceToDevice, st));
+                    gemm_small(false, false, mb, mb, mb, -0.5, Gr2.data(), mb, Gr1.data(), mb, 1.5, Gs.data(), mb, st);
+                }
+                ok = check_wanted();
             }
-            ok = check_wanted();
             if (!ok) {
                 // FP64 by bisection and inverse iteration, under the same check
                 ProfScope ps2(ctx, "syev_rr_bisect", (double)mb, st);
