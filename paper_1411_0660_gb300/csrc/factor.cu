@@ -873,15 +873,16 @@ __device__ __forceinline__ void fwd_tile_issue(T *Gs, const T *G, int64_t ld, in
 template <class T, int PB>
 __global__ void __launch_bounds__(256, PB <= 8 ? 4 : 2)
     k_fwd_step(const SolveDesc *sdescs, const int32_t *blk_desc, int nrb, int K, const int64_t *zo,
-               const int32_t *sn_start, const SolveBufs<T> *jb, int p, LaunchTrace *tr) {
+               const int32_t *sn_start, const SolveBufs<T> *jb, int p, LaunchTrace *tr, bool early) {
     static_assert(SPW == 256 && RBF == 32, "eight warps of 32 columns, a lane per row");
     TraceScope trace_scope(tr);
     extern __shared__ __align__(16) unsigned char smraw[];
     T *Gs = reinterpret_cast<T *>(smraw);                         // SPW columns x RBF rows
     T *zp = reinterpret_cast<T *>(smraw + fwd_gtile_bytes<T>());  // SPW x PB
-    T *red = Gs;                                                  // 8 x PB x RBF partials, after the products
+    T *red = Gs;                                                  // 8 x RBF x (PB + 4) partials, after the products
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int nit = nrb * K;
+    if (early) pdl_trigger();
     bool waited = false;
     for (int it = blockIdx.x; it < nit; it += gridDim.x) {
         const int job = it / nrb, b = it - job * nrb;
@@ -893,27 +894,24 @@ __global__ void __launch_bounds__(256, PB <= 8 ? 4 : 2)
         const int nr = min(RBF, R - r0);
         const int64_t zb = zo[s] + k0, ld = sg_ld(R);
         fwd_tile_issue(Gs, J.G + d.goff + r0, ld, w, (int)(ld - r0));
-        // this thread's outputs o = threadIdx.x + 256 u (row i = o % RBF, right-hand side q = o / RBF)
-        constexpr int NO = RBF * PB / 256;
-        static_assert(NO * 256 == RBF * PB, "outputs per thread");
+        // this thread's outputs o = threadIdx.x + 256 u (row i = o / PB, right-hand side q = o % PB)
+        constexpr int NO = RBF * PB / 256, LDR = PB + 4;
+        static_assert(NO * 256 == RBF * PB && 8 * RBF * LDR <= SPW * (RBF + PB), "outputs per thread; partials fit");
         T dg[NO], zold[NO];
 #pragma unroll
         for (int u = 0; u < NO; ++u) {
-            const int o = threadIdx.x + 256 * u, i = o % RBF, q = o / RBF, rr = r0 + i;
+            const int o = threadIdx.x + 256 * u, i = o / PB, q = o % PB, rr = r0 + i;
             dg[u] = (i < nr && q < p && rr < w) ? J.D[(int64_t)sn_start[s] + k0 + rr] : T(1);
         }
         if (!waited) {
             pdl_wait();
-            pdl_trigger();
+            if (!early) pdl_trigger();
             waited = true;
         }
-        for (int idx = threadIdx.x; idx < w * PB; idx += blockDim.x) {
-            const int c = idx / PB, q = idx % PB;
-            zp[idx] = q < p ? J.Z[(zb + c) * p + q] : T(0);
-        }
+        stage_rows<T, PB>(zp, J.Z + zb * p, w, p);
 #pragma unroll
         for (int u = 0; u < NO; ++u) {
-            const int o = threadIdx.x + 256 * u, i = o % RBF, q = o / RBF, rr = r0 + i;
+            const int o = threadIdx.x + 256 * u, i = o / PB, q = o % PB, rr = r0 + i;
             zold[u] = (i < nr && q < p && rr >= w) ? J.Z[(zb + rr) * p + q] : T(0);
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -924,6 +922,7 @@ __global__ void __launch_bounds__(256, PB <= 8 ? 4 : 2)
         {
             const int c0 = wp * 32, c1 = min(w, c0 + 32);
             if (lane < nr) {
+#pragma unroll 8
                 for (int c = c0; c < c1; ++c) {
                     const T l = Gs[c * RBF + lane];
 #pragma unroll
@@ -933,15 +932,15 @@ __global__ void __launch_bounds__(256, PB <= 8 ? 4 : 2)
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < PB; ++q) red[(wp * PB + q) * RBF + lane] = acc[q];
+        for (int q = 0; q < PB; q += 16 / (int)sizeof(T)) Vec16<T>::put(red + (wp * RBF + lane) * LDR + q, acc + q);
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < NO; ++u) {
-            const int o = threadIdx.x + 256 * u, i = o % RBF, q = o / RBF;
+            const int o = threadIdx.x + 256 * u, i = o / PB, q = o % PB;
             if (i >= nr || q >= p) continue;
             T v = T(0);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v += red[(j * PB + q) * RBF + i];
+            for (int j = 0; j < 8; ++j) v += red[(j * RBF + i) * LDR + q];
             const int rr = r0 + i;
             if (rr < w) {
                 // a panel row is final here: also its diagonal-scaled value for the backward sweep
@@ -1140,7 +1139,7 @@ __global__ void __launch_bounds__(256) k_bwd_narrow(const SolveDesc *sdescs, int
 template <class T, int PB>
 __global__ void __launch_bounds__(256) k_bwd_update(const SolveDesc *sdescs, const int32_t *items, const int64_t *zo,
                                                     const int32_t *sn_start, const SolveBufs<T> *jb, int p,
-                                                    LaunchTrace *tr) {
+                                                    LaunchTrace *tr, bool early) {
     TraceScope trace_scope(tr);
     const T *Gp = jb[blockIdx.z].G;
     T *Zs = jb[blockIdx.z].Zs, *x = jb[blockIdx.z].y;
@@ -1148,9 +1147,10 @@ __global__ void __launch_bounds__(256) k_bwd_update(const SolveDesc *sdescs, con
     extern __shared__ __align__(16) unsigned char smraw[];
     T *Gs = reinterpret_cast<T *>(smraw);    // RBB columns x bwd_ldg rows
     T *vs = Gs + RBB * bwd_ldg<T>();         // RBK x PB
-    T *red = PB == 8 ? Gs : vs + RBK * PB;  // 8 warps x 8 x RBB partial sums
+    T *red = PB == bwd_qc<T, PB>() ? Gs : vs + RBK * PB;  // the warps' partial sums
     const SolveDesc di = sdescs[items[2 * blockIdx.x]], dj = sdescs[items[2 * blockIdx.x + 1]];
     const int cc = blockIdx.y * RBB;
+    if (early) pdl_trigger();
     if (cc >= di.w) {
         pdl_wait();
         return;
@@ -1161,23 +1161,18 @@ __global__ void __launch_bounds__(256) k_bwd_update(const SolveDesc *sdescs, con
     const int64_t zi = zo[s] + di.k0 + cc, zj = zo[s] + dj.k0;
     const bool fin = dj.k0 == di.k0 + di.w;
     pdl_wait();
-    pdl_trigger();
-    {
-        static_assert(RBK == 256, "one row of v per thread");
-        const int r = threadIdx.x;
-        T *vr = vs + r * PB;
-#pragma unroll
-        for (int q = 0; q < PB; ++q) vr[q] = (r < wj && q < p) ? Zs[(zj + r) * p + q] : T(0);
-    }
-    // the accumulator entries this thread updates: outputs o = threadIdx.x + 256 h of each 8-wide
-    // chunk of right-hand sides (column c = o % RBB, q = q0 + o / RBB)
-    constexpr int NQ = PB / 8;
-    T old[NQ][2];
+    if (!early) pdl_trigger();
+    static_assert(RBK == 256, "stage_rows fills v");
+    stage_rows<T, PB>(vs, Zs + zj * p, wj, p);
+    // the accumulator entries this thread updates: outputs o = threadIdx.x + 256 h of each QC-wide
+    // chunk of right-hand sides (column c = o / QC, q = q0 + o % QC)
+    constexpr int QC = bwd_qc<T, PB>(), NQ = PB / QC, NH = RBB * QC / 256;
+    T old[NQ][NH];
 #pragma unroll
     for (int u = 0; u < NQ; ++u)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = 8 * u + o / RBB, c = o % RBB;
+        for (int h = 0; h < NH; ++h) {
+            const int o = threadIdx.x + 256 * h, c = o / QC, q = QC * u + o % QC;
             old[u][h] = (c < wc && q < p) ? Zs[(zi + c) * p + q] : T(0);
         }
     cp_async_commit_wait();
@@ -1185,11 +1180,11 @@ __global__ void __launch_bounds__(256) k_bwd_update(const SolveDesc *sdescs, con
     T *xp = x + ((int64_t)sn_start[s] + di.k0 + cc) * p;
 #pragma unroll
     for (int u = 0; u < NQ; ++u) {
-        T o2[2];
-        bwd_tile_product<T, PB>(Gs, vs, red, nrv * E, 8 * u, o2);
+        T o2[NH];
+        bwd_tile_product<T, PB>(Gs, vs, red, nrv * E, QC * u, o2);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = 8 * u + o / RBB, c = o % RBB;
+        for (int h = 0; h < NH; ++h) {
+            const int o = threadIdx.x + 256 * h, c = o / QC, q = QC * u + o % QC;
             if (c < wc && q < p) {
                 const T v = old[u][h] - o2[h];
                 Zs[(zi + c) * p + q] = v;
@@ -1208,29 +1203,43 @@ __global__ void k_trace_reset(LaunchTrace *tr, int n) {
 }
 
 // Forward gather of one level from the row lists: Z[dst] = y[own] (or 0) + the children's
-// contributions in tree order; one thread per (row, right-hand side).
-template <class T>
-__global__ void k_fwd_gather_rows(int64_t nrows, const int64_t *dst, const int64_t *own, const int64_t *cptr,
-                                  const int64_t *src, const SolveBufs<T> *jb, int p, LaunchTrace *tr) {
+// contributions in tree order; one thread per row and VE right-hand sides (16 bytes where p allows).
+// The lists and the first children are read before the wait.
+template <class T, int VE>
+__global__ void __launch_bounds__(256) k_fwd_gather_rows(int nrows, const int64_t *dst, const int64_t *own,
+                                                         const int64_t *cptr, const int64_t *src,
+                                                         const SolveBufs<T> *jb, int p, LaunchTrace *tr) {
     TraceScope trace_scope(tr);
     const T *y = jb[blockIdx.z].y;
     T *Z = jb[blockIdx.z].Z;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = t / p;
-    const int q = (int)(t - row * p);
-    int64_t o = -1, d = 0, c0 = 0, c1 = 0;
-    if (row < nrows) {
+    struct alignas(sizeof(T) * VE) Pack { T v[VE]; };
+    const unsigned int t = blockIdx.x * blockDim.x + threadIdx.x, pv = (unsigned int)p / VE, row = t / pv;
+    const int q = (int)(t - row * pv) * VE;
+    int64_t o = -1, d = 0, c0 = 0, c1 = 0, s0 = 0, s1 = 0;
+    if (row < (unsigned int)nrows) {
         o = own[row];
         d = dst[row];
         c0 = cptr[row];
         c1 = cptr[row + 1];
+        if (c0 < c1) s0 = src[c0];
+        if (c0 + 1 < c1) s1 = src[c0 + 1];
     }
     pdl_wait();
     pdl_trigger();
-    if (row >= nrows) return;
-    T v = o >= 0 ? y[o * p + q] : T(0);
-    for (int64_t c = c0; c < c1; ++c) v += Z[src[c] * p + q];
-    Z[d * p + q] = v;
+    if (row >= (unsigned int)nrows) return;
+    auto at = [&](const T *b, int64_t r) { return *reinterpret_cast<const Pack *>(b + r * p + q); };
+    Pack v{}, x0{}, x1{};
+    if (o >= 0) v = at(y, o);
+    if (c0 < c1) x0 = at(Z, s0);
+    if (c0 + 1 < c1) x1 = at(Z, s1);
+#pragma unroll
+    for (int e = 0; e < VE; ++e) v.v[e] = (v.v[e] + x0.v[e]) + x1.v[e];
+    for (int64_t c = c0 + 2; c < c1; ++c) {
+        const Pack xc = at(Z, src[c]);
+#pragma unroll
+        for (int e = 0; e < VE; ++e) v.v[e] += xc.v[e];
+    }
+    *reinterpret_cast<Pack *>(Z + d * p + q) = v;
 }
 
 // Start of the backward sweep of one level (grid: the level's row blocks x column chunks), tiles
@@ -1256,8 +1265,8 @@ __global__ void __launch_bounds__(256) k_bwd_step(const SolveDesc *sdescs, const
     extern __shared__ __align__(16) unsigned char smraw[];
     T *Gs = reinterpret_cast<T *>(smraw);    // RBB columns x bwd_ldg rows
     T *vs = Gs + RBB * bwd_ldg<T>();         // RBK x PB
-    T *red = PB == 8 ? Gs : vs + RBK * PB;  // 8 warps x 8 x RBB partial sums
-    __shared__ int s_last;
+    T *red = PB == bwd_qc<T, PB>() ? Gs : vs + RBK * PB;  // the warps' partial sums
+    __shared__ int s_last, vsrc[RBK];
     const int di = blk_desc[blockIdx.x];
     const SolveDesc d = sdescs[di];
     const int cc = blockIdx.y * RBB;
@@ -1272,24 +1281,54 @@ __global__ void __launch_bounds__(256) k_bwd_step(const SolveDesc *sdescs, const
     const int wc = min(RBB, w - cc);
     const int64_t zb = zo[s] + k0, ld = sg_ld(R);
     bwd_tile_issue(Gs, Gp + d.goff + (int64_t)cc * ld + r0, ld, wc, nrv);
-    // thread i loads row i of v: the panel's y, zero on later panels' rows, -x on the contribution block
+    // row i of v: the panel's y, zero on later panels' rows, -x on the contribution block.  Thread i puts its
+    // row's place in shared memory (row of yfw or x; odd: x, negated; -1: zero); the values are then read
+    // side by side
     static_assert(RBK == 256, "one row of v per thread");
-    const int i = threadIdx.x, rr = r0 + i;
-    const int kind = i >= nr ? 0 : (b == 0 ? 1 : (rr < cb0 ? 0 : 3));
-    const int64_t src = kind == 1 ? ((int64_t)sn_start[s] + k0 + rr) * p
-                      : kind == 3 ? (int64_t)rows[rows_off[s] + k0 + rr] * p : 0;
+    {
+        const int i = threadIdx.x, rr = r0 + i;
+        const int kind = i >= nr ? 0 : (b == 0 ? 1 : (rr < cb0 ? 0 : 3));
+        vsrc[i] = kind == 1 ? 2 * (sn_start[s] + k0 + rr) : (kind == 3 ? 2 * rows[rows_off[s] + k0 + rr] + 1 : -1);
+    }
+    __syncthreads();
     pdl_wait();
     pdl_trigger();
-    {
-        T *vr = vs + i * PB;
-        if (kind == 0) {
+    auto vrow = [&](int r, T &sg) -> const T * {
+        const int v = vsrc[r];
+        sg = v < 0 ? T(0) : ((v & 1) ? T(-1) : T(1));
+        return v < 0 ? nullptr : ((v & 1) ? x : yfw) + (int64_t)(v >> 1) * p;
+    };
+    if (p == PB) {  // 16-byte aligned rows
+        using V = typename Vec16<T>::type;
+        constexpr int NV = PB / E;
+        V v[NV];
+        T sg[NV];
 #pragma unroll
-            for (int q = 0; q < PB; ++q) vr[q] = T(0);
-        } else {
-            const T *sp = kind == 1 ? yfw + src : x + src;
-            const T sg = kind == 1 ? T(1) : T(-1);
+        for (int u = 0; u < NV; ++u) {
+            const int idx = threadIdx.x + 256 * u;
+            const T *sp = vrow(idx / NV, sg[u]);
+            v[u] = sp ? reinterpret_cast<const V *>(sp)[idx % NV] : V{};
+        }
 #pragma unroll
-            for (int q = 0; q < PB; ++q) vr[q] = q < p ? sg * sp[q] : T(0);
+        for (int u = 0; u < NV; ++u) {
+            T e4[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) e4[e] = sg[u] * Vec16<T>::get(v[u], e);
+            Vec16<T>::put(vs + (threadIdx.x + 256 * u) * E, e4);
+        }
+    } else {
+#pragma unroll
+        for (int u0 = 0; u0 < PB; u0 += 8) {
+            T v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int idx = threadIdx.x + 256 * (u0 + u), q = idx % PB;
+                T sg;
+                const T *sp = vrow(idx / PB, sg);
+                v[u] = sp && q < p ? sg * sp[q] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) vs[threadIdx.x + 256 * (u0 + u)] = v[u];
         }
     }
     cp_async_commit_wait();
@@ -1299,19 +1338,20 @@ __global__ void __launch_bounds__(256) k_bwd_step(const SolveDesc *sdescs, const
     T *zsp = Zs + (zb + cc) * p;
     T *xp = k0 + w >= ncs ? x + ((int64_t)sn_start[s] + k0 + cc) * p : nullptr;
 #pragma unroll
-    for (int q0 = 0; q0 < PB; q0 += 8) {
-        T o2[2];
+    for (int q0 = 0; q0 < PB; q0 += bwd_qc<T, PB>()) {
+        constexpr int QC = bwd_qc<T, PB>(), NH = RBB * QC / 256;
+        T o2[NH];
         bwd_tile_product<T, PB>(Gs, vs, red, nrv * E, q0, o2);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int o = threadIdx.x + 256 * h, q = q0 + o / RBB, c = o % RBB;
+        for (int h = 0; h < NH; ++h) {
+            const int o = threadIdx.x + 256 * h, c = o / QC, q = q0 + o % QC;
             if (nb == 1) {
                 if (c < wc && q < p) {
                     zsp[c * p + q] = o2[h];
                     if (xp) xp[c * p + q] = o2[h];
                 }
             } else {
-                out[q * RBB + c] = o2[h];
+                out[c * PB + q] = o2[h];
             }
         }
     }
@@ -1622,7 +1662,11 @@ static void solve_levels(const Plan &pl, const SolveBufs<T> *jb, unsigned K, int
     [[maybe_unused]] const size_t fsm = fwd_step_smem<T, PB>(), bsm = bwd_step_smem<T, PB>();
     [[maybe_unused]] int64_t fwd_cap = 0;
     if constexpr (sizeof(T) == 4) fwd_cap = resident_grid(k_fwd_step<T, PB>, fsm);
-    int it = 0;
+    // Of three panel launches in a row two let their successor in before their own wait, so that up to three
+    // launches' descriptors and tiles are under way (L = 18, 8 right-hand sides: 749 us a solve; all after the
+    // wait 801, every second 761, all before it 801: the deeper the queue, the slower each release).
+    int it = 0, par = 0;
+    auto early = [&] { return ++par % 3 != 0; };
     auto next_tr = [&](int kind) -> LaunchTrace * {
         if (!trb) return nullptr;
         if (kinds) kinds->push_back(kind);
@@ -1631,9 +1675,14 @@ static void solve_levels(const Plan &pl, const SolveBufs<T> *jb, unsigned K, int
     for (int l = 0; l < pl.nlevels; ++l) {
         {
             const int64_t f0 = pl.lvl_fg_ptr[l], nrows = pl.lvl_fg_ptr[l + 1] - f0;
-            launch_pdl(k_fwd_gather_rows<T>, dim3((unsigned)((nrows * p + 255) / 256), 1, K), dim3(256), 0, st, nrows,
-                       pl.d_fg_dst.data() + f0, pl.d_fg_own.data() + f0, pl.d_fg_cptr.data() + f0,
-                       (const int64_t *)pl.d_fg_src.data(), jb, p, next_tr(0));
+            auto gather = [&](auto kern, int ve) {
+                launch_pdl(kern, dim3((unsigned)((nrows * (p / ve) + 255) / 256), 1, K), dim3(256), 0, st, (int)nrows,
+                           pl.d_fg_dst.data() + f0, pl.d_fg_own.data() + f0, pl.d_fg_cptr.data() + f0,
+                           (const int64_t *)pl.d_fg_src.data(), jb, p, next_tr(0));
+            };
+            constexpr int VE = 16 / sizeof(T);
+            if (p % VE == 0) gather(k_fwd_gather_rows<T, VE>, VE);
+            else gather(k_fwd_gather_rows<T, 1>, 1);
         }
         for (int si = pl.lvl_sstep_ptr[l]; si < pl.lvl_sstep_ptr[l + 1]; ++si) {
             const SolveStep &ss = pl.ssteps[si];
@@ -1651,7 +1700,7 @@ static void solve_levels(const Plan &pl, const SolveBufs<T> *jb, unsigned K, int
             const int64_t items = ss.nrb * (int64_t)K;
             launch_pdl(k_fwd_step<T, PB>, dim3((unsigned)std::min<int64_t>(items, fwd_cap)), dim3(256), fsm, st, sd,
                        (const int32_t *)pl.d_fblk_desc.data() + ss.fblk0, (int)ss.nrb, (int)K, pl.d_sn_zo.data(),
-                       pl.d_sn_start.data(), jb, p, next_tr(1));
+                       pl.d_sn_start.data(), jb, p, next_tr(1), early());
             }
         }
     }
@@ -1683,7 +1732,7 @@ static void solve_levels(const Plan &pl, const SolveBufs<T> *jb, unsigned K, int
             const BwdUpd &bu = pl.bupd[u];
             launch_pdl(k_bwd_update<T, PB>, dim3((unsigned)bu.nit, SUBS, K), dim3(256), bsm, st,
                        (const SolveDesc *)pl.d_sdescs.data(), (const int32_t *)pl.d_bu_items.data() + 2 * bu.it0,
-                       pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, next_tr(3));
+                       pl.d_sn_zo.data(), pl.d_sn_start.data(), jb, p, next_tr(3), early());
         }
         }
     }

@@ -45,7 +45,9 @@ extern thread_local long long t_launches;  // this thread's share (graph capture
 // predecessor in the stream is still running.  It must execute pdl_wait() -- which returns once
 // the predecessor grid has completed and its writes are visible -- before it touches anything the
 // predecessor writes or reads, and on every path before it exits (so that completion stays
-// transitive along the stream).  pdl_trigger() lets the successor launch early.
+// transitive along the stream).  pdl_trigger() lets the successor launch once every CTA of this grid has
+// issued it or exited; it may come before the wait (what a successor does before its own wait reads only
+// the plan and the factor).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(256) k_df_bwd(DfArgs A, const T *Gp, const T *
     extern __shared__ __align__(16) unsigned char smraw[];
     T *Gs = reinterpret_cast<T *>(smraw);    // RBB columns x bwd_ldg rows
     T *vs = Gs + RBB * bwd_ldg<T>();         // RBK x PB
-    T *red = PB == 8 ? Gs : vs + RBK * PB;  // 8 warps x 8 x RBB partial sums
+    T *red = PB == bwd_qc<T, PB>() ? Gs : vs + RBK * PB;  // the warps' partial sums
     __shared__ int s_t, s_ok, s_last;
     const int tid = threadIdx.x;
     for (;;) {
@@ -260,19 +260,20 @@ __global__ void __launch_bounds__(256) k_df_bwd(DfArgs A, const T *Gp, const T *
         T *out = P + (A.poff[qd] + (int64_t)it.b * SUBS + ci) * tile;
         T *zsp = Zs + (zb + cc) * p, *xp = x + ((int64_t)A.sn_start[s] + k0 + cc) * p;
 #pragma unroll
-        for (int q0 = 0; q0 < PB; q0 += 8) {
-            T o2[2];
+        for (int q0 = 0; q0 < PB; q0 += bwd_qc<T, PB>()) {
+            constexpr int QC = bwd_qc<T, PB>(), NH = RBB * QC / 256;
+            T o2[NH];
             bwd_tile_product<T, PB>(Gs, vs, red, nrv * E, q0, o2);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int o = tid + 256 * h, q = q0 + o / RBB, c = o % RBB;
+            for (int h = 0; h < NH; ++h) {
+                const int o = tid + 256 * h, c = o / QC, q = q0 + o % QC;
                 if (nb == 1) {
                     if (c < wc && q < p) {
                         zsp[c * p + q] = o2[h];
                         xp[c * p + q] = o2[h];
                     }
                 } else {
-                    out[q * RBB + c] = o2[h];
+                    out[c * PB + q] = o2[h];
                 }
             }
         }
