@@ -697,6 +697,18 @@ __device__ bool gm_dots(int64_t e0, int64_t e1, int k1, int p, const double *V, 
     return true;
 }
 
+// nr[0, p) = squared norms -> norms, and their reciprocals (zero for zero) in nr[p, 2 p).  By p threads: a root
+// and a division are some thirty FP64 instructions, which hold the SM's FP64 pipe for every warp that runs them
+// (in all sixteen warps 4 us of a step).
+__device__ void gm_inverse_norms(int p, double *nr) {
+    if ((int)threadIdx.x < p) {
+        const double nn = sqrt(nr[threadIdx.x]);
+        nr[threadIdx.x] = nn;
+        nr[p + threadIdx.x] = nn > 0.0 ? 1.0 / nn : 0.0;
+    }
+    __syncthreads();
+}
+
 // Layout per column of Hall: Hc[(kmax+1) x kmax] column-major, cs/sn[kmax], g[kmax+1].
 __host__ __device__ inline size_t gm_hall(int kmax) { return (size_t)(kmax + 1) * kmax + 3 * (size_t)(kmax + 1); }
 
@@ -723,7 +735,8 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_step(int64_t n, int k, int p,
     if (!gm_dots(e0, e1, 1, p, W, 0, W, part + 2 * part_len, nr, red, bar, base + 3 * gridDim.x, err)) return;
     {
         double *Vn = V + (int64_t)k1 * vstride;
-        const double nn = sqrt(nr[q]), inv = nn > 0.0 ? 1.0 / nn : 0.0;
+        gm_inverse_norms(p, nr);
+        const double inv = nr[p + q];
         if (t < S)
             for (int64_t e = e0 + t; e < e1; e += S) Vn[e] = W[e] * inv;
     }
@@ -740,7 +753,7 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_step(int64_t n, int k, int p,
             col[i] = cs[i] * a + sn[i] * b;
             a = -sn[i] * a + cs[i] * b;
         }
-        const double b = sqrt(nr[t]);
+        const double b = nr[t];
         const double r = hypot(a, b);
         const double c = r > 0.0 ? a / r : 1.0, s_ = r > 0.0 ? b / r : 0.0;
         cs[k] = c;
@@ -762,14 +775,15 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_start(int64_t n, int p, int k
     double *red = sm_gm, *nr = red + GM_BATCH * GM_THREADS;
     const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per), e0 = r0 * p, e1 = r1 * p;
     if (!gm_dots(e0, e1, 1, p, Rr, 0, Rr, part, nr, red, bar, base + gridDim.x, err)) return;
-    const double nn = sqrt(nr[q]), inv = nn > 0.0 ? 1.0 / nn : 0.0;
+    gm_inverse_norms(p, nr);
+    const double inv = nr[p + q];
     if (t < S)
         for (int64_t e = e0 + t; e < e1; e += S) V[e] = Rr[e] * inv;
     if (blockIdx.x == 0 && t < p) {
         const int ld = kmax + 1;
         double *g = Hall + (size_t)t * gm_hall(kmax) + ld * kmax + 2 * ld;
         for (int i = 0; i < ld; ++i) g[i] = 0.0;
-        g[0] = nn;
+        g[0] = nr[t];
     }
 }
 
@@ -1047,7 +1061,7 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
     unsigned long long *err = Gbar.data();
     unsigned int *bar = reinterpret_cast<unsigned int *>(Gbar.data() + 1);
     const unsigned nbk = nblk(blk);
-    const size_t smem0 = (GM_BATCH * GM_THREADS + 32) * sizeof(double);
+    const size_t smem0 = (GM_BATCH * GM_THREADS + 64) * sizeof(double);
     smem_limit((const void *)k_gm_start, smem0);
     smem_limit((const void *)k_gm_step, smem0 + (size_t)2 * 64 * 32 * sizeof(double));
     double prev = INFINITY;
@@ -1174,28 +1188,34 @@ __global__ void k_normalize_first(int64_t n, double *V, int ldv, const double *p
 // ---- plain Lanczos steps of the extremal bounds ----
 constexpr int LZ_THREADS = 512, LZ_TPR = 4;  // threads a CTA, lanes a row
 
-// Sum over the CTA in a fixed order; every thread gets it.
-__device__ double lz_block_sum(double s, double *red) {
+// Sum of s over the grid: the CTAs' sums meet in part[] (one slot each) and every CTA adds them in the same
+// order, so that all use the same bits.  Past a warp's own sum, warp 0 works for the CTA (the others would
+// only hold the FP64 pipe); its lane 0 leaves the total in bc[0] and, where `root` is set, its square root and
+// the reciprocal of that (zero for zero) in bc[1], bc[2].  False if the wait for the other CTAs expired.
+__device__ bool lz_grid_sum(double s, bool root, double *part, unsigned int *bar, unsigned int target, double *red,
+                            unsigned long long *err, double *bc) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    double t = (threadIdx.x & 31) < LZ_THREADS / 32 ? red[threadIdx.x & 31] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    return t;
-}
-
-// Sum of s over the grid: the CTAs' sums meet in part[] (one slot each) and every CTA adds them in the same
-// order, so that all use the same bits.  False if the wait for the other CTAs expired.
-__device__ bool lz_grid_sum(double s, double *part, unsigned int *bar, unsigned int target, double *red,
-                            unsigned long long *err, double *total) {
-    const double b = lz_block_sum(s, red);
-    if (threadIdx.x == 0) part[blockIdx.x] = b;
+    if (threadIdx.x < 32) {
+        double t = threadIdx.x < LZ_THREADS / 32 ? red[threadIdx.x] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) part[blockIdx.x] = t;
+    }
     if (!grid_wait(bar, target, err)) return false;
-    double t = 0.0;
-    for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    *total = t;
+    if (threadIdx.x < 32) {
+        double t = 0.0;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) {
+            bc[0] = t;
+            if (root) {
+                bc[1] = sqrt(t);
+                bc[2] = bc[1] > 0.0 ? 1.0 / bc[1] : 0.0;
+            }
+        }
+    }
+    __syncthreads();
     return true;
 }
 
@@ -1210,42 +1230,53 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lz_steps(int64_t n, const int64_
                                                          const double *__restrict__ val, int j0, int steps, double *w,
                                                          double *vprev, double *u, double *alpha, double *beta,
                                                          double *part, unsigned int *bar, unsigned long long *err) {
-    __shared__ double red[LZ_THREADS / 32];
+    __shared__ double red[LZ_THREADS / 32], bc[3];
+    // thread t of the CTA: its group of LZ_TPR lanes sums rows r0 + k gs; lane `sub` keeps the row of k % LZ_TPR = sub
     const int sub = threadIdx.x % LZ_TPR;
-    const int64_t g0 = ((int64_t)blockIdx.x * LZ_THREADS + threadIdx.x) / LZ_TPR;
+    const int64_t r0 = ((int64_t)blockIdx.x * LZ_THREADS + threadIdx.x) / LZ_TPR;
+    const int64_t rw = ((int64_t)blockIdx.x * LZ_THREADS + (threadIdx.x & ~31)) / LZ_TPR;  // the warp's first row
     const int64_t gs = (int64_t)gridDim.x * LZ_THREADS / LZ_TPR;
-    double bprev = j0 > 0 ? beta[j0 - 1] : 0.0;
+    double bprev = j0 > 0 ? beta[j0 - 1] : 0.0, inv = j0 > 0 ? (bprev > 0.0 ? 1.0 / bprev : 0.0) : 1.0;
     unsigned int target = 0;
     for (int j = j0; j < j0 + steps; ++j) {
-        const double inv = j > 0 ? (bprev > 0.0 ? 1.0 / bprev : 0.0) : 1.0;
         double dot = 0.0;
-        for (int64_t ib = g0 - g0 % (32 / LZ_TPR); ib < n; ib += gs) {  // the warp's rows (uniform: shuffles below)
-            const int64_t i = ib + g0 % (32 / LZ_TPR);
-            double s = 0.0;
-            if (i < n)
-                for (int64_t e = rowptr[i] + sub; e < rowptr[i + 1]; e += LZ_TPR) s = fma(val[e], __ldcg(w + col[e]), s);
+        for (int64_t k = 0; rw + k * gs < n; k += LZ_TPR) {  // (uniform in the warp: shuffles below)
+            double s[LZ_TPR], own = 0.0;
 #pragma unroll
-            for (int o = 1; o < LZ_TPR; o *= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (i < n && sub == 0) {
-                const double x = s * inv - bprev * vprev[i];
+            for (int q = 0; q < LZ_TPR; ++q) {
+                const int64_t i = r0 + (k + q) * gs;
+                s[q] = 0.0;
+                if (i < n)
+                    for (int64_t e = rowptr[i] + sub; e < rowptr[i + 1]; e += LZ_TPR)
+                        s[q] = fma(val[e], __ldcg(w + col[e]), s[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < LZ_TPR; ++q) {
+#pragma unroll
+                for (int o = 1; o < LZ_TPR; o *= 2) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+                if (q == sub) own = s[q];
+            }
+            const int64_t i = r0 + (k + sub) * gs;
+            if (i < n) {
+                const double x = own * inv - bprev * vprev[i];
                 u[i] = x;
                 dot += w[i] * inv * x;
             }
         }
-        double a, b2;
         target += gridDim.x;
-        if (!lz_grid_sum(dot, part, bar, target, red, err, &a)) return;
+        if (!lz_grid_sum(dot, false, part, bar, target, red, err, bc)) return;
+        const double a = bc[0];
         double nr = 0.0;
-        for (int64_t i = g0; i < n; i += gs)
-            if (sub == 0) {
-                const double v = w[i] * inv, x = u[i] - a * v;
-                vprev[i] = v;
-                w[i] = x;
-                nr += x * x;
-            }
+        for (int64_t i = r0 + sub * gs; i < n; i += LZ_TPR * gs) {
+            const double v = w[i] * inv, x = u[i] - a * v;
+            vprev[i] = v;
+            w[i] = x;
+            nr += x * x;
+        }
         target += gridDim.x;
-        if (!lz_grid_sum(nr, part + gridDim.x, bar, target, red, err, &b2)) return;
-        bprev = sqrt(b2);
+        if (!lz_grid_sum(nr, true, part + gridDim.x, bar, target, red, err, bc)) return;
+        bprev = bc[1];
+        inv = bc[2];
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             alpha[j] = a;
             beta[j] = bprev;
