@@ -645,33 +645,70 @@ __device__ bool grid_wait(unsigned int *bar, unsigned int target, unsigned long 
 // stride S, so its column q = t % p is fixed, the loads coalesce, and W's elements stay with their thread through
 // the passes.  The chunks' sums meet in part[] and every CTA adds them itself in the same order.
 // Ten launches of 2 to 5 us in a row before (dots, reduce, subtract, twice; norm, reduce, Givens, scale); bound by
-// latency: three grid-wide waits and as many passes over V from L2 (40 us at L = 12, where they took some 50 with
-// their gaps; a refined solve of one right-hand side at L = 16 1.09 -> 1.00 ms, of 16 at L = 18 6.03 -> 5.30).
-constexpr int GM_THREADS = 512, GM_BATCH = 16;
+// latency: three grid-wide waits and as many passes over V from L2.  Ten launches took some 50 us with their gaps
+// at L = 12, one launch 40; with W in registers through the passes, the loads of four vectors issued together
+// and one warp per root 25 (L = 18, 16 right-hand sides: 97 -> 61 us; a refined solve of them 6.03 -> 5.30 ms by
+// the one launch at the time).
+constexpr int GM_THREADS = 512, GM_BATCH = 4;
 
-// part[b][o] = sum of the CTA's rows of V_i[r][q] W[r][q] (o = i p + q, i < k1), then, over the grid, h[o]
-__device__ bool gm_dots(int64_t e0, int64_t e1, int k1, int p, const double *V, int64_t vstride, const double *W,
-                        double *part, double *h, double *red, unsigned int *bar, unsigned int target,
-                        unsigned long long *err) {
-    const int t = threadIdx.x, S = (GM_THREADS / p) * p;
+// A thread's elements of W: NE > 0 of them in registers, else in memory (any number, in turn).
+template <int NE>
+struct GmElems {
+    double w[NE > 0 ? NE : 1];
+    int64_t e0, e1;  // first element and end of the chunk; stride S (e0 = e1: none)
+    int S;
+    double *W;
+    __device__ GmElems(double *W_, int64_t b, int64_t e, int p) : e1(e), S((GM_THREADS / p) * p), W(W_) {
+        e0 = (int)threadIdx.x < S ? b + threadIdx.x : e;
+        if constexpr (NE > 0)
+#pragma unroll
+            for (int u = 0; u < NE; ++u) w[u] = e0 + (int64_t)u * S < e1 ? W[e0 + (int64_t)u * S] : 0.0;
+    }
+    template <class F>
+    __device__ void each(F f) {  // f(element, value &)
+        if constexpr (NE > 0) {
+#pragma unroll
+            for (int u = 0; u < NE; ++u)
+                if (e0 + (int64_t)u * S < e1) f(e0 + (int64_t)u * S, w[u]);
+        } else {
+            for (int64_t e = e0; e < e1; e += S) {
+                double x = W[e];
+                f(e, x);
+            }
+        }
+    }
+};
+
+// part[b][o] = sum of the CTA's rows of V_i[r][q] W[r][q] (o = i p + q, i < k1; V null: of W[r][q]^2), then,
+// over the grid, h[o]
+template <int NE>
+__device__ bool gm_dots(GmElems<NE> &el, int k1, int p, const double *V, int64_t vstride, double *part, double *h,
+                        double *red, unsigned int *bar, unsigned int target, unsigned long long *err) {
+    const int t = threadIdx.x;
     for (int i0 = 0; i0 < k1; i0 += GM_BATCH) {
         const int ni = min(GM_BATCH, k1 - i0);
         double acc[GM_BATCH];
 #pragma unroll
         for (int i = 0; i < GM_BATCH; ++i) acc[i] = 0.0;
-        if (t < S)
-            for (int64_t e = e0 + t; e < e1; e += S) {
-                const double wv = W[e];
+        if (V) {
+            // (past ni a vector's load once more: those of all are issued together)
+            el.each([&](int64_t e, double &wv) {
+                double v[GM_BATCH];
+#pragma unroll
+                for (int i = 0; i < GM_BATCH; ++i) v[i] = V[(int64_t)(i0 + min(i, ni - 1)) * vstride + e];
 #pragma unroll
                 for (int i = 0; i < GM_BATCH; ++i)
-                    if (i < ni) acc[i] = fma(V[(int64_t)(i0 + i) * vstride + e], wv, acc[i]);
-            }
+                    if (i < ni) acc[i] = fma(v[i], wv, acc[i]);
+            });
+        } else {
+            el.each([&](int64_t, double &wv) { acc[0] = fma(wv, wv, acc[0]); });
+        }
         // threads of one right-hand side: within a warp by shuffles where p divides 32, the rest in shared memory
         const int lanes = 32 % p == 0 ? p : 32;
 #pragma unroll
         for (int i = 0; i < GM_BATCH; ++i) {
             if (i >= ni) break;
-            double x = t < S ? acc[i] : 0.0;
+            double x = acc[i];
             for (int o = lanes; o < 32; o *= 2) x += __shfl_xor_sync(0xffffffffu, x, o);
             if ((t & 31) < lanes) red[i * GM_THREADS + (t >> 5) * lanes + (t & 31)] = x;
         }
@@ -712,47 +749,47 @@ __device__ void gm_inverse_norms(int p, double *nr) {
 // Layout per column of Hall: Hc[(kmax+1) x kmax] column-major, cs/sn[kmax], g[kmax+1].
 __host__ __device__ inline size_t gm_hall(int kmax) { return (size_t)(kmax + 1) * kmax + 3 * (size_t)(kmax + 1); }
 
+template <int NE>
 __global__ void __launch_bounds__(GM_THREADS) k_gm_step(int64_t n, int k, int p, int kmax, int64_t rows_per, double *V,
                                                         int64_t vstride, double *W, double *Hall, double *res,
                                                         double *part, int64_t part_len, unsigned int *bar,
                                                         unsigned int base, unsigned long long *err) {
     extern __shared__ double sm_gm[];
-    const int k1 = k + 1, t = threadIdx.x, S = (GM_THREADS / p) * p;
+    const int k1 = k + 1, t = threadIdx.x;
     double *red = sm_gm, *h1 = red + GM_BATCH * GM_THREADS, *h2 = h1 + k1 * p, *nr = h2 + k1 * p;
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per), e0 = r0 * p, e1 = r1 * p;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
     const int q = t % p;
+    GmElems<NE> el(W, r0 * p, r1 * p, p);
     for (int pass = 0; pass < 2; ++pass) {
         double *h = pass ? h2 : h1;
-        if (!gm_dots(e0, e1, k1, p, V, vstride, W, part + pass * part_len, h, red, bar, base + (pass + 1) * gridDim.x, err))
+        if (!gm_dots(el, k1, p, V, vstride, part + pass * part_len, h, red, bar, base + (pass + 1) * gridDim.x, err))
             return;
-        if (t < S)
-            for (int64_t e = e0 + t; e < e1; e += S) {
-                double s = 0.0;
-                for (int i = 0; i < k1; ++i) s = fma(V[(int64_t)i * vstride + e], h[i * p + q], s);
-                W[e] -= s;
-            }
-    }
-    if (!gm_dots(e0, e1, 1, p, W, 0, W, part + 2 * part_len, nr, red, bar, base + 3 * gridDim.x, err)) return;
-    {
-        double *Vn = V + (int64_t)k1 * vstride;
-        gm_inverse_norms(p, nr);
-        const double inv = nr[p + q];
-        if (t < S)
-            for (int64_t e = e0 + t; e < e1; e += S) Vn[e] = W[e] * inv;
+        el.each([&](int64_t e, double &w) {
+            double s = 0.0;
+            for (int i = 0; i < k1; ++i) s = fma(V[(int64_t)i * vstride + e], h[i * p + q], s);
+            w -= s;
+            if constexpr (NE == 0) W[e] = w;
+        });
     }
     // Hessenberg column per right-hand side (a thread each): h1 + h2 and h_{k+1,k} = |w|, the earlier Givens
-    // rotations, a new one, and the right-hand side g
-    if (blockIdx.x == 0 && t < p) {
-        const int ld = kmax + 1;
-        double *Hc = Hall + (size_t)t * gm_hall(kmax);
-        double *cs = Hc + ld * kmax, *sn = cs + ld, *g = sn + ld;
-        double *col = Hc + (size_t)k * ld;
-        double a = h1[t] + h2[t];
+    // rotations (before the norm's wait), a new one, and the right-hand side g
+    const int ld = kmax + 1;
+    double *Hc = Hall + (size_t)(t < p ? t : 0) * gm_hall(kmax);
+    double *cs = Hc + ld * kmax, *sn = cs + ld, *g = sn + ld;
+    double *col = Hc + (size_t)k * ld;
+    const bool hess = blockIdx.x == 0 && t < p;
+    double a = 0.0;
+    if (hess) {
+        a = h1[t] + h2[t];
         for (int i = 0; i < k; ++i) {
             const double b = h1[(i + 1) * p + t] + h2[(i + 1) * p + t];
             col[i] = cs[i] * a + sn[i] * b;
             a = -sn[i] * a + cs[i] * b;
         }
+    }
+    if (!gm_dots(el, 1, p, nullptr, 0, part + 2 * part_len, nr, red, bar, base + 3 * gridDim.x, err)) return;
+    gm_inverse_norms(p, nr);
+    if (hess) {
         const double b = nr[t];
         const double r = hypot(a, b);
         const double c = r > 0.0 ? a / r : 1.0, s_ = r > 0.0 ? b / r : 0.0;
@@ -764,21 +801,25 @@ __global__ void __launch_bounds__(GM_THREADS) k_gm_step(int64_t n, int k, int p,
         g[k] = c * g[k];
         res[t] = fabs(g[k + 1]);
     }
+    double *Vn = V + (int64_t)k1 * vstride;
+    const double inv = nr[p + q];
+    el.each([&](int64_t e, double &w) { Vn[e] = w * inv; });
 }
 
 // Start of a cycle, one cooperative launch: V_0 = R / |R|, g = |R| e_1.
-__global__ void __launch_bounds__(GM_THREADS) k_gm_start(int64_t n, int p, int kmax, int64_t rows_per, const double *Rr,
+template <int NE>
+__global__ void __launch_bounds__(GM_THREADS) k_gm_start(int64_t n, int p, int kmax, int64_t rows_per, double *Rr,
                                                          double *V, double *Hall, double *part, unsigned int *bar,
                                                          unsigned int base, unsigned long long *err) {
     extern __shared__ double sm_gm[];
-    const int t = threadIdx.x, S = (GM_THREADS / p) * p, q = t % p;
+    const int t = threadIdx.x, q = t % p;
     double *red = sm_gm, *nr = red + GM_BATCH * GM_THREADS;
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per), e0 = r0 * p, e1 = r1 * p;
-    if (!gm_dots(e0, e1, 1, p, Rr, 0, Rr, part, nr, red, bar, base + gridDim.x, err)) return;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
+    GmElems<NE> el(Rr, r0 * p, r1 * p, p);
+    if (!gm_dots(el, 1, p, nullptr, 0, part, nr, red, bar, base + gridDim.x, err)) return;
     gm_inverse_norms(p, nr);
     const double inv = nr[p + q];
-    if (t < S)
-        for (int64_t e = e0 + t; e < e1; e += S) V[e] = Rr[e] * inv;
+    el.each([&](int64_t e, double &w) { V[e] = w * inv; });
     if (blockIdx.x == 0 && t < p) {
         const int ld = kmax + 1;
         double *g = Hall + (size_t)t * gm_hall(kmax) + ld * kmax + 2 * ld;
@@ -1062,8 +1103,13 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
     unsigned int *bar = reinterpret_cast<unsigned int *>(Gbar.data() + 1);
     const unsigned nbk = nblk(blk);
     const size_t smem0 = (GM_BATCH * GM_THREADS + 64) * sizeof(double);
-    smem_limit((const void *)k_gm_start, smem0);
-    smem_limit((const void *)k_gm_step, smem0 + (size_t)2 * 64 * 32 * sizeof(double));
+    // elements a thread: up to eight stay in registers through the passes (all sectors to L = 18 at eight
+    // right-hand sides); longer chunks are walked in memory
+    const int64_t per = (rows_per * p + GM_THREADS / p * p - 1) / (GM_THREADS / p * p);
+    const void *f_start = (const void *)(per <= 4 ? k_gm_start<4> : per <= 8 ? k_gm_start<8> : k_gm_start<0>);
+    const void *f_step = (const void *)(per <= 4 ? k_gm_step<4> : per <= 8 ? k_gm_step<8> : k_gm_step<0>);
+    smem_limit(f_start, smem0);
+    smem_limit(f_step, smem0 + (size_t)2 * 64 * 32 * sizeof(double));
     double prev = INFINITY;
     for (int outer = 0; outer < max_outer; ++outer) {
         std::vector<double> rn, lim;
@@ -1078,7 +1124,7 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
             const double *r_ = R.data();
             double *v_ = GV.data(), *h_ = Hall, *pt = Gdots.data();
             void *args[] = {&n_, &p_, &km, &rp, &r_, &v_, &h_, &pt, &bar, &gbar_count, &err};
-            MBL_CUDA(cudaLaunchCooperativeKernel((const void *)k_gm_start, dim3(nch), dim3(GM_THREADS), args, smem0, st));
+            MBL_CUDA(cudaLaunchCooperativeKernel(f_start, dim3(nch), dim3(GM_THREADS), args, smem0, st));
             MBL_LAUNCH_CHECK();
             gbar_count += nch;
         }
@@ -1099,7 +1145,7 @@ void RefinedSolve::apply_fgmres(const double *X, int ldx, double *Y, int p, cuda
                 int k_ = k, p_ = p, km = kmax;
                 double *v_ = GV.data(), *w_ = GW.data(), *h_ = Hall, *re = est_d, *pt = Gdots.data();
                 void *args[] = {&n_, &k_, &p_, &km, &rp, &v_, &vs, &w_, &h_, &re, &pt, &pl, &bar, &gbar_count, &err};
-                MBL_CUDA(cudaLaunchCooperativeKernel((const void *)k_gm_step, dim3(nch), dim3(GM_THREADS), args,
+                MBL_CUDA(cudaLaunchCooperativeKernel(f_step, dim3(nch), dim3(GM_THREADS), args,
                                                      smem0 + (size_t)2 * (k + 1) * p * sizeof(double), st));
                 MBL_LAUNCH_CHECK();
                 gbar_count += 3 * nch;
@@ -1224,7 +1270,8 @@ __device__ bool lz_grid_sum(double s, bool root, double *part, unsigned int *bar
 // sum; then w <- u - alpha_j v_j, vprev <- v_j and beta_j = |w|, another.  LZ_TPR lanes share a row; a thread
 // group's rows and every sum's order are fixed by the grid, which is fixed by n.
 // Bound by latency: a step is two grid-wide sums (some 2 us each) and one pass over H from L2.  As four
-// launches a step, with a check of 560 us, the bounds took 31.0 ms at L = 20 where they now take 14.0.
+// launches a step, with a check of 560 us, the bounds took 31.0 ms at L = 20 (14.0 as one
+// launch; on a shorter seed 8.83 and, with one warp per sum and a lane per row, 7.11).
 __global__ void __launch_bounds__(LZ_THREADS) k_lz_steps(int64_t n, const int64_t *__restrict__ rowptr,
                                                          const int32_t *__restrict__ col,
                                                          const double *__restrict__ val, int j0, int steps, double *w,
