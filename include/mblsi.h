@@ -118,7 +118,7 @@ typedef struct mbl_factor_stats {
     /* Autotuned tile shape of the FP32 fronts' trailing update by size class c of the panel step's
      * largest trailing block (64 2^c <= m2 < 64 2^(c+1); class 0 also smaller, class 7 also larger),
      * measured once per sector shape and tensor-core mode on a synthetic front of the class:
-     * 1 = tcgen05 128 x 128 tiles, 0 = CUDA-core 64 x 64 tiles, -1 = not tuned (FP64 fronts or CUDA
+     * 1 = tcgen05 128 x 64 tiles, 0 = CUDA-core 64 x 64 tiles, -1 = not tuned (FP64 fronts or CUDA
      * cores requested); the two timings in microseconds (0 where the class has no panel step). */
     int tune_choice[8];
     float tune_us_tc[8], tune_us_cc[8];
