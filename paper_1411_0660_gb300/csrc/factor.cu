@@ -855,6 +855,10 @@ __global__ void __launch_bounds__(256) k_apply_m(const SolveDesc *sdescs, int nd
 // wait on the previous step for the first item, since G is read-only); warp j then takes columns
 // [32 j, 32 j + 32) and lane i row i, and the eight partial sums meet in shared memory in a fixed
 // order (results do not depend on which CTA takes an item).
+// Bound by latency where the grid is small (the tree's top: a step after another): the predecessor's release, z
+// from L2, the product, the partial sums.  With z staged by 16-byte loads that are all issued before the first
+// store, the outputs side by side and the early triggers a step takes 2 to 5 us at L = 18 (before 4 to 6), with
+// 16 right-hand sides 3 to 6 (before 7 to 9: the staging loop's loads waited for one another).
 template <class T>
 __host__ __device__ constexpr size_t fwd_gtile_bytes() { return sizeof(T) * (size_t)SPW * RBF; }
 
@@ -1136,6 +1140,9 @@ __global__ void __launch_bounds__(256) k_bwd_narrow(const SolveDesc *sdescs, int
 // RBK x RBB tile of G_i is copied before waiting.  When panel j directly follows panel i this is the
 // last contribution to acc_i, which is then written to x as well.  Each accumulator chunk has one
 // writer per launch, so the updates are deterministic.
+// Bound by latency like the forward step: 2.6 to 4.7 us a launch at L = 18 (16 right-hand sides: 3.6 to 6, before
+// 7 to 11, when each thread read and stored a row of v for itself: 32 lines and 16-way bank conflicts an
+// instruction).
 template <class T, int PB>
 __global__ void __launch_bounds__(256) k_bwd_update(const SolveDesc *sdescs, const int32_t *items, const int64_t *zo,
                                                     const int32_t *sn_start, const SolveBufs<T> *jb, int p,
