@@ -194,7 +194,7 @@ struct Ctx {
 void server_shutdown(Ctx *ctx);
 
 // Small device results to the host through the context's pinned buffer (a copy into pageable memory goes by
-// the driver's own staging, several microseconds more): add() queues a copy on `st`, done() waits for the
+// CUDA's own staging, several microseconds more): add() queues a copy on `st`, done() waits for the
 // stream and hands the values out.  At most PIN_BYTES between two done().
 constexpr size_t PIN_BYTES = 64 << 10;
 struct ReadBack {
